@@ -1,0 +1,483 @@
+"""The work a user of this package has it do, as cases that can be timed and checked.
+
+Every case goes through `paper_2112_05051_gb300.richards` as a program calls it: the
+residual and the Jacobian (what an outer Newton driver calls), the AMG setup, refresh
+and V-cycle, the Krylov solve of a Newton correction, and whole backward-Euler steps,
+alone and in a batch.  Sizes, soils, boundary conditions and solver options are those
+of the package's workloads (`synth.WORKLOADS`), its request stream (n^3 columns with
+n in 24..96, log-normal K_s) and its tests, with ragged and odd grids among them.
+
+`exact` restates the discretisation (Sec. 2.1 of arXiv 2112.05051) in plain torch FP64
+and solves its linear and nonlinear systems by BiCGStab and Newton far below the
+solver's own tolerances.
+"""
+import math
+
+import numpy as np
+import torch
+
+from paper_2112_05051_gb300 import richards as rb
+from paper_2112_05051_gb300 import synth
+
+SOIL = synth.Soil()
+MEANS = {"arithmetic": synth.KMEAN_ARITH, "upstream": synth.KMEAN_UPSTREAM, "harmonic": synth.KMEAN_HARMONIC,
+         "geometric": synth.KMEAN_GEOMETRIC}
+DRY, WET_TOP = synth.P_INITIAL, synth.P_TOP
+
+
+def _case(op, nx, ny, nz, mean, **kw):
+    c = {"op": op, "nx": nx, "ny": ny, "nz": nz, "mean": mean, "sigma": 0.0, "bc": "column", "dt": 1.0,
+         "mixed": False, "krylov": "fgmres", "restart": 30, "nu": 2, "coarse": 2000, "batch": 1}
+    c.update(kw)
+    return c
+
+
+def listed():
+    return [
+        # the smallest call: one residual with its norms on the 16^3 grid of the FP64 test workload,
+        # as an outer nonlinear driver evaluates it (launches and the read-back count)
+        dict(_case("residual", 16, 16, 16, "arithmetic"), name="residual_16"),
+        # the residual of the 128^3 upstream workload, once per Newton and line-search trial
+        dict(_case("residual", 128, 128, 128, "upstream"), name="residual_128_upstream"),
+        # the residual for callers that may not allocate, on a ragged heterogeneous grid
+        dict(_case("noalloc", 97, 65, 49, "harmonic", sigma=1.0), name="noalloc_97x65x49"),
+        # J and A_aux of the paper's infiltration box (Dirichlet on every face, a pressure field on
+        # the top one) at half its horizontal resolution, odd sizes, handed to the caller
+        dict(_case("jacobian", 399, 401, 19, "upstream", bc="paper", dt=0.2), name="jacobian_399x401x19"),
+        # the preconditioner alone: V(2,2) in FP64 on the 128^3 workload
+        dict(_case("vcycle", 128, 128, 128, "upstream"), name="vcycle_128"),
+        # one Newton correction of the 128^3 workload: FGMRES(30) with V(2,2), all FP64
+        dict(_case("solve", 128, 128, 128, "upstream"), name="fgmres30_128"),
+        # one Newton correction of the paper's infiltration box: FGMRES(10), V(1,1), FP32 hierarchy
+        dict(_case("solve", 399, 401, 19, "upstream", bc="paper", dt=0.2, mixed=True, restart=10, nu=1),
+             name="fgmres10_paper_mixed"),
+        # one Newton correction of a served request: FCG, V(1,1), FP32 hierarchy, heterogeneous soil
+        dict(_case("solve", 48, 48, 48, "arithmetic", sigma=0.5, mixed=True, krylov="fcg", nu=1, coarse=500),
+             name="fcg_48_mixed"),
+        # the hierarchy of a fresh problem of a request's size, built and applied once
+        dict(_case("setup", 64, 64, 64, "arithmetic", sigma=1.0, nu=1, coarse=500), name="setup_64"),
+        # what a Newton iteration prepares: Jacobian, refresh of the hierarchy, first application
+        dict(_case("refresh", 128, 128, 128, "upstream"), name="refresh_128"),
+        # a whole backward-Euler step of the 128^3 workload
+        dict(_case("step", 128, 128, 128, "upstream", dt=4.0), name="step_128"),
+        # a batch of small same-shape requests stepped together
+        dict(_case("batch", 32, 32, 32, "upstream", sigma=0.25, mixed=True, krylov="fcg", nu=1, coarse=500, dt=0.25,
+                   batch=8), name="batch_8x32"),
+    ]
+
+
+def _size(rng, lo, hi):
+    """A size spread over its logarithm; odd ones as often as even ones."""
+    return max(lo, min(hi, int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))))
+
+
+def draw(rng):
+    op = rng.choice(["residual", "noalloc", "jacobian", "vcycle", "solve_fgmres", "solve_paper", "solve_fcg", "setup",
+                     "refresh", "step", "batch"])
+    any_mean = rng.choice(list(MEANS))
+    smooth_mean = rng.choice(["arithmetic", "upstream"])
+    if op == "residual":
+        return _case(op, _size(rng, 12, 160), _size(rng, 12, 160), _size(rng, 8, 128), any_mean,
+                     sigma=rng.choice([0.0, 1.0]))
+    if op == "noalloc":
+        return _case(op, _size(rng, 12, 128), _size(rng, 12, 128), _size(rng, 8, 96), any_mean,
+                     sigma=rng.choice([0.0, 1.0]))
+    if op == "jacobian":
+        if rng.random() < 0.5:
+            return _case(op, _size(rng, 40, 400), _size(rng, 40, 400), _size(rng, 4, 19), any_mean, bc="paper", dt=0.2)
+        return _case(op, _size(rng, 12, 144), _size(rng, 12, 144), _size(rng, 8, 128), any_mean,
+                     sigma=rng.choice([0.0, 1.0]))
+    if op in ("vcycle", "refresh"):
+        n = _size(rng, 24, 128)
+        return _case(op, n, max(20, n - rng.randrange(8)), max(20, n - rng.randrange(12)), smooth_mean,
+                     nu=rng.choice([1, 2]))
+    if op == "solve_fgmres":
+        n = _size(rng, 24, 120)
+        return _case("solve", n, max(20, n - rng.randrange(8)), max(20, n - rng.randrange(12)), smooth_mean,
+                     mixed=rng.random() < 0.5, nu=rng.choice([1, 2]))
+    if op == "solve_paper":
+        n = _size(rng, 60, 360)
+        return _case("solve", n, max(56, n - rng.randrange(9)), max(4, round(38 * n / 798)), "upstream", bc="paper",
+                     dt=0.2, mixed=rng.random() < 0.7, restart=10, nu=1)
+    if op == "solve_fcg":
+        n = _size(rng, 16, 96)
+        return _case("solve", n, max(14, n - rng.randrange(6)), max(14, n - rng.randrange(6)), "arithmetic",
+                     sigma=rng.choice([0.0, 0.25, 0.5]), mixed=rng.random() < 0.7, krylov="fcg", nu=1, coarse=500)
+    if op == "setup":
+        n = _size(rng, 24, 96)
+        return _case(op, n, max(20, n - rng.randrange(6)), max(20, n - rng.randrange(6)), smooth_mean,
+                     sigma=rng.choice([0.0, 0.5, 1.0]), nu=1, coarse=500)
+    if op == "step":
+        n = _size(rng, 16, 104)
+        fcg = n < 48
+        return _case(op, n, max(14, n - rng.randrange(6)), max(14, n - rng.randrange(6)),
+                     "arithmetic" if fcg else "upstream", dt=rng.choice([1.0, 4.0]), mixed=rng.random() < 0.5,
+                     krylov="fcg" if fcg else "fgmres", nu=1 if fcg else 2, coarse=500 if fcg else 2000)
+    return _case(op, _size(rng, 20, 36), _size(rng, 20, 36), _size(rng, 20, 36), "upstream", sigma=0.25, mixed=True,
+                 krylov="fcg", nu=1, coarse=500, dt=0.25, batch=rng.choice([2, 3, 5, 8]))
+
+
+# ---------------------------------------------------------------- inputs
+
+
+def _grid(c):
+    if c["bc"] == "paper":
+        return synth.Grid(c["nx"], c["ny"], c["nz"], 64.0, 64.0, 1.0)
+    return synth.Grid(c["nx"], c["ny"], c["nz"])
+
+
+def _bc(c, grid):
+    return synth.paper_infiltration_bc(grid, DRY) if c["bc"] == "paper" else synth.infiltration_bc(WET_TOP)
+
+
+def _pressure(c, grid, seed, hours=0):
+    """Pressure head of an infiltration under way, (nz, ny, nx): a wetting front under the wet part
+    of the top face whose depth and lateral shape come from the seed, plus a little noise."""
+    rng = np.random.Generator(np.random.PCG64([int(seed), 11]))
+    depth, ph1, ph2 = rng.uniform(0.12, 0.25), rng.uniform(0, 6.28), rng.uniform(0, 6.28)
+    depth *= 1.0 + 0.02 * hours
+    ax = lambda n: (torch.arange(n, dtype=torch.float64, device="cuda") + 1.0) / (n + 1)  # noqa: E731
+    x, y, z = ax(grid.nx)[None, None, :], ax(grid.ny)[None, :, None], ax(grid.nz)[:, None, None]
+    front = torch.exp(-(1.0 - z) / depth)
+    if c["bc"] == "paper":
+        edge = lambda t: torch.sigmoid((t - 0.25) / 0.02) * torch.sigmoid((0.75 - t) / 0.02)  # noqa: E731
+        p = DRY + 50.0 * edge(x) * edge(y) * front
+    else:
+        lateral = 1.0 - 0.1 * (1.0 + torch.sin(6.28 * x + ph1) * torch.sin(6.28 * y + ph2))
+        p = DRY + (WET_TOP - DRY) * lateral * front
+    gen = torch.Generator(device="cuda").manual_seed(int(seed) + 5)
+    return (p + 0.02 * torch.randn(p.shape, generator=gen, dtype=torch.float64, device="cuda")).contiguous()
+
+
+def _conductivity(c, grid, seed):
+    """Log-normal K_s on the host (as a program reads its soil), or None for the homogeneous soil."""
+    if not c["sigma"]:
+        return None
+    per = [synth.ks_field(grid, 1000 + 64 * int(seed) + b, c["sigma"]) for b in range(c["batch"])]
+    return per[0] if c["batch"] == 1 else np.concatenate(per)
+
+
+def _device_ks(ks):
+    return None if ks is None else torch.as_tensor(ks, dtype=torch.float64).cuda()
+
+
+def _amg_opts(c):
+    return rb.default_amg_opts(seed=2, coarse_max=c["coarse"], nu1=c["nu"], nu2=c["nu"], smooth_levels=2)
+
+
+def _newton_opts(c):
+    return rb.default_newton_opts(kind=rb.KRYLOV_FCG if c["krylov"] == "fcg" else rb.KRYLOV_FGMRES,
+                                  restart=c["restart"], seed=2, coarse_max=c["coarse"], nu1=c["nu"], nu2=c["nu"],
+                                  smooth_levels=2)
+
+
+def prepare(case, seed):
+    c, grid = case, _grid(case)
+    bc, mean = _bc(c, grid), MEANS[c["mean"]]
+    ks = _conductivity(c, grid, seed)
+    prec = rb.PREC_MIXED if c["mixed"] else rb.PREC_FP64
+    s = {"c": c}
+    if c["op"] == "batch":
+        one = [torch.full((grid.n,), DRY, dtype=torch.float64, device="cuda") for _ in range(c["batch"])]
+        s["p0"] = torch.cat(one)
+        s["ctx"] = rb.BatchContext(grid, c["batch"], SOIL, bc, mean, ks, precision=prec)
+        s["p"], s["opts"] = torch.empty_like(s["p0"]), _newton_opts(c)
+        return s
+    p = _pressure(c, grid, seed)
+    s["p"] = p.reshape(-1)
+    if c["op"] == "noalloc":
+        s.update(grid=grid, bc=bc, mean=mean, ks=_device_ks(ks))
+    else:
+        s["ctx"] = rb.Context(grid, SOIL, bc, mean, ks, precision=prec)
+    ctx = s.get("ctx")
+    if c["op"] in ("residual", "noalloc", "solve"):
+        s["s_old"] = _constitutive(_pressure(c, grid, seed, hours=-1).reshape(-1), SOIL.ks)[0].contiguous()
+        s["F"] = torch.empty_like(s["p"])
+    if c["op"] == "jacobian":
+        s["J7"] = torch.empty(7 * grid.n, dtype=torch.float64, device="cuda")
+        s["A7"] = torch.empty(7 * grid.n, dtype=torch.float64, device="cuda")
+    if c["op"] in ("vcycle", "solve", "setup"):
+        ctx.jacobian(s["p"], c["dt"])
+    if c["op"] in ("vcycle", "solve"):
+        ctx.amg_setup(_amg_opts(c))
+    if c["op"] in ("vcycle", "setup", "refresh"):
+        gen = torch.Generator(device="cuda").manual_seed(int(seed) + 9)
+        s["r"] = torch.randn(grid.n, generator=gen, dtype=torch.float64, device="cuda")
+        s["z"] = torch.empty_like(s["r"])
+    if c["op"] == "refresh":
+        ctx.jacobian(s["p"], c["dt"])
+        ctx.amg_setup(_amg_opts(c))
+        s["p2"] = _pressure(c, grid, seed, hours=3).reshape(-1)
+    if c["op"] == "setup":
+        s["opts"] = _amg_opts(c)
+    if c["op"] == "solve":
+        s["b"] = (-_residual(c, grid, bc, _device_ks(ks), p, s["s_old"].reshape(p.shape))).reshape(-1).contiguous()
+        s["x"] = torch.empty_like(s["b"])
+    if c["op"] == "step":
+        s["p0"], s["p"], s["opts"] = s["p"], torch.empty_like(s["p"]), _newton_opts(c)
+    return s
+
+
+def run(s):
+    c, ctx = s["c"], s.get("ctx")
+    if c["op"] == "residual":
+        return [s["F"], list(ctx.residual(s["p"], s["s_old"], c["dt"], s["F"]))]
+    if c["op"] == "noalloc":
+        status, norms = rb.residual_noalloc(s["grid"], SOIL, s["bc"], s["mean"], s["p"], s["s_old"], c["dt"], s["F"],
+                                            ks=s["ks"])
+        rb.check(status, "rich_residual_noalloc")
+        return [s["F"], list(norms)]
+    if c["op"] == "jacobian":
+        ctx.jacobian(s["p"], c["dt"], s["J7"], s["A7"])
+        return [s["J7"], s["A7"]]
+    if c["op"] == "vcycle":
+        ctx.vcycle(s["r"], s["z"])
+        return s["z"]
+    if c["op"] == "solve":
+        ctx.krylov_solve(s["b"], s["x"], kind=rb.KRYLOV_FCG if c["krylov"] == "fcg" else rb.KRYLOV_FGMRES,
+                         restart=c["restart"])
+        return s["x"]
+    if c["op"] == "setup":
+        ctx.amg_setup(s["opts"])
+        ctx.vcycle(s["r"], s["z"])
+        return s["z"]
+    if c["op"] == "refresh":
+        ctx.jacobian(s["p2"], c["dt"])
+        ctx.amg_update(rb.AMG_REFRESH)
+        ctx.vcycle(s["r"], s["z"])
+        return s["z"]
+    s["p"].copy_(s["p0"])
+    if c["op"] == "step":
+        ctx.step(s["p"], c["dt"], s["opts"])
+    else:
+        ctx.step_batch(s["p"], c["dt"], s["opts"])
+    return s["p"]
+
+
+def work(case):
+    """Inputs read once and outputs written once; arithmetic of the formulas once per cell.  For the
+    solves, one pass over the Jacobian and over the preconditioner's matrices per nominal iteration
+    (convergence to 1e-7 takes about a dozen with these hierarchies; three corrections per step)."""
+    c = case
+    n = float(c["nx"] * c["ny"] * c["nz"] * c["batch"])
+    field = 8.0 * n if c["sigma"] else 0.0
+    half = 4.0 if c["mixed"] else 8.0
+    law, faces = 60.0, 60.0                      # flops of the constitutive law; of the six faces
+    cycle = n * (half * 5 * (2 * c["nu"] + 1) * 1.5 + 16.0)
+    cycle_flops = n * 2.0 * 7 * (2 * c["nu"] + 1) * 1.5
+    if c["op"] in ("residual", "noalloc"):
+        return {"bytes": 24.0 * n + field, "flops": n * (law + faces)}
+    if c["op"] == "jacobian":
+        return {"bytes": 8.0 * n * 15 + field, "flops": n * (law + 2 * faces)}
+    if c["op"] == "vcycle":
+        return {"bytes": cycle, "flops": cycle_flops}
+    if c["op"] in ("setup", "refresh"):
+        jac = c["op"] == "refresh"
+        return {"bytes": cycle + (8.0 * n * 15 if jac else 56.0 * n) + n * 12.0 * 20,
+                "flops": cycle_flops + n * (2.0 * 100 + (law + 2 * faces if jac else 0.0))}
+    its = 12.0
+    solve = its * (cycle + 72.0 * n + 24.0 * n)
+    solve_flops = its * (cycle_flops + n * (13.0 + 12.0))
+    if c["op"] == "solve":
+        return {"bytes": solve, "flops": solve_flops}
+    return {"bytes": 3 * (solve + 8.0 * n * 15 + n * 12.0 * 20 + 24.0 * n) + field,
+            "flops": 3 * (solve_flops + n * (2 * law + 3 * faces + 2.0 * 100))}
+
+
+# ---------------------------------------------------------------- the same in plain torch FP64
+
+
+def _constitutive(p, ks):
+    """s, s', K, K' of the Haverkamp laws."""
+    so, ap = SOIL, (-p).clamp(min=1e-300)
+    pb, pg, wet = ap ** so.beta, ap ** so.gamma, p >= 0
+    S = so.alpha * (so.theta_s - so.theta_r) / (so.alpha + pb) + so.theta_r
+    dS = so.alpha * so.beta * (pb / ap) * (so.theta_s - so.theta_r) / (so.alpha + pb) ** 2
+    K = ks * so.a / (so.a + pg)
+    dK = so.a * so.gamma * ks * (pg / ap) / (so.a + pg) ** 2
+    zero = torch.zeros_like(p)
+    return (torch.where(wet, zero + so.theta_s, S), torch.where(wet, zero, dS), torch.where(wet, zero + ks, K),
+            torch.where(wet, zero, dK))
+
+
+def _mean(kind, kl, ku, pl, pu):
+    """Face conductivity and its derivatives by the lower and the upper cell's K."""
+    if kind == "arithmetic":
+        half = torch.full_like(kl, 0.5)
+        return 0.5 * (kl + ku), half, half
+    if kind == "upstream":
+        up = (pu - pl >= 0).double()
+        return torch.where(up > 0, ku, kl), 1 - up, up
+    if kind == "geometric":
+        g = torch.sqrt(kl * ku)
+        return g, 0.5 * g / kl, 0.5 * g / ku
+    s = kl + ku
+    return 2 * kl * ku / s, 2 * (ku / s) ** 2, 2 * (kl / s) ** 2
+
+
+def _faces(c, grid, bc, ks, p):
+    """Per axis and side: (p, K, dK) of the neighbour of every cell, and the masks of the faces that
+    carry a flux and of those with an unknown behind them."""
+    ksf = torch.full_like(p, SOIL.ks) if ks is None else ks.reshape(p.shape)
+    S, dS, K, dK = _constitutive(p, ksf)
+    out = []
+    for f in range(6):
+        dim, hi = 2 - (f >> 1), f & 1
+        n = p.shape[dim]
+        edge = [slice(None)] * 3
+        edge[dim] = slice(n - 1, n) if hi else slice(0, 1)
+        edge = tuple(edge)
+        value = bc.field(f)
+        gp = torch.full_like(p[edge], bc.value[f])
+        if value is not None:
+            gp = torch.as_tensor(value, dtype=torch.float64).cuda().reshape(gp.shape)
+        gk = _constitutive(gp, ksf[edge])[2]
+
+        def shift(a, ghost):
+            body = a.narrow(dim, 1, n - 1) if hi else a.narrow(dim, 0, n - 1)
+            return torch.cat([body, ghost], dim) if hi else torch.cat([ghost, body], dim)
+
+        inside = torch.ones_like(p, dtype=torch.bool)
+        inside[edge] = False
+        flux = inside.clone()
+        if bc.kind[f] == synth.BC_DIRICHLET:
+            flux[edge] = True
+        out.append((f, shift(p, gp), shift(K, gk), shift(dK, torch.zeros_like(gk)), flux, inside))
+    return S, dS, K, dK, out
+
+
+def _residual(c, grid, bc, ks, p, s_old):
+    S, _, K, _, faces = _faces(c, grid, bc, ks, p)
+    F = SOIL.rho_phi * (S - s_old) / c["dt"]
+    for f, pn, kn, _, flux, _ in faces:
+        h, side = grid.h[f >> 1], 1.0 if f & 1 else -1.0
+        ka = _mean(c["mean"], *((K, kn, p, pn) if f & 1 else (kn, K, pn, p)))[0]
+        t = ka * (p - pn) / (h * h)
+        if f >> 1 == 2:
+            t = t - side * (K + kn) / (2 * h)
+        F = F + torch.where(flux, t, torch.zeros_like(t))
+    return F
+
+
+def _jacobian(c, grid, bc, ks, p):
+    _, dS, K, dK, faces = _faces(c, grid, bc, ks, p)
+    J = torch.zeros((7,) + tuple(p.shape), dtype=torch.float64, device=p.device)
+    A = torch.zeros_like(J)
+    J[0] = A[0] = SOIL.rho_phi * dS / c["dt"]
+    zero = torch.zeros_like(p)
+    for f, pn, kn, dkn, flux, inside in faces:
+        h, side = grid.h[f >> 1], 1.0 if f & 1 else -1.0
+        if f & 1:
+            ka, own, other = _mean(c["mean"], K, kn, p, pn)
+        else:
+            ka, other, own = _mean(c["mean"], kn, K, pn, p)
+        w, dp = ka / (h * h), (p - pn) / (h * h)
+        diag, off = own * dK * dp + w, other * dkn * dp - w
+        if f >> 1 == 2:
+            diag, off = diag - side * dK / (2 * h), off - side * dkn / (2 * h)
+        J[0] += torch.where(flux, diag, zero)
+        A[0] += torch.where(flux, w, zero)
+        J[1 + f] = torch.where(inside, off, zero)
+        A[1 + f] = torch.where(inside, -w, zero)
+    return J, A
+
+
+def _apply(J, x):
+    y = J[0] * x
+    for f in range(6):
+        dim, n = 2 - (f >> 1), x.shape[2 - (f >> 1)]
+        if n < 2:
+            continue
+        lo, hi = (0, 1) if f & 1 else (1, 0)
+        y.narrow(dim, lo, n - 1).add_(J[1 + f].narrow(dim, lo, n - 1) * x.narrow(dim, hi, n - 1))
+    return y
+
+
+def _linear(J, b, tol=3e-14, cycles=6, maxit=4000):
+    """x with J x = b by diagonally scaled BiCGStab, restarted from the true residual; None if it stalls."""
+    dot = lambda u, v: float((u * v).sum())  # noqa: E731
+    d, bn = 1.0 / J[0], float(b.norm())
+    x, best = torch.zeros_like(b), math.inf
+    for _ in range(cycles):
+        r = b - _apply(J, x)
+        rn = float(r.norm())
+        if rn <= tol * bn or rn > 0.5 * best:
+            break
+        best, goal = rn, max(1e-10 * rn, 0.3 * tol * bn)
+        r0, rho, p, e = r.clone(), dot(r, r), r.clone(), torch.zeros_like(b)
+        for _ in range(maxit):
+            ph = d * p
+            v = _apply(J, ph)
+            alpha = rho / dot(r0, v)
+            s = r - alpha * v
+            sh = d * s
+            t = _apply(J, sh)
+            tt = dot(t, t)
+            if not tt > 0:
+                e = e + alpha * ph
+                break
+            w = dot(t, s) / tt
+            e = e + alpha * ph + w * sh
+            r = s - w * t
+            if not math.isfinite(w) or float(r.norm()) <= goal:
+                break
+            new = dot(r0, r)
+            p, rho = r + (new / rho) * (alpha / w) * (p - w * v), new
+        if bool(torch.isfinite(e).all()):
+            x = x + e
+    return x if float((b - _apply(J, x)).norm()) <= 1e-12 * bn else None
+
+
+def _newton(c, grid, bc, ks, p):
+    """p after a backward-Euler step from p, by damped Newton down to the rounding of the residual."""
+    s_old = _constitutive(p, SOIL.ks)[0]
+    F = _residual(c, grid, bc, ks, p, s_old)
+    fn = f0 = float(F.norm())
+    for _ in range(40):
+        d = _linear(_jacobian(c, grid, bc, ks, p)[0], -F, tol=1e-13)
+        if d is None:
+            return None
+        lam = 1.0
+        while True:
+            trial = p + lam * d
+            Ft = _residual(c, grid, bc, ks, trial, s_old)
+            ft = float(Ft.norm())
+            if ft < fn or lam < 1e-6:
+                break
+            lam *= 0.5
+        if not ft < fn:
+            return p if fn <= 1e-10 * f0 else None
+        p, F, fn = trial, Ft, ft
+        if float(d.norm()) <= 1e-13 * float(p.norm()):
+            return p
+    return p if fn <= 1e-10 * f0 else None
+
+
+def exact(case, seed):
+    c, grid = case, _grid(case)
+    bc = _bc(c, grid)
+    if c["op"] in ("vcycle", "setup", "refresh"):
+        return None  # what a V-cycle gives depends on the hierarchy: there is no value outside this package
+    ks = _conductivity(c, grid, seed)
+    if c["op"] == "batch":
+        got, n = [], grid.n
+        for b in range(c["batch"]):
+            p = torch.full((grid.nz, grid.ny, grid.nx), DRY, dtype=torch.float64, device="cuda")
+            q = _newton(c, grid, bc, _device_ks(None if ks is None else ks[b * n:(b + 1) * n]), p)
+            if q is None:
+                return None
+            got.append(q.reshape(-1))
+        return torch.cat(got)
+    p, ks = _pressure(c, grid, seed), _device_ks(ks)
+    if c["op"] == "jacobian":
+        J, A = _jacobian(c, grid, bc, ks, p)
+        return [J.reshape(-1), A.reshape(-1)]
+    if c["op"] == "step":
+        q = _newton(c, grid, bc, ks, p)
+        return None if q is None else q.reshape(-1)
+    s_old = _constitutive(_pressure(c, grid, seed, hours=-1), SOIL.ks)[0]
+    F = _residual(c, grid, bc, ks, p, s_old)
+    if c["op"] == "solve":
+        x = _linear(_jacobian(c, grid, bc, ks, p)[0], -F)
+        return None if x is None else x.reshape(-1)
+    return [F.reshape(-1), [float(F.norm()), float(F.abs().max())]]
