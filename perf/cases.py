@@ -61,7 +61,7 @@ def listed():
         # a whole backward-Euler step of the 128^3 workload
         dict(_case("step", 128, 128, 128, "upstream", dt=4.0), name="step_128"),
         # a batch of small same-shape requests stepped together
-        dict(_case("batch", 32, 32, 32, "upstream", sigma=0.25, mixed=True, krylov="fcg", nu=1, coarse=500, dt=0.25,
+        dict(_case("batch", 32, 32, 32, "upstream", sigma=0.25, mixed=True, krylov="fcg", nu=1, coarse=500, dt=0.1,
                    batch=8), name="batch_8x32"),
     ]
 
@@ -114,7 +114,7 @@ def draw(rng):
                      "arithmetic" if fcg else "upstream", dt=rng.choice([1.0, 4.0]), mixed=rng.random() < 0.5,
                      krylov="fcg" if fcg else "fgmres", nu=1 if fcg else 2, coarse=500 if fcg else 2000)
     return _case(op, _size(rng, 20, 36), _size(rng, 20, 36), _size(rng, 20, 36), "upstream", sigma=0.25, mixed=True,
-                 krylov="fcg", nu=1, coarse=500, dt=0.25, batch=rng.choice([2, 3, 5, 8]))
+                 krylov="fcg", nu=1, coarse=500, dt=0.1, batch=rng.choice([2, 3, 5, 8]))
 
 
 # ---------------------------------------------------------------- inputs
