@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/richards.h"
+#include "fixpow.cuh"
 
 namespace rich {
 
@@ -75,7 +76,23 @@ inline int red_grid(long long n) {
 
 struct SoilP {
   double alpha, beta, ts, tr, a, gamma, ks, rho_phi;
+  double cs, cds, cdk;        // alpha (ts - tr), alpha beta (ts - tr), a gamma
+  unsigned long long qb, qg;  // beta, gamma for fixpow_exp2; both 0: pow() throughout
 };
+
+// The fixed-point powers serve exponents in (0, 32) and constants whose sums with the
+// powers (below 2^960) have a normal reciprocal; other soils take pow().
+inline SoilP soil_params(const rich_soil* s) {
+  SoilP p{s->alpha, s->beta, s->theta_s, s->theta_r, s->a, s->gamma, s->ks_const, s->rho_phi};
+  p.cs = s->alpha * (s->theta_s - s->theta_r);
+  p.cds = s->alpha * s->beta * (s->theta_s - s->theta_r);
+  p.cdk = s->a * s->gamma;
+  p.qb = fixpow_exponent(s->beta);
+  p.qg = fixpow_exponent(s->gamma);
+  auto normal = [](double v) { return v >= 1e-280 && v <= 1e280; };
+  if (!p.qb || !p.qg || !normal(s->alpha) || !normal(s->a)) p.qb = p.qg = 0;
+  return p;
+}
 
 struct GridP {
   int nx, ny, nz;
@@ -307,35 +324,67 @@ namespace rich {
 
 // ---------------------------------------------------------------- device helpers
 
-// Constitutive law, eqs. (s(p)), (K(p)) and (derivativeofcoefficients) of Sec. 2-3.
-// |p|^beta and |p|^gamma share one log|p|; |p|^(x-1) = |p|^x / |p|.
+// Constitutive law, eqs. (s(p)), (K(p)) and (derivativeofcoefficients) of Sec. 2-3, for
+// p < 0 outside the fixed-point domain (|p| beyond 2^+-30, unusual soils); |p|^(x-1) =
+// |p|^x / |p|.
+struct Law {
+  double S, dS, K, dK;
+};
+static __device__ __noinline__ Law law_general(double ap, double ks, double alpha, double beta, double ts, double tr,
+                                               double a, double gamma) {
+  const double pb = pow(ap, beta);
+  const double pg = pow(ap, gamma);
+  const double r_ap = 1.0 / ap;
+  const double r_s = 1.0 / (alpha + pb);
+  const double r_k = 1.0 / (a + pg);
+  return Law{alpha * (ts - tr) * r_s + tr, alpha * beta * (pb * r_ap) * (ts - tr) * (r_s * r_s), ks * a * r_k,
+             a * gamma * ks * (pg * r_ap) * (r_k * r_k)};
+}
+__device__ __forceinline__ Law law_general(double p, double ks, const SoilP& so) {
+  return law_general(-p, ks, so.alpha, so.beta, so.ts, so.tr, so.a, so.gamma);
+}
+
+// Whether p is negative with |p| in the domain of the fixed-point powers (sign bit set,
+// binary exponent in [-30, 29]; integer tests: no FP64 compare).
+__device__ __forceinline__ bool law_fast(double p, const SoilP& so) {
+  constexpr unsigned lo = 0x80000000u | ((unsigned)(1023 - kFixPowExp) << 20);
+  return so.qb != 0 && (unsigned)__double2hiint(p) - lo < ((unsigned)(2 * kFixPowExp) << 20);
+}
+__device__ __forceinline__ long long law_log(double p) {
+  return fixpow_log2((unsigned long long)__double_as_longlong(p) & 0x7fffffffffffffffull);
+}
+
+// K(p) (and, below, the rest of the law) from the fixed-point powers: the sums, one
+// reciprocal each and the products are all that runs in FP64 (K alone 6 operations, the
+// whole law 23 against about 95 through log()/exp() and divisions).  FP64 pipe bound
+// both ways: the law of 2.1M cells took 380 us before and takes 110.
+__device__ __forceinline__ double conductivity_only(double p, double ks, const SoilP& so) {
+  if (law_fast(p, so)) return (ks * so.a) * fast_rcp(so.a + fixpow_exp2(law_log(p), so.qg));
+  return p < 0.0 ? law_general(p, ks, so).K : ks;
+}
+
 __device__ __forceinline__ void constit(double p, double ks, const SoilP& so, double& S, double& dS,
                                         double& K, double& dK) {
-  if (p < 0.0) {
-    double ap = -p;
-    double lp = log(ap);
-    double pb = exp(so.beta * lp);
-    double pg = exp(so.gamma * lp);
-    // three reciprocals instead of six divisions (FP64 division is a software
-    // sequence on GB300's narrow FP64 pipe)
-    const double r_ap = 1.0 / ap;
-    const double r_s = 1.0 / (so.alpha + pb);
-    const double r_k = 1.0 / (so.a + pg);
-    S = so.alpha * (so.ts - so.tr) * r_s + so.tr;
-    dS = so.alpha * so.beta * (pb * r_ap) * (so.ts - so.tr) * (r_s * r_s);
-    K = ks * so.a * r_k;
-    dK = so.a * so.gamma * ks * (pg * r_ap) * (r_k * r_k);
+  if (law_fast(p, so)) {
+    const long long y = law_log(p);
+    const double pb = fixpow_exp2(y, so.qb), pg = fixpow_exp2(y, so.qg);
+    const double r_ap = fast_rcp(-p), r_s = fast_rcp(so.alpha + pb), r_k = fast_rcp(so.a + pg);
+    S = fma(so.cs, r_s, so.tr);
+    dS = (so.cds * (pb * r_ap)) * (r_s * r_s);
+    K = (ks * so.a) * r_k;
+    dK = (so.cdk * ks) * (pg * r_ap) * (r_k * r_k);
+  } else if (p < 0.0) {
+    const Law w = law_general(p, ks, so);
+    S = w.S;
+    dS = w.dS;
+    K = w.K;
+    dK = w.dK;
   } else {
     S = so.ts;
     dS = 0.0;
     K = ks;
     dK = 0.0;
   }
-}
-
-__device__ __forceinline__ double conductivity_only(double p, double ks, const SoilP& so) {
-  if (p < 0.0) return ks * so.a / (so.a + exp(so.gamma * log(-p)));
-  return ks;
 }
 
 // The mean used on the faces normal to axis: a split code (RICH_KMEAN_SPLIT) takes

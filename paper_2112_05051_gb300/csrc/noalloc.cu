@@ -170,8 +170,7 @@ extern "C" int rich_residual_noalloc(const rich_grid* grid, const rich_soil* soi
     g.inv_h[d] = 1.0 / h[d];
     g.inv_h2[d] = 1.0 / (h[d] * h[d]);
   }
-  SoilP so{soil->alpha, soil->beta, soil->theta_s, soil->theta_r, soil->a, soil->gamma, soil->ks_const,
-           soil->rho_phi};
+  const SoilP so = soil_params(soil);
   BCP b;
   for (int f = 0; f < 6; ++f) {
     b.kind[f] = bc->kind[f];

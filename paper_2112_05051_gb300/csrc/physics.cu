@@ -478,8 +478,7 @@ int rich_create(const rich_grid* grid, const rich_soil* soil, int kmean, const r
     c->g.inv_h[d] = 1.0 / h[d];
     c->g.inv_h2[d] = 1.0 / (h[d] * h[d]);
   }
-  c->soil = SoilP{soil->alpha, soil->beta, soil->theta_s, soil->theta_r, soil->a, soil->gamma, soil->ks_const,
-                  soil->rho_phi};
+  c->soil = soil_params(soil);
   for (int f = 0; f < 6; ++f) {
     c->bc.kind[f] = bc->kind[f];
     c->bc.value[f] = bc->value[f];
