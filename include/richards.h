@@ -361,7 +361,7 @@ int rich_residual3(rich_ctx* ctx, const double* p_dev, const double* s_old_dev, 
  * Inputs as for rich_create/rich_residual (soil->ks_field_dev is read in place,
  * not copied); F_dev receives Phi; norms_host, if not NULL, receives
  * {||Phi||_2, ||Phi||_inf} and the call then synchronises the stream.
- * The only scratch is a file-scope device array of about 1 MB shared by all
+ * The only scratch is a file-scope device array of about 40 kB shared by all
  * calls; grids above 134,217,728 cells (512^3) return RICH_ELIMIT.  The first
  * call on a device looks up the array's device address (cudaGetSymbolAddress),
  * so make that first call before any stream capture.  Calls that overlap on the

@@ -288,11 +288,8 @@ static int batch_step(rich_ctx* c, BatchWork& w, int S, double* p, double dt, co
   }
   std::vector<double> fn(S), tol(S), flo(S), f0(S), slope(S), lam(S), ft(S), flo_t(S);
   std::vector<int> conv(S, 0), done(S, 0), newton_act(S, 0), search(S, 0), lin_fail, lin_its;
-  RICH_CHECK(constit_eval(c, p));
-  RICH_CUDA(cudaMemcpyAsync(c->s_old, c->S, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
-  RICH_CHECK(residual_eval(c, p, c->s_old, dt, c->F, true, true, S));
-  RICH_CUDA(cudaMemcpyAsync(w.hsc, c->dsc, sizeof(double) * 3 * S, cudaMemcpyDeviceToHost, c->st));
-  RICH_CUDA(cudaStreamSynchronize(c->st));
+  RICH_CHECK(residual_eval(c, p, nullptr, dt, c->F, true, true, c->s_old, S));
+  RICH_CHECK(wait_scalars(c, 3 * S, w.hsc));
   for (int s = 0; s < S; ++s) {
     fn[s] = sqrt(w.hsc[s]);
     flo[s] = kFloor * sqrt(w.hsc[2 * S + s]);
@@ -365,9 +362,8 @@ static int batch_step(rich_ctx* c, BatchWork& w, int S, double* p, double dt, co
       RICH_CUDA(cudaMemcpyAsync(w.dlam, w.hsc, sizeof(double) * S, cudaMemcpyHostToDevice, c->st));
       k_seg_axpby<<<vgrid, kBlock, 0, c->st>>>(ns, p, w.dlam, c->d, c->ptrial);
       RICH_LAUNCH_CHECK();
-      RICH_CHECK(residual_eval(c, c->ptrial, c->s_old, dt, c->Ft, true, false, S));
-      RICH_CUDA(cudaMemcpyAsync(w.hsc, c->dsc, sizeof(double) * 3 * S, cudaMemcpyDeviceToHost, c->st));
-      RICH_CUDA(cudaStreamSynchronize(c->st));
+      RICH_CHECK(residual_eval(c, c->ptrial, c->s_old, dt, c->Ft, true, true, nullptr, S));
+      RICH_CHECK(wait_scalars(c, 3 * S, w.hsc));
       bool more = false;
       for (int s = 0; s < S; ++s) {
         ft[s] = 0.5 * w.hsc[s];
@@ -442,8 +438,7 @@ int rich_create_batch(const rich_grid* grid, int nbatch, const rich_soil* soil, 
   int s = rich_create(&g, soil, kmean, bc, precision, stream, out);
   if (s != RICH_OK) return s;
   (*out)->g.nzs = grid->nz;
-  (*out)->g.inv_h[2] = 1.0 / hz;
-  (*out)->g.inv_h2[2] = 1.0 / (hz * hz);
+  (*out)->g.set_spacing(hs);
   (*out)->nbatch = nbatch;
   return RICH_OK;
 }

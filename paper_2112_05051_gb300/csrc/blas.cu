@@ -174,6 +174,12 @@ int fetch_scalars(rich_ctx* c, const double* dsrc, int count, double* host) {
   return RICH_OK;
 }
 
+int wait_scalars(rich_ctx* c, int count, double* host) {
+  RICH_CUDA(cudaStreamSynchronize(c->st));
+  for (int i = 0; i < count; ++i) host[i] = c->hsc[i];
+  return RICH_OK;
+}
+
 // ---------------------------------------------------------------- dot products
 
 __global__ void k_dot(const double* __restrict__ x, const double* __restrict__ y, long long n,

@@ -76,7 +76,7 @@ inline int red_grid(long long n) {
 
 struct SoilP {
   double alpha, beta, ts, tr, a, gamma, ks, rho_phi;
-  double cs, cds, cdk;        // alpha (ts - tr), alpha beta (ts - tr), a gamma
+  double cs, cds, cdk, cka;   // alpha (ts - tr), alpha beta (ts - tr), a gamma, ks a
   unsigned long long qb, qg;  // beta, gamma for fixpow_exp2; both 0: pow() throughout
 };
 
@@ -87,6 +87,7 @@ inline SoilP soil_params(const rich_soil* s) {
   p.cs = s->alpha * (s->theta_s - s->theta_r);
   p.cds = s->alpha * s->beta * (s->theta_s - s->theta_r);
   p.cdk = s->a * s->gamma;
+  p.cka = s->ks_const * s->a;
   p.qb = fixpow_exponent(s->beta);
   p.qg = fixpow_exponent(s->gamma);
   auto normal = [](double v) { return v >= 1e-280 && v <= 1e280; };
@@ -100,6 +101,18 @@ struct GridP {
   long long n;
   double inv_h[3];   // 1/h_d
   double inv_h2[3];  // 1/h_d^2
+  double half_h2[3]; // 1/(2 h_d^2)
+  double twice_h2[3];  // 2/h_d^2
+  double half_hz;    // 1/(2 h_z)
+  void set_spacing(const double h[3]) {
+    for (int d = 0; d < 3; ++d) {
+      inv_h[d] = 1.0 / h[d];
+      inv_h2[d] = 1.0 / (h[d] * h[d]);
+      half_h2[d] = 0.5 * inv_h2[d];
+      twice_h2[d] = 2.0 * inv_h2[d];
+    }
+    half_hz = 0.5 * inv_h[2];
+  }
 };
 
 struct BCP {
@@ -285,10 +298,9 @@ struct rich_ctx {
   cudaStream_t st = nullptr;
   int device = 0;
   double* ks = nullptr;        // per-cell K_s or nullptr
-  // constitutive values at the last p given to constit()
+  // K, K' and s' at the last p of a constitutive pass or a storing residual
   double* K = nullptr;
   double* dK = nullptr;
-  double* S = nullptr;
   double* dS = nullptr;
   // stencils (7n)
   double* J7 = nullptr;
@@ -303,6 +315,7 @@ struct rich_ctx {
   double* partials = nullptr;  // kRedBlocks * 64
   double* dsc = nullptr;       // device scalars (256)
   double* hsc = nullptr;       // pinned host mirror (128)
+  unsigned* ticket = nullptr;  // finished blocks per segment of a reduction (32, zero between launches)
   int* iflag = nullptr;        // device int flags (16)
   int* hflag = nullptr;        // pinned host (16)
   // Newton work
@@ -358,9 +371,16 @@ __device__ __forceinline__ long long law_log(double p) {
 // reciprocal each and the products are all that runs in FP64 (K alone 6 operations, the
 // whole law 23 against about 95 through log()/exp() and divisions).  FP64 pipe bound
 // both ways: the law of 2.1M cells took 380 us before and takes 110.
-__device__ __forceinline__ double conductivity_only(double p, double ks, const SoilP& so) {
-  if (law_fast(p, so)) return (ks * so.a) * fast_rcp(so.a + fixpow_exp2(law_log(p), so.qg));
+__device__ __forceinline__ double conductivity_only(double p, double ks, double ksa, const SoilP& so) {
+  if (law_fast(p, so)) return ksa * fast_rcp(so.a + fixpow_exp2(law_log(p), so.qg));
   return p < 0.0 ? law_general(p, ks, so).K : ks;
+}
+__device__ __forceinline__ double conductivity_only(double p, double ks, const SoilP& so) {
+  return conductivity_only(p, ks, ks * so.a, so);
+}
+__device__ __forceinline__ double saturation_only(double p, const SoilP& so) {
+  if (law_fast(p, so)) return fma(so.cs, fast_rcp(so.alpha + fixpow_exp2(law_log(p), so.qb)), so.tr);
+  return p < 0.0 ? law_general(p, 1.0, so).S : so.ts;
 }
 
 __device__ __forceinline__ void constit(double p, double ks, const SoilP& so, double& S, double& dS,
@@ -397,6 +417,19 @@ inline bool kmean_valid(int kmean) {
   if (kmean >= 0 && kmean <= 3) return true;
   if ((kmean & ~0x1FF) != 0 || !(kmean & RICH_KMEAN_SPLIT_FLAG)) return false;
   return ((kmean >> 4) & 0xF) <= 3 && (kmean & 0xF) <= 3;
+}
+
+// Whether the upstream mean takes the upper cell, p_U - p_L >= 0, for dp = p_L - p_U
+// (an integer test: sign bit or zero).
+__device__ __forceinline__ bool dp_upstream(double dp) {
+  const int hi = __double2hiint(dp);
+  return hi < 0 || (hi | __double2loint(dp)) == 0;
+}
+
+// 1/q: three FP64 operations where q's exponent leaves room, else a division.
+__device__ __forceinline__ double safe_rcp(double q) {
+  const unsigned e = ((unsigned)__double2hiint(q) >> 20) & 0x7ffu;
+  return e - 123u < 1800u ? fast_rcp(q) : 1.0 / q;
 }
 
 // Face mean between the lower (L) and upper (+d side, U) cell and its partials.
@@ -525,12 +558,18 @@ void dfree(T*& p) {
 
 // physics.cu
 int constit_eval(rich_ctx* c, const double* p);
-// constit_current: the context's K, K', s, s' already hold the values of this p
-// (the last constitutive evaluation was at the same pressure), so they are reused.
-// nseg > 1: the grid stacks nseg problems along z and the norms are summed per problem
-// (dsc[q * nseg + s] for quantity q of problem s).
+// Phi(p) into F.  Newton's form also stores K, K' and s' for the Jacobian at this p and sums
+// the round-off scale.  s_init, if not NULL: s_old is not read, s(p) stands in for it (Phi at
+// the start of a step) and is written there.
+// norms: the sums, per problem when nseg > 1 (the grid stacks nseg problems along z), are
+// left at dsc[q * nseg + s] and in the pinned mirror hsc (quantity q: 0 ||F||^2, 1 ||F||_inf,
+// 2 ||term magnitudes||^2, Newton's form only), valid once the stream has been waited for.
 int residual_eval(rich_ctx* c, const double* p, const double* s_old, double dt, double* F, bool want_norms,
-                  bool constit_current = false, int nseg = 1);
+                  bool newton = false, double* s_init = nullptr, int nseg = 1);
+// Waits for the context's stream and returns the first `count` scalars of the pinned mirror.
+int wait_scalars(rich_ctx* c, int count, double* host);
+// constit_current: the context's K, K', s' already hold the values of this p (the last
+// storing residual was at the same pressure).
 int jacobian_eval(rich_ctx* c, const double* p, double dt, bool constit_current = false);
 int stencil_apply(rich_ctx* c, const double* A7, const double* x, double* y);
 int refresh_a0_values(rich_ctx* c);

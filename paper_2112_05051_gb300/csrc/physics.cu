@@ -11,7 +11,7 @@
 // The Jacobian is its exact derivative (chain rule through K_av; Supplementary A
 // and C print the interior entries), and the diffusion-only matrix keeps
 // K_av/h_d^2 couplings plus the storage diagonal (Sec. 4, q_prec = -K grad p).
-#include "common.cuh"
+#include "residual.cuh"
 
 namespace rich {
 
@@ -22,15 +22,13 @@ void set_cuda_error(cudaError_t e, const char* where) {
 }
 
 __global__ void k_constit(long long n, SoilP so, const double* __restrict__ p, const double* __restrict__ ks,
-                          double* __restrict__ K, double* __restrict__ dK, double* __restrict__ S,
-                          double* __restrict__ dS) {
+                          double* __restrict__ K, double* __restrict__ dK, double* __restrict__ dS) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
        c += (long long)gridDim.x * blockDim.x) {
     double s_, ds_, k_, dk_;
     constit(p[c], ks ? ks[c] : so.ks, so, s_, ds_, k_, dk_);
     K[c] = k_;
     dK[c] = dk_;
-    S[c] = s_;
     dS[c] = ds_;
   }
 }
@@ -90,9 +88,7 @@ __global__ void k_face_apply(GridP g, int f, long long m, const double* __restri
 __global__ void k_saturation(long long n, SoilP so, const double* __restrict__ p, double* __restrict__ s) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
        c += (long long)gridDim.x * blockDim.x) {
-    double s_, ds_, k_, dk_;
-    constit(p[c], so.ks, so, s_, ds_, k_, dk_);
-    s[c] = s_;
+    s[c] = saturation_only(p[c], so);
   }
 }
 
@@ -136,61 +132,6 @@ __device__ __forceinline__ bool face_neighbour(const GridP& g, const BCP& bc, co
   nb.dK = dK ? dK[q] : 0.0;
   nb.idx = q;
   return true;
-}
-
-__global__ void k_residual(GridP g, SoilP so, BCP bc, int kmean, const double* __restrict__ p,
-                           const double* __restrict__ K, const double* __restrict__ S,
-                           const double* __restrict__ s_old, const double* __restrict__ ks, double dt,
-                           double* __restrict__ F, double* __restrict__ partials) {
-  double acc[2] = {0.0, 0.0};
-  double amax = 0.0;
-  const double rdt = so.rho_phi / dt;  // one division per thread, not per cell
-  // gridDim.y problems stacked along z: block row y sums the cells of problem y
-  const long long ns = g.n / gridDim.y;
-  const long long c0 = (long long)blockIdx.y * ns, c1 = c0 + ns;
-  for (long long c = c0 + blockIdx.x * (long long)blockDim.x + threadIdx.x; c < c1;
-       c += (long long)gridDim.x * blockDim.x) {
-    int i = (int)(c % g.nx);
-    long long r = c / g.nx;
-    int j = (int)(r % g.ny);
-    int k = (int)(r / g.ny);
-    double pc = p[c], Kc = K[c];
-    double ksc = ks ? ks[c] : so.ks;
-    double sc = S[c], so_c = s_old[c];
-    double phi = (sc - so_c) * rdt;
-    double mag = (fabs(sc) + fabs(so_c)) * rdt;
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      FaceNb nb;
-      if (!face_neighbour(g, bc, so, f, i, j, k, c, p, K, nullptr, ksc, nb)) continue;
-      int axis = f >> 1;
-      double side = (f & 1) ? 1.0 : -1.0;
-      double dL, dU;
-      double ka = (f & 1) ? face_mean(axis_mean(kmean, axis), Kc, nb.K, pc, nb.p, dL, dU)
-                          : face_mean(axis_mean(kmean, axis), nb.K, Kc, nb.p, pc, dL, dU);
-      double t = ka * (pc - nb.p) * g.inv_h2[axis];
-      double m = ka * (fabs(pc) + fabs(nb.p)) * g.inv_h2[axis];
-      if (axis == 2) {
-        t -= side * (Kc + nb.K) * 0.5 * g.inv_h[2];
-        m += (Kc + nb.K) * 0.5 * g.inv_h[2];
-      }
-      phi += t;
-      mag += m;
-    }
-    F[c] = phi;
-    acc[0] += phi * phi;
-    acc[1] += mag * mag;
-    double a = fabs(phi);
-    amax = (a > amax || a != a) ? a : amax;  // NaN propagates into the max
-  }
-  block_sum<2>(acc);
-  double m = block_max(amax);
-  if (threadIdx.x == 0) {  // partials[(q * nseg + seg) * gridDim.x + block]
-    const long long S = gridDim.y, b = blockIdx.y * (long long)gridDim.x + blockIdx.x;
-    partials[b] = acc[0];
-    partials[S * gridDim.x + b] = m;
-    partials[2 * S * gridDim.x + b] = acc[1];
-  }
 }
 
 __global__ void k_assemble(GridP g, SoilP so, BCP bc, int kmean, const double* __restrict__ p,
@@ -305,28 +246,29 @@ __global__ void k_a0_fill(GridP g, const int* __restrict__ rowptr, int* __restri
 // ---------------------------------------------------------------- host wrappers
 
 int constit_eval(rich_ctx* c, const double* p) {
-  k_constit<<<grid_for(c->g.n), kBlock, 0, c->st>>>(c->g.n, c->soil, p, c->ks, c->K, c->dK, c->S, c->dS);
+  k_constit<<<grid_for(c->g.n), kBlock, 0, c->st>>>(c->g.n, c->soil, p, c->ks, c->K, c->dK, c->dS);
   RICH_LAUNCH_CHECK();
   return RICH_OK;
 }
 
 int residual_eval(rich_ctx* c, const double* p, const double* s_old, double dt, double* F, bool want_norms,
-                  bool constit_current, int nseg) {
-  if (!constit_current) RICH_CHECK(constit_eval(c, p));
-  int nb = red_grid(c->g.n / nseg);
-  if ((long long)nb * nseg * 3 > (long long)kRedBlocks * 64) return RICH_ELIMIT;  // partials buffer
+                  bool newton, double* s_init, int nseg) {
+  // three quantities per segment and block in the partials buffer
+  const int room = kRedBlocks * 64 / (3 * nseg);
+  const ResPlan pl = residual_plan(c->g, nseg, std::min(16 * kNumSM, room));
+  ResOut out{};
+  if (want_norms) out = ResOut{c->partials, (long long)nseg * pl.nb, c->ticket, c->dsc, c->hsc};
+  const double rdt = c->soil.rho_phi / dt;
   {
-    ProfScope ps("residual", c->st, (double)c->g.n * (32.0 + (c->ks ? 8.0 : 0.0)));
-    k_residual<<<dim3(nb, nseg), kBlock, 0, c->st>>>(c->g, c->soil, c->bc, c->kmean, p, c->K, c->S, s_old, c->ks, dt,
-                                                     F, c->partials);
+    ProfScope ps("residual", c->st, (double)c->g.n * (24.0 + (newton ? 24.0 : 0.0) + (c->ks ? 8.0 : 0.0)));
+    if (newton)
+      residual_launch<true>(pl, nseg, c->st, c->g, c->soil, c->bc, c->kmean, p, s_old, c->ks, rdt, F, c->K, c->dK,
+                            c->dS, s_init, out);
+    else
+      residual_launch<false>(pl, nseg, c->st, c->g, c->soil, c->bc, c->kmean, p, s_old, c->ks, rdt, F, nullptr, nullptr,
+                             nullptr, nullptr, out);
   }
   RICH_LAUNCH_CHECK();
-  if (want_norms) {  // dsc[q * nseg + s]: q = 0 ||F||^2, 1 ||F||_inf, 2 ||term magnitudes||^2
-    const long long S = nseg;
-    RICH_CHECK(finish_sums(c, c->partials, nb, nseg, c->dsc + 0));
-    for (int s = 0; s < nseg; ++s) RICH_CHECK(finish_max(c, c->partials + (S + s) * nb, nb, c->dsc + S + s));
-    RICH_CHECK(finish_sums(c, c->partials + 2 * S * nb, nb, nseg, c->dsc + 2 * S));
-  }
   return RICH_OK;
 }
 
@@ -474,10 +416,7 @@ int rich_create(const rich_grid* grid, const rich_soil* soil, int kmean, const r
   c->g.n = n;
   double h[3];
   grid_spacing(grid, h);
-  for (int d = 0; d < 3; ++d) {
-    c->g.inv_h[d] = 1.0 / h[d];
-    c->g.inv_h2[d] = 1.0 / (h[d] * h[d]);
-  }
+  c->g.set_spacing(h);
   c->soil = soil_params(soil);
   for (int f = 0; f < 6; ++f) {
     c->bc.kind[f] = bc->kind[f];
@@ -495,10 +434,11 @@ int rich_create(const rich_grid* grid, const rich_soil* soil, int kmean, const r
     rich_destroy(c);
     return st_;
   };
-  if ((s = dalloc(&c->K, n)) || (s = dalloc(&c->dK, n)) || (s = dalloc(&c->S, n)) || (s = dalloc(&c->dS, n)) ||
+  if ((s = dalloc(&c->K, n)) || (s = dalloc(&c->dK, n)) || (s = dalloc(&c->dS, n)) || (s = dalloc(&c->ticket, 32)) ||
       (s = dalloc(&c->J7, 7 * n)) || (s = dalloc(&c->A7, 7 * n)) || (s = dalloc(&c->partials, (long long)kRedBlocks * 64)) ||
       (s = dalloc(&c->dsc, 256)) || (s = dalloc(&c->iflag, 16)))
     return fail(s);
+  if (cudaMemsetAsync(c->ticket, 0, 32 * sizeof(unsigned), c->st) != cudaSuccess) return fail(RICH_ECUDA);
   {
     // 128 doubles then 16 ints of pinned host memory from the process-wide pool
     char* blk = static_cast<char*>(pinned_get());
@@ -546,7 +486,7 @@ int rich_destroy(rich_ctx* c) {
   dfree(c->ks);
   dfree(c->K);
   dfree(c->dK);
-  dfree(c->S);
+  dfree(c->ticket);
   dfree(c->dS);
   dfree(c->J7);
   dfree(c->A7);
@@ -630,7 +570,7 @@ int rich_residual(rich_ctx* c, const double* p, const double* s_old, double dt, 
   RICH_CHECK(residual_eval(c, p, s_old, dt, F, norms != nullptr));
   if (norms) {
     double h[2];
-    RICH_CHECK(fetch_scalars(c, c->dsc, 2, h));
+    RICH_CHECK(wait_scalars(c, 2, h));
     norms[0] = sqrt(h[0]);
     norms[1] = h[1];
     if (!std::isfinite(norms[0]) || !std::isfinite(norms[1])) return RICH_ENONFINITE;
@@ -641,9 +581,9 @@ int rich_residual(rich_ctx* c, const double* p, const double* s_old, double dt, 
 int rich_residual3(rich_ctx* c, const double* p, const double* s_old, double dt, double* F, double* norms) {
   if (!c || !p || !s_old || !F || !norms || !(dt > 0)) return RICH_EINVAL;
   AllocStream guard(c->st);
-  RICH_CHECK(residual_eval(c, p, s_old, dt, F, true));
+  RICH_CHECK(residual_eval(c, p, s_old, dt, F, true, true));
   double h[3];
-  RICH_CHECK(fetch_scalars(c, c->dsc, 3, h));  // ||F||^2, ||F||_inf, ||m||^2
+  RICH_CHECK(wait_scalars(c, 3, h));  // ||F||^2, ||F||_inf, ||m||^2
   norms[0] = sqrt(h[0]);
   norms[1] = h[1];
   norms[2] = sqrt(h[2]);

@@ -1584,12 +1584,9 @@ static int step_body(rich_ctx* c, double* p, double dt, const rich_newton_opts* 
   double h[3];
   {
     Phase ph(pt, &st->ms_feval);
-    // s_old = s(p^{l-1}) is the saturation the constitutive pass computes at p
-    RICH_CHECK(constit_eval(c, p));
-    RICH_CUDA(cudaMemcpyAsync(c->s_old, c->S, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
-    RICH_CHECK(residual_eval(c, p, c->s_old, dt, c->F, true, true));
+    RICH_CHECK(residual_eval(c, p, nullptr, dt, c->F, true, true, c->s_old));  // s_old = s(p^{l-1})
   }
-  RICH_CHECK(fetch_scalars(c, c->dsc, 3, h));
+  RICH_CHECK(wait_scalars(c, 3, h));
   double fn = sqrt(h[0]);
   double floor_ = kFloor * sqrt(h[2]);
   if (!std::isfinite(fn)) return RICH_ENONFINITE;
@@ -1648,9 +1645,9 @@ static int step_body(rich_ctx* c, double* p, double dt, const rich_newton_opts* 
         Phase ph(pt, &st->ms_feval);
         k_axpby<<<g, kBlock, 0, c->st>>>(n, p, lam, c->d, c->ptrial);
         RICH_LAUNCH_CHECK();
-        RICH_CHECK(residual_eval(c, c->ptrial, c->s_old, dt, c->Ft, true));
+        RICH_CHECK(residual_eval(c, c->ptrial, c->s_old, dt, c->Ft, true, true));
       }
-      RICH_CHECK(fetch_scalars(c, c->dsc, 3, h));
+      RICH_CHECK(wait_scalars(c, 3, h));
       st->line_search_evals++;
       ft = 0.5 * h[0];
       floor_t = kFloor * sqrt(h[2]);
