@@ -432,37 +432,6 @@ __device__ __forceinline__ double safe_rcp(double q) {
   return e - 123u < 1800u ? fast_rcp(q) : 1.0 / q;
 }
 
-// Face mean between the lower (L) and upper (+d side, U) cell and its partials.
-__device__ __forceinline__ double face_mean(int kmean, double kL, double kU, double pL, double pU,
-                                            double& dL, double& dU) {
-  if (kmean == RICH_KMEAN_ARITH) {
-    dL = 0.5;
-    dU = 0.5;
-    return 0.5 * (kL + kU);
-  }
-  if (kmean == RICH_KMEAN_UPSTREAM) {
-    bool up = (pU - pL) >= 0.0;
-    dL = up ? 0.0 : 1.0;
-    dU = up ? 1.0 : 0.0;
-    return up ? kU : kL;
-  }
-  if (kmean == RICH_KMEAN_GEOMETRIC) {
-    double g = sqrt(kL * kU);
-    dL = kL > 0.0 ? 0.5 * g / kL : 0.0;
-    dU = kU > 0.0 ? 0.5 * g / kU : 0.0;
-    return g;
-  }
-  double s = kL + kU;
-  if (s > 0.0) {
-    double is = 1.0 / s;
-    dL = 2.0 * kU * kU * is * is;
-    dU = 2.0 * kL * kL * is * is;
-    return 2.0 * kL * kU * is;
-  }
-  dL = dU = 0.0;
-  return 0.0;
-}
-
 // Warp/block sum of NQ doubles in a fixed order; result valid in thread 0.
 template <int NQ>
 __device__ __forceinline__ void block_sum(double (&v)[NQ]) {
@@ -570,7 +539,9 @@ int residual_eval(rich_ctx* c, const double* p, const double* s_old, double dt, 
 int wait_scalars(rich_ctx* c, int count, double* host);
 // constit_current: the context's K, K', s' already hold the values of this p (the last
 // storing residual was at the same pressure).
-int jacobian_eval(rich_ctx* c, const double* p, double dt, bool constit_current = false);
+// J7b, A7b, if not NULL, receive copies of the two stencils.
+int jacobian_eval(rich_ctx* c, const double* p, double dt, bool constit_current = false, double* J7b = nullptr,
+                  double* A7b = nullptr);
 int stencil_apply(rich_ctx* c, const double* A7, const double* x, double* y);
 int refresh_a0_values(rich_ctx* c);
 

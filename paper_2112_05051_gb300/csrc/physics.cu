@@ -92,95 +92,179 @@ __global__ void k_saturation(long long n, SoilP so, const double* __restrict__ p
   }
 }
 
-// Neighbour data of face f of cell (i,j,k).  Returns false for a no-flux boundary face.
-struct FaceNb {
+// A neighbour as the assembly sees it; `unknown` false for a Dirichlet ghost.
+struct AsmNb {
   double p, K, dK;
-  long long idx;   // -1 for a Dirichlet ghost, kInterfaceGhost for a neighbouring subdomain's cell
+  bool unknown;
 };
-constexpr long long kInterfaceGhost = -2;
 
-__device__ __forceinline__ bool face_neighbour(const GridP& g, const BCP& bc, const SoilP& so, int f, int i, int j,
-                                               int k, long long c, const double* __restrict__ p,
-                                               const double* __restrict__ K, const double* __restrict__ dK,
-                                               double ksc, FaceNb& nb) {
-  int axis = f >> 1;
-  int side = (f & 1) ? 1 : -1;
-  // a batch stacks problems along z: their top and bottom layers are boundaries
-  int coord = axis == 0 ? i : (axis == 1 ? j : (g.nzs == g.nz ? k : k % g.nzs));
-  int extent = axis == 0 ? g.nx : (axis == 1 ? g.ny : g.nzs);
-  bool bnd = side > 0 ? (coord == extent - 1) : (coord == 0);
-  if (bnd) {
-    if (bc.kind[f] == RICH_BC_NOFLUX) return false;
-    nb.p = bc_value(bc, f, i, j, k, g.nx, g.ny);
-    if (bc.kind[f] == RICH_BC_INTERFACE) {  // a cell of the neighbouring subdomain, with its own K_s
-      const double* gk = bc.gks[f];
-      double s_, ds_;
-      constit(nb.p, gk ? gk[face_index(f, i, j, k, g.nx, g.ny)] : so.ks, so, s_, ds_, nb.K, nb.dK);
-      if (!dK) nb.dK = 0.0;
-      nb.idx = kInterfaceGhost;
-      return true;
-    }
+// Ghost of the boundary cell (i, j, k) on face f; false for a no-flux face.
+__device__ __forceinline__ bool asm_ghost(const GridP& g, const BCP& bc, const SoilP& so, int f, int i, int j, int k,
+                                          double ksc, AsmNb& nb) {
+  if (bc.kind[f] == RICH_BC_NOFLUX) return false;
+  nb.p = bc_value(bc, f, i, j, k, g.nx, g.ny);
+  nb.unknown = bc.kind[f] == RICH_BC_INTERFACE;
+  if (nb.unknown) {  // a cell of the neighbouring subdomain, with its own K_s
+    const double* gk = bc.gks[f];
+    double s, ds;
+    constit(nb.p, gk ? gk[face_index(f, i, j, k, g.nx, g.ny)] : so.ks, so, s, ds, nb.K, nb.dK);
+  } else {
     nb.K = conductivity_only(nb.p, ksc, so);
     nb.dK = 0.0;
-    nb.idx = -1;
-    return true;
   }
-  long long stride = axis == 0 ? 1LL : (axis == 1 ? (long long)g.nx : (long long)g.nx * g.ny);
-  long long q = c + side * stride;
-  nb.p = p[q];
-  nb.K = K[q];
-  nb.dK = dK ? dK[q] : 0.0;
-  nb.idx = q;
   return true;
 }
 
-__global__ void k_assemble(GridP g, SoilP so, BCP bc, int kmean, const double* __restrict__ p,
-                           const double* __restrict__ K, const double* __restrict__ dK,
-                           const double* __restrict__ dS, const double* __restrict__ ks, double dt,
-                           double* __restrict__ J7, double* __restrict__ A7) {
-  const double rdt = so.rho_phi / dt;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < g.n;
-       c += (long long)gridDim.x * blockDim.x) {
-    int i = (int)(c % g.nx);
-    long long r = c / g.nx;
-    int j = (int)(r % g.ny);
-    int k = (int)(r / g.ny);
-    double pc = p[c], Kc = K[c], dKc = dK[c];
-    double ksc = ks ? ks[c] : so.ks;
-    double dj = dS[c] * rdt;
-    double da = dj;
-#pragma unroll
-    for (int f = 0; f < 6; ++f) {
-      FaceNb nb;
-      double offj = 0.0, offa = 0.0;
-      if (face_neighbour(g, bc, so, f, i, j, k, c, p, K, dK, ksc, nb)) {
-        int axis = f >> 1;
-        double side = (f & 1) ? 1.0 : -1.0;
-        double dL, dU;
-        double ka = (f & 1) ? face_mean(axis_mean(kmean, axis), Kc, nb.K, pc, nb.p, dL, dU)
-                            : face_mean(axis_mean(kmean, axis), nb.K, Kc, nb.p, pc, dL, dU);
-        double dself = (f & 1) ? dL : dU;
-        double dnb = (f & 1) ? dU : dL;
-        double w = ka * g.inv_h2[axis];
-        double dp = (pc - nb.p) * g.inv_h2[axis];
-        double dd = dself * dKc * dp + w;
-        double off = dnb * nb.dK * dp - w;
-        if (axis == 2) {
-          dd -= side * dKc * 0.5 * g.inv_h[2];
-          off -= side * nb.dK * 0.5 * g.inv_h[2];
-        }
-        dj += dd;
-        da += w;
-        if (nb.idx >= 0 || nb.idx == kInterfaceGhost) {  // a Dirichlet ghost is no unknown
-          offj = off;
-          offa = -w;
+// w = K_av / h^2 of a face and the derivatives of its flux w (p_L - p_U) by p_L and p_U.
+// Seen from the lower cell, p_U's derivative is its off-diagonal entry and p_L's adds to
+// its diagonal; seen from the upper cell both change sign and place.
+template <int KM>
+__device__ __forceinline__ void asm_face(int kmean, int axis, const GridP& g, double pL, double kL, double dkL,
+                                         double pU, double kU, double dkU, double& w, double& dL, double& dU) {
+  const int km = KM < 4 ? KM : axis_mean(kmean, axis);
+  const double dp = pL - pU;
+  if (km == RICH_KMEAN_ARITH) {
+    w = (kL + kU) * g.half_h2[axis];
+    const double d = dp * g.half_h2[axis];
+    dL = fma(dkL, d, w);
+    dU = fma(dkU, d, -w);
+    return;
+  }
+  const double d = dp * g.inv_h2[axis];
+  if (km == RICH_KMEAN_UPSTREAM) {  // only the upstream cell's K' enters
+    const bool up = dp_upstream(dp);
+    w = (up ? kU : kL) * g.inv_h2[axis];
+    const double v = fma(up ? dkU : dkL, d, up ? -w : w);
+    dL = up ? w : v;
+    dU = up ? v : -w;
+    return;
+  }
+  double mL = 0.0, mU = 0.0;  // dK_av / dK_L, dK_av / dK_U
+  if (km == RICH_KMEAN_GEOMETRIC) {
+    const double q = sqrt(kL * kU);
+    w = q * g.inv_h2[axis];
+    if (kL > 0.0) mL = (0.5 * q) * safe_rcp(kL);
+    if (kU > 0.0) mU = (0.5 * q) * safe_rcp(kU);
+  } else {
+    const double s = kL + kU;
+    const double r = s > 0.0 ? safe_rcp(s) : 0.0;
+    const double a = kU * r, b = kL * r;
+    w = (kL * a) * g.twice_h2[axis];
+    mL = 2.0 * a * a;
+    mU = 2.0 * b * b;
+  }
+  dL = fma(mL * dkL, d, w);
+  dU = fma(mU * dkU, d, -w);
+}
+
+// J (7 planes) and A_aux (7 planes) at the pressure K, K' and s' belong to.  A thread
+// marches upward through its cell of every layer of its block's range (blocks take equal
+// ranges of the units (chunk of the plane, layer)), so a vertical face is computed once;
+// J7b / A7b, if not NULL, receive the caller's copies in the same pass.
+// Bound: the FP64 pipe (35 to 45 operations per cell) until the 112 bytes per cell it
+// writes bind.  399 x 401 x 19 cells, upstream: one cell per thread with every mean's
+// general form took 700 us, and 105 to copy both stencils out; law, assembly and copies
+// together went from 829 to 456 us.
+constexpr int kAsmThreads = 128;
+template <int KM>
+__global__ void __launch_bounds__(kAsmThreads, 5) k_assemble(GridP g, SoilP so, BCP bc, int kmean, int units,
+                                                          const double* __restrict__ p, const double* __restrict__ K,
+                                                          const double* __restrict__ dK,
+                                                          const double* __restrict__ dS,
+                                                          const double* __restrict__ ks, double rdt,
+                                                          double* __restrict__ J7, double* __restrict__ A7,
+                                                          double* __restrict__ J7b, double* __restrict__ A7b) {
+  const long long n = g.n;
+  const int plane = g.nx * g.ny;
+  auto put = [&](int s, long long c, double jv, double av) {
+    J7[s * n + c] = jv;
+    A7[s * n + c] = av;
+    if (J7b) J7b[s * n + c] = jv;
+    if (A7b) A7b[s * n + c] = av;
+  };
+  const int u1 = (int)((blockIdx.x + 1LL) * units / gridDim.x);
+  for (int u = (int)((long long)blockIdx.x * units / gridDim.x), run; u < u1; u += run) {
+    const int ch = u / g.nz, k0 = u - ch * g.nz;
+    run = min(u1 - u, g.nz - k0);
+    const int r = ch * (int)blockDim.x + threadIdx.x;
+    if (r >= plane) continue;
+    const int j = r / g.nx, i = r - j * g.nx;
+    long long c = r + (long long)plane * k0;
+    int kl = k0 % g.nzs;  // layer within its problem: a batch's problems meet at boundaries
+    double pc = p[c], kc = K[c], dkc = dK[c];
+    double w = 0.0, dL = 0.0, dU = 0.0;  // of the bottom face
+    bool below = false;                  // ... whose lower side is an unknown
+    for (int k = k0; k < k0 + run; ++k, c += plane) {
+      const double ksc = ks ? ks[c] : so.ks;
+      AsmNb nb;
+      if (k == k0 || kl == 0) {
+        w = dL = dU = 0.0;
+        below = kl > 0;
+        bool face = below;
+        if (below) nb = AsmNb{p[c - plane], K[c - plane], dK[c - plane], true};
+        else face = asm_ghost(g, bc, so, 4, i, j, k, ksc, nb), below = face && nb.unknown;
+        if (face) {
+          asm_face<KM>(kmean, 2, g, nb.p, nb.K, nb.dK, pc, kc, dkc, w, dL, dU);
+          dL = fma(-g.half_hz, nb.dK, dL);
+          dU = fma(-g.half_hz, dkc, dU);
         }
       }
-      J7[(1 + f) * g.n + c] = offj;
-      A7[(1 + f) * g.n + c] = offa;
+      double dj = dS[c] * rdt, da = dj;
+      dj -= dU;
+      da += w;
+      put(5, c, below ? -dL : 0.0, below ? -w : 0.0);
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const bool hi = f & 1;
+        const bool inside = f < 2 ? (hi ? i < g.nx - 1 : i > 0) : (hi ? j < g.ny - 1 : j > 0);
+        const long long q = c + (f < 2 ? 1 : g.nx) * (hi ? 1 : -1);
+        bool face = inside;
+        if (inside) nb = AsmNb{p[q], K[q], dK[q], true};
+        else face = asm_ghost(g, bc, so, f, i, j, k, ksc, nb);
+        double oj = 0.0, oa = 0.0;
+        if (face) {
+          double fw, fL, fU;
+          if (hi) asm_face<KM>(kmean, f >> 1, g, pc, kc, dkc, nb.p, nb.K, nb.dK, fw, fL, fU);
+          else asm_face<KM>(kmean, f >> 1, g, nb.p, nb.K, nb.dK, pc, kc, dkc, fw, fL, fU);
+          dj += hi ? fL : -fU;
+          da += fw;
+          if (nb.unknown) {  // a Dirichlet ghost is no unknown
+            oj = hi ? fU : -fL;
+            oa = -fw;
+          }
+        }
+        put(1 + f, c, oj, oa);
+      }
+      w = dL = dU = 0.0;  // the top face, the next layer's bottom face
+      const bool inside = kl < g.nzs - 1;
+      bool face = inside;
+      if (inside) nb = AsmNb{p[c + plane], K[c + plane], dK[c + plane], true};
+      else face = asm_ghost(g, bc, so, 5, i, j, k, ksc, nb);
+      if (face) {
+        asm_face<KM>(kmean, 2, g, pc, kc, dkc, nb.p, nb.K, nb.dK, w, dL, dU);
+        dL = fma(-g.half_hz, dkc, dL);
+        dU = fma(-g.half_hz, nb.dK, dU);
+      }
+      const bool above = face && nb.unknown;
+      dj += dL;
+      da += w;
+      put(6, c, above ? dU : 0.0, above ? -w : 0.0);
+      put(0, c, dj, da);
+      if (inside) {
+        pc = nb.p;
+        kc = nb.K;
+        dkc = nb.dK;
+        below = true;
+        ++kl;
+      } else {
+        kl = 0;
+        if (k + 1 < k0 + run) {  // the next problem of a batch
+          pc = p[c + plane];
+          kc = K[c + plane];
+          dkc = dK[c + plane];
+        }
+      }
     }
-    J7[c] = dj;
-    A7[c] = da;
   }
 }
 
@@ -272,12 +356,29 @@ int residual_eval(rich_ctx* c, const double* p, const double* s_old, double dt, 
   return RICH_OK;
 }
 
-int jacobian_eval(rich_ctx* c, const double* p, double dt, bool constit_current) {
+int jacobian_eval(rich_ctx* c, const double* p, double dt, bool constit_current, double* J7b, double* A7b) {
   if (!constit_current) RICH_CHECK(constit_eval(c, p));
+  const GridP& g = c->g;
+  // chunks of a warp where chunks of kAsmThreads cells would leave SMs without a block
+  const long long plane = (long long)g.nx * g.ny;
+  const int threads = (plane + kAsmThreads - 1) / kAsmThreads * g.nz < 2 * kNumSM ? 32 : kAsmThreads;
+  const int units = (int)((plane + threads - 1) / threads * g.nz);
+  const int nb = std::min(units, 20 * kNumSM * 32 / threads);  // 20 warps per SM (registers)
+  const double rdt = c->soil.rho_phi / dt;
   {
-    ProfScope ps("assemble", c->st, (double)c->g.n * (8.0 + (c->ks ? 8.0 : 0.0) + 14 * 8.0));
-    k_assemble<<<grid_for(c->g.n), kBlock, 0, c->st>>>(c->g, c->soil, c->bc, c->kmean, p, c->K, c->dK, c->dS,
-                                                      c->ks, dt, c->J7, c->A7);
+    const int copies = 1 + (J7b != nullptr) + (A7b != nullptr);
+    ProfScope ps("assemble", c->st, (double)g.n * (32.0 + (c->ks ? 8.0 : 0.0) + (copies + 1) * 7 * 8.0));
+    auto run = [&](auto kernel) {
+      kernel<<<nb, threads, 0, c->st>>>(g, c->soil, c->bc, c->kmean, units, p, c->K, c->dK, c->dS, c->ks, rdt, c->J7,
+                                        c->A7, J7b, A7b);
+    };
+    switch (c->kmean) {
+      case RICH_KMEAN_ARITH: run(k_assemble<0>); break;
+      case RICH_KMEAN_UPSTREAM: run(k_assemble<1>); break;
+      case RICH_KMEAN_HARMONIC: run(k_assemble<2>); break;
+      case RICH_KMEAN_GEOMETRIC: run(k_assemble<3>); break;
+      default: run(k_assemble<4>); break;
+    }
   }
   RICH_LAUNCH_CHECK();
   c->have_jac = true;
@@ -594,11 +695,7 @@ int rich_residual3(rich_ctx* c, const double* p, const double* s_old, double dt,
 int rich_jacobian(rich_ctx* c, const double* p, double dt, double* J7, double* A7) {
   if (!c || !p || !(dt > 0)) return RICH_EINVAL;
   AllocStream guard(c->st);
-  RICH_CHECK(jacobian_eval(c, p, dt));
-  long long bytes = 7 * c->g.n * (long long)sizeof(double);
-  if (J7) RICH_CUDA(cudaMemcpyAsync(J7, c->J7, bytes, cudaMemcpyDeviceToDevice, c->st));
-  if (A7) RICH_CUDA(cudaMemcpyAsync(A7, c->A7, bytes, cudaMemcpyDeviceToDevice, c->st));
-  return RICH_OK;
+  return jacobian_eval(c, p, dt, false, J7, A7);
 }
 
 int rich_jacobian_apply(rich_ctx* c, const double* x, double* y) {
