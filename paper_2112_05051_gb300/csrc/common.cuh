@@ -50,9 +50,6 @@ void count_launches(long long k);  // k may be negative (launches recorded into 
 // Moves the start of the open timed launch to now (work done on the stream since
 // it opened, e.g. a one-time layout, is not charged to the launch).
 void prof_restart(cudaStream_t st);
-// Corrects the algorithmic bytes and flops of the last timed launch if it was `name`
-// (for launches whose work a device-side decision settled after they were queued).
-void prof_adjust_last(const char* name, double bytes, double flops);
 struct ProfScope {
   bool on;
   cudaStream_t st;
@@ -283,6 +280,7 @@ struct KrylovWork {
   double* z = nullptr;
   double* w = nullptr;
   double* hcoef = nullptr;  // device coefficients (m+1)
+  double* gram = nullptr;   // V^T V of FGMRES' basis (64 x 64)
   int fail_reason = 0;      // last failure: 0 none, FCG 1 maxit, 2 (p, J p) <= 0, 3 residual growth;
                             // 4 stagnation (an FCG window or an FGMRES restart cycle, krylov.stall)
 };

@@ -620,6 +620,7 @@ int rich_destroy(rich_ctx* c) {
   dfree(k.z);
   dfree(k.w);
   dfree(k.hcoef);
+  dfree(k.gram);
   pinned_put(c->hsc);
   delete c;
   return RICH_OK;

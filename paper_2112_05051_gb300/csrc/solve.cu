@@ -969,24 +969,41 @@ static int vcycle_capture(rich_ctx* c) {
   return RICH_OK;
 }
 
-// The V-cycle's kernels from r into z, launched (or captured) as they come.
-static int vcycle_direct(rich_ctx* c, const double* r, double* z) {
-  Hierarchy& H = c->H;
+// The level-0 right-hand side from r, and the result x into z.
+static int vcycle_in(rich_ctx* c, const double* r) {
+  Level& L0 = c->H.lv[0];
   const long long n = c->g.n;
   if (c->prec == RICH_PREC_MIXED) {
-    Level& L0 = H.lv[0];
     k_d2f<<<grid_for(n), kBlock, 0, c->st>>>(n, r, (float*)L0.b);
     RICH_LAUNCH_CHECK();
-    float* x = nullptr;
-    RICH_CHECK(vcycle_level<float>(c, 0, (const float*)L0.b, &x));
-    k_f2d<<<grid_for(n), kBlock, 0, c->st>>>(n, x, z);
+  } else {
+    RICH_CUDA(cudaMemcpyAsync(L0.b, r, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
+  }
+  return RICH_OK;
+}
+static int vcycle_out(rich_ctx* c, const void* x, double* z) {
+  const long long n = c->g.n;
+  if (c->prec == RICH_PREC_MIXED) {
+    k_f2d<<<grid_for(n), kBlock, 0, c->st>>>(n, (const float*)x, z);
     RICH_LAUNCH_CHECK();
   } else {
-    double* x = nullptr;
-    RICH_CHECK(vcycle_level<double>(c, 0, r, &x));
     RICH_CUDA(cudaMemcpyAsync(z, x, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
   }
   return RICH_OK;
+}
+
+// The V-cycle's kernels from the level-0 right-hand side into z, launched (or captured) as
+// they come.
+static int vcycle_direct(rich_ctx* c, double* z) {
+  Level& L0 = c->H.lv[0];
+  if (c->prec == RICH_PREC_MIXED) {
+    float* x = nullptr;
+    RICH_CHECK(vcycle_level<float>(c, 0, (const float*)L0.b, &x));
+    return vcycle_out(c, x, z);
+  }
+  double* x = nullptr;
+  RICH_CHECK(vcycle_level<double>(c, 0, (const double*)L0.b, &x));
+  return vcycle_out(c, x, z);
 }
 
 // Whether the V-cycle of this hierarchy may run from a captured graph now.
@@ -996,34 +1013,26 @@ static bool vcycle_graphable(rich_ctx* c) {
          !profiling_active();
 }
 
-int vcycle_apply(rich_ctx* c, const double* r, double* z) {
+// The V-cycle on the staged right-hand side (the level-0 buffer b) into z.
+static int vcycle_staged(rich_ctx* c, double* z) {
   Hierarchy& H = c->H;
-  if (!H.built) return RICH_ESTATE;
-  if (H.opts.precond == RICH_PRECOND_AS) return as_apply(c, r, z);
-  long long n = c->g.n;
   if (vcycle_graphable(c) && H.vc_calls > 0) {  // the first application launched directly
     if (!H.vc_exec) RICH_CHECK(vcycle_capture(c));
     if (H.vc_exec) {
-      Level& L0 = H.lv[0];
-      if (c->prec == RICH_PREC_MIXED) {
-        k_d2f<<<grid_for(n), kBlock, 0, c->st>>>(n, r, (float*)L0.b);
-        RICH_LAUNCH_CHECK();
-      } else {
-        RICH_CUDA(cudaMemcpyAsync(L0.b, r, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
-      }
       RICH_CUDA(cudaGraphLaunch(H.vc_exec, c->st));
       count_launches(H.vc_nodes);
-      if (c->prec == RICH_PREC_MIXED) {
-        k_f2d<<<grid_for(n), kBlock, 0, c->st>>>(n, (const float*)H.vc_out, z);
-        RICH_LAUNCH_CHECK();
-      } else {
-        RICH_CUDA(cudaMemcpyAsync(z, H.vc_out, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
-      }
-      return RICH_OK;
+      return vcycle_out(c, H.vc_out, z);
     }
   }
   ++H.vc_calls;
-  return vcycle_direct(c, r, z);
+  return vcycle_direct(c, z);
+}
+
+int vcycle_apply(rich_ctx* c, const double* r, double* z) {
+  if (!c->H.built) return RICH_ESTATE;
+  if (c->H.opts.precond == RICH_PRECOND_AS) return as_apply(c, r, z);
+  RICH_CHECK(vcycle_in(c, r));
+  return vcycle_staged(c, z);
 }
 
 // ---------------------------------------------------------------- Krylov kernels (FP64)
@@ -1066,70 +1075,187 @@ __global__ void k_fcg_update(long long n, double* __restrict__ x, double* __rest
   if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
 }
 
-// Batched dot products h[q] = V[q] . w: block (bx, q) reduces its share of one
-// vector; w is re-read per q from L2, V streams from HBM once.
-__global__ void k_bdot(long long n, const double* __restrict__ V, const double* __restrict__ w,
-                       double* __restrict__ partials, const int* __restrict__ run) {
-  int q = blockIdx.y;
-  if (run && !*run) {  // skipped pass: zero partials
-    if (threadIdx.x == 0) partials[(long long)q * gridDim.x + blockIdx.x] = 0.0;
-    return;
+// ---- Gram-Schmidt of FGMRES, in two passes over the basis (classical Gram-Schmidt with
+// the second projection taken from the basis' Gram matrix: Swirydowicz, Langou, Ananthan,
+// Yang, Thomas, "Low synchronization Gram-Schmidt and generalized minimal residual
+// algorithms", 2021).  With G = V^T V, whose last row is the new vector's dots, the
+// coefficients of two projections are h = h1 + (I - G) h1, h1 = V^T w, so the basis is read
+// once for the dots (with w and with the newest vector) and once for w - V h; V stays
+// orthogonal to about ten units of rounding.  Bound: the FP64 pipe, three operations per
+// basis element (explicit second projections take four and read the basis four times).
+// Where w - V h loses more than 1e-2 of w's norm, the host asks for one explicit pass more.
+// 128^3, FGMRES(30): 667 us per iteration with two explicit projections, 598 with these passes.
+constexpr int kGsThreads = 256;
+constexpr int kGsBlocks = 2 * kNumSM;  // of the dots (fixed: deterministic summation order)
+constexpr int kGsTile = 4;             // basis vectors per sweep over a block's elements
+constexpr int kGsLd = 64;              // row length of the Gram matrix
+// Device scalars of an iteration (restart <= 63): h in [0, j], ||w - V h|| and its reciprocal.
+constexpr int kSlotNorm = 63, kSlotInv = 64;
+
+// Sums of 8 values over a warp by halving: after the exchange at distances 16, 8 and 4 a
+// lane holds one value, summed on at 2 and 1: 9 additions instead of 40.  The lane's value
+// is number lane >> 2.
+__device__ __forceinline__ double warp_sum8(double (&a)[8]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 4; k > 0; k >>= 1) {
+    const bool up = lane & (4 * k);
+#pragma unroll
+    for (int q = 0; q < k; ++q) {
+      const double keep = up ? a[q + k] : a[q], send = up ? a[q] : a[q + k];
+      a[q] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * k);
+    }
   }
-  const double* v = V + (long long)q * n;
+  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+  return a[0];
+}
+
+// h1 = V^T w and the newest row of G = V^T V (nv vectors, vj = V[nv - 1]); the last block
+// to finish forms h and leaves it at s[0, nv) and in the pinned mirror.
+__global__ void __launch_bounds__(kGsThreads) k_gs_dots(long long n, int nv, const double* __restrict__ V,
+                                                        const double* __restrict__ w, double* __restrict__ part,
+                                                        double* __restrict__ gram, unsigned* __restrict__ ticket,
+                                                        double* __restrict__ s, double* __restrict__ mirror) {
+  constexpr int W = kGsThreads / 32;
+  __shared__ double sh[W][2 * kGsTile];
+  __shared__ double tot[2 * kGsLd];
+  __shared__ bool last;
+  const double* vj = V + (long long)(nv - 1) * n;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long long stride = (long long)gridDim.x * kGsThreads;
+  for (int q0 = 0; q0 < nv; q0 += kGsTile) {
+    double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    const double* v0 = V + (long long)q0 * n;
+    const int m = min(kGsTile, nv - q0);
+    long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x;
+    if (m == kGsTile) {
+      for (; i + stride < n; i += 2 * stride) {
+        const double w0 = w[i], w1 = w[i + stride], x0 = vj[i], x1 = vj[i + stride];
+        double p[kGsTile], r[kGsTile];
+#pragma unroll
+        for (int q = 0; q < kGsTile; ++q) {
+          p[q] = v0[q * n + i];
+          r[q] = v0[q * n + i + stride];
+        }
+#pragma unroll
+        for (int q = 0; q < kGsTile; ++q) {
+          a[q] = fma(p[q], w0, a[q]);
+          a[q + 4] = fma(p[q], x0, a[q + 4]);
+          a[q] = fma(r[q], w1, a[q]);
+          a[q + 4] = fma(r[q], x1, a[q + 4]);
+        }
+      }
+    }
+    for (; i < n; i += stride) {
+      const double w0 = w[i], x0 = vj[i];
+#pragma unroll
+      for (int q = 0; q < kGsTile; ++q)
+        if (q < m) {
+          const double p = v0[q * n + i];
+          a[q] = fma(p, w0, a[q]);
+          a[q + 4] = fma(p, x0, a[q + 4]);
+        }
+    }
+    const double r = warp_sum8(a);
+    if ((lane & 3) == 0) sh[wid][lane >> 2] = r;
+    __syncthreads();
+    if (threadIdx.x < 8 && (threadIdx.x & 3) < m) {
+      double t = 0.0;
+      for (int k = 0; k < W; ++k) t += sh[k][threadIdx.x];
+      const int q = (threadIdx.x >> 2) * kGsLd + q0 + (threadIdx.x & 3);
+      part[(long long)q * gridDim.x + blockIdx.x] = t;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < 8) __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int t = wid; t < 2 * nv; t += W) {
+    const int q = t < nv ? t : kGsLd + t - nv;
+    double a = 0.0;
+    for (int k = lane; k < (int)gridDim.x; k += 32) a += __ldcg(&part[(long long)q * gridDim.x + k]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if (lane == 0) tot[q] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x < nv) gram[(nv - 1) * kGsLd + threadIdx.x] = gram[threadIdx.x * kGsLd + nv - 1] = tot[kGsLd + threadIdx.x];
+  __syncthreads();
+  for (int i = wid; i < nv; i += W) {  // h_i = h1_i + sum_q (I - G)_iq h1_q
+    double d = 0.0;
+    for (int q = lane; q < nv; q += 32) d = fma((q == i ? 1.0 : 0.0) - gram[i * kGsLd + q], tot[q], d);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+    if (lane == 0) s[i] = mirror[i] = tot[i] + d;
+  }
+  if (threadIdx.x == 0) *ticket = 0;
+}
+
+// out = w - V h (w may be out) and its norm: the last block leaves ||out|| and 1/||out||
+// (0 for a zero vector) in the scalars and the norm in the mirror.
+__global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, const double* __restrict__ V,
+                                                          const double* w, double* out, double* __restrict__ part,
+                                                          unsigned* __restrict__ ticket, double* __restrict__ s,
+                                                          double* __restrict__ mirror) {
+  __shared__ double hs[kGsLd];
+  __shared__ bool last;
+  for (int q = threadIdx.x; q < nv; q += kGsThreads) hs[q] = s[q];
+  __syncthreads();
+  const long long stride = (long long)gridDim.x * kGsThreads;
   double acc[1] = {0.0};
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    acc[0] += v[i] * w[i];
-  block_sum<1>(acc);
-  if (threadIdx.x == 0) partials[(long long)q * gridDim.x + blockIdx.x] = acc[0];
-}
-
-constexpr int kBdotBlocks = 2 * kNumSM;  // x-blocks per vector (fixed: deterministic summation order)
-
-static void launch_multidot(int nb, cudaStream_t st, long long n, int nv, const double* V, const double* w,
-                            double* partials, const int* run = nullptr) {
-  (void)nb;
-  k_bdot<<<dim3(kBdotBlocks, nv), kBlock, 0, st>>>(n, V, w, partials, run);
-}
-
-// w -= sum_q h[q] V[q], in place
-__global__ void k_orth_axpy(long long n, int nv, const double* __restrict__ V, const double* __restrict__ h,
-                            double* w) {
-  __shared__ double hs[64];
-  for (int q = threadIdx.x; q < nv; q += blockDim.x) hs[q] = h[q];
-  __syncthreads();
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+  long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x;
+  for (; i + stride < n; i += 2 * stride) {
+    double t = w[i], u = w[i + stride];
+    const double* v = V + i;
+#pragma unroll 4
+    for (int q = 0; q < nv; ++q, v += n) {
+      t = fma(-hs[q], v[0], t);
+      u = fma(-hs[q], v[stride], u);
+    }
+    out[i] = t;
+    out[i + stride] = u;
+    acc[0] = fma(t, t, acc[0]);
+    acc[0] = fma(u, u, acc[0]);
+  }
+  for (; i < n; i += stride) {
     double t = w[i];
-    for (int q = 0; q < nv; ++q) t -= hs[q] * V[(long long)q * n + i];
-    w[i] = t;
+    for (int q = 0; q < nv; ++q) t = fma(-hs[q], V[(long long)q * n + i], t);
+    out[i] = t;
+    acc[0] = fma(t, t, acc[0]);
+  }
+  block_sum<1>(acc);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = acc[0];
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  acc[0] = 0.0;
+  for (int k = threadIdx.x; k < (int)gridDim.x; k += kGsThreads) acc[0] += __ldcg(&part[k]);
+  block_sum<1>(acc);
+  if (threadIdx.x == 0) {
+    const double h = sqrt(acc[0]);
+    s[kSlotNorm] = mirror[kSlotNorm] = h;
+    s[kSlotInv] = h > 0 ? 1.0 / h : 0.0;
+    *ticket = 0;
   }
 }
 
-// Device scalars of an FGMRES iteration (restart <= 63, so j <= 62): h1 in [0, j],
-// h2 in [64, 64 + j]; ||w'||^2 and the DGKS decision in the slots neither reaches
-// (both come back with the one 128-double read-back); ||w||^2, read on the device
-// only, past the read-back.
-constexpr int kSlotW1 = 63, kSlotRun = 127, kSlotW = 130;
-
-// DGKS decision on the device: run the second pass when ||w'||^2 < ||w||^2 / 2
-// (also left in s[i_out] as 1.0 / 0.0 for the host's read-back of the scalars)
-__global__ void k_dgks(double* __restrict__ s, int i_w, int i_wp, int i_out, int* __restrict__ run) {
-  const int r = s[i_wp] < 0.5 * s[i_w] ? 1 : 0;
-  *run = r;
-  s[i_out] = r;
-}
-
-// out = f * (w - sum_q h2[q] V[q]); without a second pass (run == 0) out = f * w
-__global__ void k_orth_final(long long n, int nv, const double* __restrict__ V, const double* __restrict__ h2,
-                             const double* __restrict__ w, double f, double* __restrict__ out,
-                             const int* __restrict__ run) {
-  __shared__ double hs[64];
-  if (run && !*run) nv = 0;
-  for (int q = threadIdx.x; q < nv; q += blockDim.x) hs[q] = h2[q];
-  __syncthreads();
+// V = f src (f from the device if fdev), and the V-cycle's right-hand side with it.
+template <class T>
+__global__ void k_stage(long long n, const double* src, const double* __restrict__ fdev, double f, double* V,
+                        T* __restrict__ b) {
+  if (fdev) f = *fdev;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    double t = w[i];
-    for (int q = 0; q < nv; ++q) t -= hs[q] * V[(long long)q * n + i];
-    out[i] = f * t;
+    const double v = f * src[i];
+    V[i] = v;
+    if (b) b[i] = (T)v;
   }
 }
 
@@ -1178,6 +1304,7 @@ static int ensure_krylov(rich_ctx* c, int m) {
     RICH_CHECK(dalloc(&k.hcoef, 128));
     k.n = n;
   }
+  if (m > 0 && !k.gram) RICH_CHECK(dalloc(&k.gram, kGsLd * kGsLd));
   if (m > 0 && k.m < m) {
     dfree(k.V);
     dfree(k.Z);
@@ -1198,7 +1325,12 @@ static int fcg_iteration(rich_ctx* c, double* x, double* q, const double* qprev,
   const long long n = c->g.n;
   const int g = grid_for(n), nb = red_grid(n);
   double* s = c->dsc;  // 0 rr, 1 zq, 2 pq, 3 pr, 4 pq_prev
-  RICH_CHECK(capturing ? vcycle_direct(c, k.r, k.z) : vcycle_apply(c, k.r, k.z));
+  if (capturing) {
+    RICH_CHECK(vcycle_in(c, k.r));
+    RICH_CHECK(vcycle_direct(c, k.z));
+  } else {
+    RICH_CHECK(vcycle_apply(c, k.r, k.z));
+  }
   if (first) {
     RICH_CUDA(cudaMemcpyAsync(k.p, k.z, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
   } else {
@@ -1336,13 +1468,48 @@ static int fcg(rich_ctx* c, const double* b, double* x, const rich_krylov_opts* 
   return RICH_ENOTCONV_LIN;
 }
 
-// Flexible GMRES(m) (Saad) with classical Gram-Schmidt and one re-orthogonalisation.
+// V = f src (f = *fdev if given), z = M V.
+static int fgmres_precondition(rich_ctx* c, const double* src, const double* fdev, double f, double* V, double* z) {
+  const long long n = c->g.n;
+  const int g = grid_for(n);
+  if (c->H.opts.precond == RICH_PRECOND_AS) {
+    k_stage<double><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, nullptr);
+    RICH_LAUNCH_CHECK();
+    return as_apply(c, V, z);
+  }
+  void* b = c->H.lv[0].b;
+  if (c->prec == RICH_PREC_MIXED) k_stage<float><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, (float*)b);
+  else k_stage<double><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, (double*)b);
+  RICH_LAUNCH_CHECK();
+  return vcycle_staged(c, z);
+}
+
+// One pass of the orthogonalisation: out = w - V h against nv vectors; h and ||out|| in the
+// mirror once the stream has been waited for.
+static int gs_pass(rich_ctx* c, int nv, const double* w, double* out) {
+  KrylovWork& k = c->kw;
+  const long long n = c->g.n;
+  const int g = std::min(grid_for(n), kGsBlocks), gu = std::min(grid_for(n, 2 * kBlock), 8 * kNumSM);
+  {
+    ProfScope ps("multidot", c->st, (double)n * 8.0 * (nv + 1), 4.0 * n * nv);
+    k_gs_dots<<<g, kGsThreads, 0, c->st>>>(n, nv, k.V, w, c->partials, k.gram, c->ticket, c->dsc, c->hsc);
+  }
+  RICH_LAUNCH_CHECK();
+  {
+    ProfScope ps("orth_axpy", c->st, (double)n * 8.0 * (nv + 2), 2.0 * n * (nv + 1));
+    k_gs_update<<<gu, kGsThreads, 0, c->st>>>(n, nv, k.V, w, out, c->partials, c->ticket, c->dsc, c->hsc);
+  }
+  RICH_LAUNCH_CHECK();
+  return RICH_OK;
+}
+
+// Flexible GMRES(m) (Saad) with classical Gram-Schmidt and re-orthogonalisation (gs_pass).
 static int fgmres(rich_ctx* c, const double* b, double* x, const rich_krylov_opts* o, rich_krylov_stats* st) {
   KrylovWork& k = c->kw;
+  if (!c->H.built) return RICH_ESTATE;
   long long n = c->g.n;
   int m = o->restart;
   int g = grid_for(n);
-  int nb = red_grid(n);
   double* s = c->dsc;
   RICH_CHECK(nrm2sq(c, b, n, s));
   double h0[1];
@@ -1365,65 +1532,33 @@ static int fgmres(rich_ctx* c, const double* b, double* x, const rich_krylov_opt
   const double* r0 = b;
   int its = 0;
   for (;;) {
-    k_scale<<<g, kBlock, 0, c->st>>>(n, r0, 1.0 / beta, k.V);
-    RICH_LAUNCH_CHECK();
     std::fill(gv.begin(), gv.end(), 0.0);
     gv[0] = beta;
     int jdone = 0;
     bool conv = false;
     for (int j = 0; j < m; ++j) {
       double* Vj = k.V + (long long)j * n;
+      double* Vn = Vj + n;
       double* Zj = k.Z + (long long)j * n;
-      RICH_CHECK(vcycle_apply(c, Vj, Zj));
+      // V[j] = r0 / beta, or the last pass's vector over its norm, scaled as it is staged
+      RICH_CHECK(j == 0 ? fgmres_precondition(c, r0, nullptr, 1.0 / beta, Vj, Zj)
+                        : fgmres_precondition(c, Vj, s + kSlotInv, 0.0, Vj, Zj));
       RICH_CHECK(stencil_apply(c, c->J7, Zj, k.w));
-      // Classical Gram-Schmidt with selective re-orthogonalisation (DGKS):
-      //   h1 = V^T w; w' = w - V h1; if ||w'||^2 < ||w||^2/2: h2 = V^T w' (else 0);
-      //   V[j+1] = (w' - V h2) / hn, hn^2 = ||w'||^2 - ||h2||^2 (V orthonormal).
-      // The decision stays on the device; one read-back per iteration.
-      int* run = c->iflag + 2;
-      RICH_CHECK(nrm2sq(c, k.w, n, s + kSlotW));
-      {
-        ProfScope ps("multidot", c->st, (double)n * 8.0 * (j + 2), 2.0 * n * (j + 1));
-        launch_multidot(nb, c->st, n, j + 1, k.V, k.w, c->partials);
-      }
-      RICH_LAUNCH_CHECK();
-      RICH_CHECK(finish_sums(c, c->partials, kBdotBlocks, j + 1, s));
-      {
-        // w -= V h1 (w read and written; j + 1 FMAs per cell)
-        ProfScope ps("orth_axpy", c->st, (double)n * 8.0 * (j + 3), 2.0 * n * (j + 1));
-        k_orth_axpy<<<g, kBlock, 0, c->st>>>(n, j + 1, k.V, s, k.w);
-      }
-      RICH_LAUNCH_CHECK();
-      RICH_CHECK(nrm2sq(c, k.w, n, s + kSlotW1));
-      k_dgks<<<1, 1, 0, c->st>>>(s, kSlotW, kSlotW1, kSlotRun, run);
-      RICH_LAUNCH_CHECK();
-      {
-        ProfScope ps("multidot", c->st, (double)n * 8.0 * (j + 2), 2.0 * n * (j + 1));
-        launch_multidot(nb, c->st, n, j + 1, k.V, k.w, c->partials, run);
-      }
-      RICH_LAUNCH_CHECK();
-      RICH_CHECK(finish_sums(c, c->partials, kBdotBlocks, j + 1, s + 64));
-      RICH_CUDA(cudaMemcpyAsync(c->hsc, s, 128 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
+      RICH_CHECK(gs_pass(c, j + 1, k.w, Vn));
       RICH_CUDA(cudaStreamSynchronize(c->st));
-      const bool second = c->hsc[kSlotRun] != 0.0;
-      if (!second) prof_adjust_last("multidot", 0.0, 0.0);  // the skipped pass only zeroed its partials
-      double h2sq = 0.0;
+      double hn = c->hsc[kSlotNorm], hsq = 0.0;
       for (int i = 0; i <= j; ++i) {
-        Hij(i, j) = c->hsc[i] + c->hsc[64 + i];
-        h2sq += c->hsc[64 + i] * c->hsc[64 + i];
+        Hij(i, j) = c->hsc[i];
+        hsq += Hij(i, j) * Hij(i, j);
       }
-      double wsq = c->hsc[kSlotW1] - h2sq;
-      double hn = wsq > 0 ? sqrt(wsq) : 0.0;
+      if (hn * hn < 1e-4 * hsq && hn > 0) {  // cancellation: an explicit projection of what is left
+        RICH_CHECK(gs_pass(c, j + 1, Vn, Vn));
+        RICH_CUDA(cudaStreamSynchronize(c->st));
+        hn = c->hsc[kSlotNorm];
+        for (int i = 0; i <= j; ++i) Hij(i, j) += c->hsc[i];
+      }
       if (!std::isfinite(hn)) return RICH_ENONFINITE;
       Hij(j + 1, j) = hn;
-      {
-        // with the second pass: w' - V h2, scaled (j + 3 vectors); without: w' scaled (2 vectors)
-        ProfScope ps("orth_final", c->st, second ? (double)n * 8.0 * (j + 3) : 16.0 * n,
-                     second ? 2.0 * n * (j + 1) + n : (double)n);
-        k_orth_final<<<g, kBlock, 0, c->st>>>(n, j + 1, k.V, s + 64, k.w, hn > 0 ? 1.0 / hn : 0.0,
-                                             k.V + (long long)(j + 1) * n, run);
-      }
-      RICH_LAUNCH_CHECK();
       for (int i = 0; i < j; ++i) {
         double t = cs[i] * Hij(i, j) + sn[i] * Hij(i + 1, j);
         Hij(i + 1, j) = -sn[i] * Hij(i, j) + cs[i] * Hij(i + 1, j);
