@@ -462,7 +462,7 @@ int rich_measure_fma_peak(int fp64, double* tflops);
 
 /* The autotuner's choices so far, one line "mode value_bytes rows_bin mean_row_length
  * sell_offered variant best_us best_csr_variant" each (mode 0 y = A x, 1 y += A x,
- * 2 l1-Jacobi sweep, 3 residual; rows_bin = floor(4 log2 rows); sell_offered 1 where a
+ * 2 l1-Jacobi sweep, 3 residual, 4 y = b + d .* (A x); rows_bin = floor(4 log2 rows); sell_offered 1 where a
  * SELL copy was a candidate; variant = lanes per row, + 256 for four-way unrolled rows,
  * 512 / 513 for the SELL copy with 4 / 8 gathers in flight per row, 514 for the SELL
  * copy with two lanes per row, 515 for the software-pipelined one; best_csr_variant

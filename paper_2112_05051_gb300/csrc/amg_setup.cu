@@ -1463,9 +1463,84 @@ __global__ void k_stencil4(long long n, const double* __restrict__ A7, Stencil4<
   }
 }
 
+// s = l1^-1/2 and q = l1^1/2 of every row, kept in FP64 for k_scaled: the hardware's
+// approximation (2^-20) and one cubically convergent step y (1 + e/2 + 3/8 e^2),
+// e = 1 - l1 y^2; a norm near the ends of the exponent range takes sqrt() and a division.
+__global__ void k_scale_rows(long long n, const double* __restrict__ A7, double* __restrict__ s, double* __restrict__ q,
+                             float* __restrict__ s32, float* __restrict__ q32) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    double l1 = A7[i];
+#pragma unroll
+    for (int f = 1; f < 7; ++f) l1 -= A7[f * n + i];
+    double r;
+    const unsigned e = ((unsigned)__double2hiint(l1) >> 20) & 0x7ffu;
+    if (__double2hiint(l1) >= 0 && e - 123u < 1800u) {
+      double y;
+      asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(l1));
+      const double d = fma(-l1 * y, y, 1.0);
+      r = fma(y * d, fma(0.375, d, 0.5), y);
+    } else {
+      r = 1.0 / sqrt(l1);
+    }
+    s[i] = r;
+    const double p = l1 * r;
+    if (q) q[i] = p;
+    if (s32) {
+      s32[i] = (float)r;
+      q32[i] = (float)p;
+    }
+  }
+}
+
+template <class T>
+__global__ void k_scaled(GridP gr, const double* __restrict__ A7, const double* __restrict__ s, ScaledSt<T> A) {
+  const int i = blockIdx.y * kLineThreads + threadIdx.x;
+  if (i >= gr.nx) return;
+  const long long n = gr.n, c = (long long)blockIdx.x * gr.nx + i;
+  const int j = blockIdx.x % gr.ny, k = blockIdx.x / gr.ny, sxy = gr.nx * gr.ny;
+  const double sc = s[c];
+  const double d = -A7[c] * sc * sc;
+  A.g[c] = (T)(1.0 + d);
+  A.gd[c] = (T)d;
+  A.wx[c] = i < gr.nx - 1 ? (T)(-A7[2 * n + c] * sc * s[c + 1]) : T(0);
+  A.wy[c] = j < gr.ny - 1 ? (T)(-A7[4 * n + c] * sc * s[c + gr.nx]) : T(0);
+  A.wz[c] = k < gr.nz - 1 ? (T)(-A7[6 * n + c] * sc * s[c + sxy]) : T(0);
+}
+
+template <class T>
+static int scaled_alloc(ScaledSt<T>& A, long long n) {
+  if (A.g) return RICH_OK;
+  for (T** p : {&A.g, &A.gd, &A.wx, &A.wy, &A.wz, &A.s, &A.q}) RICH_CHECK(dalloc(p, n));
+  return RICH_OK;
+}
+template <class T>
+static void scaled_free(ScaledSt<T>& A) {
+  for (T** p : {&A.g, &A.gd, &A.wx, &A.wy, &A.wz, &A.s, &A.q}) dfree(*p);
+}
+
+static int fine_scaled(rich_ctx* c) {
+  Hierarchy& H = c->H;
+  const long long n = c->g.n;
+  if (c->prec == RICH_PREC_MIXED) {
+    RICH_CHECK(scaled_alloc(H.sc32, n));
+    if (!H.sc64.s) RICH_CHECK(dalloc(&H.sc64.s, n));  // FP64 factors for the weights' products
+    k_scale_rows<<<grid_for(n), kBlock, 0, c->st>>>(n, c->A7, H.sc64.s, nullptr, H.sc32.s, H.sc32.q);
+    RICH_LAUNCH_CHECK();
+    k_scaled<float><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, c->A7, H.sc64.s, H.sc32);
+  } else {
+    RICH_CHECK(scaled_alloc(H.sc64, n));
+    k_scale_rows<<<grid_for(n), kBlock, 0, c->st>>>(n, c->A7, H.sc64.s, H.sc64.q, nullptr, nullptr);
+    RICH_LAUNCH_CHECK();
+    k_scaled<double><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, c->A7, H.sc64.s, H.sc64);
+  }
+  RICH_LAUNCH_CHECK();
+  return RICH_OK;
+}
+
 // Finest-level stencil copy of the diffusion matrix for the V-cycle (FP64 or FP32).
 static int fine_stencil(rich_ctx* c) {
   Hierarchy& H = c->H;
+  if (H.scaled) return fine_scaled(c);
   long long n = c->g.n;
   bool mp = c->prec == RICH_PREC_MIXED;
   if (mp && !H.st32.diag) {
@@ -1556,6 +1631,9 @@ void amg_free(rich_ctx* c) {
   H.nlev = 0;
   dfree(H.st64.diag); dfree(H.st64.wx); dfree(H.st64.wy); dfree(H.st64.wz); dfree(H.st64.dinv);
   dfree(H.st32.diag); dfree(H.st32.wx); dfree(H.st32.wy); dfree(H.st32.wz); dfree(H.st32.dinv);
+  scaled_free(H.sc64);
+  scaled_free(H.sc32);
+  H.scaled = false;
   dfree(H.cdense);
   dfree(H.cinv32);
   dfree(H.cwork);
@@ -1899,6 +1977,7 @@ int amg_build(rich_ctx* c, const rich_amg_opts* o) {
   H.cn = H.lv[H.nlev - 1].n;
   // coarsening stalled above the dense limit: the coarsest level is smoothed
   H.dense = H.cn <= kMaxCoarseDense;
+  H.scaled = H.nlev > 1 && H.opts.smoother == RICH_SMOOTH_L1JACOBI;
   for (int l = 0; l < H.nlev; ++l) {
     RICH_CHECK(level_alloc_vectors(c, H.lv[l]));
     RICH_CHECK(level_diag_data(c, H.lv[l]));

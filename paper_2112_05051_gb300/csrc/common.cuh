@@ -221,6 +221,22 @@ struct Stencil4 {
   T* dinv = nullptr;  // 1 / (diag + sum of the six face weights), the l1-Jacobi scaling
 };
 
+// Finest level of the l1-Jacobi V-cycle, scaled symmetrically: with s = l1^-1/2 per cell
+// (l1 the row's l1 norm) and A' = s A s, x = s y and b' = s b, the sweep
+// x <- x + l1^-1 (b - A x) is y <- b' + (I - A') y: one multiply-add per entry and no
+// other FP64 operation, and the first sweep from zero is y = b' itself.  g is the diagonal
+// of I - A' and gd that of -A', wx wy wz the face weights scaled from both sides, q = 1 / s.
+template <class T>
+struct ScaledSt {
+  T* g = nullptr;
+  T* gd = nullptr;
+  T* wx = nullptr;
+  T* wy = nullptr;
+  T* wz = nullptr;
+  T* s = nullptr;
+  T* q = nullptr;
+};
+
 // Launch shape of the structured-grid kernels: one block row per (j, k) grid line,
 // blockIdx.y tiles the x direction; no 64-bit division per thread.
 constexpr int kLineThreads = 128;
@@ -231,6 +247,9 @@ inline dim3 line_grid(const GridP& g) {
 struct Hierarchy {
   Stencil4<double> st64;
   Stencil4<float> st32;
+  ScaledSt<double> sc64;
+  ScaledSt<float> sc32;
+  bool scaled = false;            // the finest level runs on sc64 / sc32 (l1-Jacobi, more than one level)
   std::vector<Level> lv;
   int nlev = 0;
   int cn = 0;                     // coarsest size

@@ -1,10 +1,11 @@
 // SELL-C-sigma copies of the coarse-level CSR matrices (the layout is described
-// with struct Sell).  The pattern is laid out once per hierarchy: the row pointer
-// comes to the host, rows are counting-sorted by decreasing length within each
-// window of kSellSigma rows (ties keep their order, so the layout is a function of
-// the pattern alone), and one kernel scatters the column indices into the slots.
+// with struct Sell).  The pattern is laid out on the device, once per hierarchy: a block
+// per window of kSellSigma rows ranks its rows by decreasing length (ties keep their
+// order, so the layout is a function of the pattern alone), a scan of the slice widths
+// gives the slot offsets, and one kernel scatters the column indices into the slots; the
+// host only learns the number of slots (a host-side sort of 2.1M rows took 5 ms).
 // Values are gathered into the slots by a second kernel, again after every
-// Galerkin refresh of the matrix.
+// Galerkin refresh of the matrix.  sell_layout is the same layout on the host.
 #include <vector>
 
 #include "common.cuh"
@@ -37,6 +38,10 @@ __global__ void k_sell_vals(int nslice, const int* __restrict__ sptr, const int*
   }
 }
 
+__global__ void k_ll_to_int(int n, const long long* __restrict__ a, int* __restrict__ b) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) b[i] = (int)a[i];
+}
+
 // The layout of a SELL copy from the row pointer alone (host): perm (32 ns entries,
 // -1 past n) and sptr (ns + 1 slot offsets).  Returns the slot count, or -1 when it
 // exceeds 32-bit offsets.
@@ -64,31 +69,61 @@ long long sell_layout(const int* rp, int n, int* perm, int* sptr) {
   return slots;
 }
 
+// One window per block: rows ranked by a counting comparison over the window's lengths;
+// the first row of each slice is its longest.
+__global__ void __launch_bounds__(kSellSigma) k_sell_rank(int n, const int* __restrict__ rp, int nslice,
+                                                          int* __restrict__ perm, int* __restrict__ slots) {
+  __shared__ int len[kSellSigma];
+  const int t = threadIdx.x, w0 = blockIdx.x * kSellSigma, row = w0 + t;
+  const int l = row < n ? rp[row + 1] - rp[row] : -1;
+  len[t] = l;
+  __syncthreads();
+  int rank = 0;
+#pragma unroll 8
+  for (int u = 0; u < kSellSigma; ++u) rank += len[u] > l || (len[u] == l && u < t);
+  const int at = w0 + rank;
+  if (at < nslice * kSellC) {
+    perm[at] = row < n ? row : -1;
+    if ((at & (kSellC - 1)) == 0) slots[at / kSellC] = kSellC * (l > 0 ? l : 0);
+  }
+}
+
 int sell_build(rich_ctx* c, const Csr<double>& M, Sell& S) {
   sell_free(S);
   const int n = M.nrows;
   if (n < kSellMinRows) return RICH_OK;
-  std::vector<int> rp(n + 1);
-  RICH_CUDA(cudaMemcpyAsync(rp.data(), M.rowptr, sizeof(int) * (n + 1), cudaMemcpyDeviceToHost, c->st));
-  RICH_CUDA(cudaStreamSynchronize(c->st));
   const int ns = (n + kSellC - 1) / kSellC;
-  std::vector<int> perm((size_t)ns * kSellC), sptr(ns + 1);
-  const long long slots = sell_layout(rp.data(), n, perm.data(), sptr.data());
-  if (slots < 0) return RICH_OK;  // too large for 32-bit slot offsets: CSR only
+  int* slots = nullptr;
+  long long* off = nullptr;
+  RICH_CHECK(dalloc(&slots, ns));
+  RICH_CHECK(dalloc(&off, ns + 1LL));
   RICH_CHECK(dalloc(&S.sptr, ns + 1));
   RICH_CHECK(dalloc(&S.perm, (long long)ns * kSellC));
-  RICH_CHECK(dalloc(&S.col, slots));
-  if (c->prec == RICH_PREC_MIXED) RICH_CHECK(dalloc(&S.val32, slots));
-  else RICH_CHECK(dalloc(&S.val, slots));
+  k_sell_rank<<<(n + kSellSigma - 1) / kSellSigma, kSellSigma, 0, c->st>>>(n, M.rowptr, ns, S.perm, slots);
+  RICH_LAUNCH_CHECK();
+  // 64-bit offsets first: the slots of a matrix with very uneven rows can pass 32 bits
+  RICH_CHECK(scan_exclusive_int_ll(c, slots, off, ns));
+  long long total = 0;
+  RICH_CUDA(cudaMemcpyAsync(&total, off + ns, sizeof(total), cudaMemcpyDeviceToHost, c->st));
+  RICH_CUDA(cudaStreamSynchronize(c->st));
+  if (total > 2147483647LL) {  // too large for 32-bit slot offsets: CSR only
+    dfree(slots);
+    dfree(off);
+    sell_free(S);
+    return RICH_OK;
+  }
+  k_ll_to_int<<<grid_for(ns + 1), kBlock, 0, c->st>>>(ns + 1, off, S.sptr);
+  RICH_LAUNCH_CHECK();
+  dfree(slots);
+  dfree(off);
+  RICH_CHECK(dalloc(&S.col, total));
+  if (c->prec == RICH_PREC_MIXED) RICH_CHECK(dalloc(&S.val32, total));
+  else RICH_CHECK(dalloc(&S.val, total));
   S.nrows = n;
   S.nslice = ns;
-  S.slots = slots;
-  RICH_CUDA(cudaMemcpyAsync(S.sptr, sptr.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice, c->st));
-  RICH_CUDA(cudaMemcpyAsync(S.perm, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice, c->st));
+  S.slots = total;
   k_sell_cols<<<grid_for((long long)ns * kSellC), kBlock, 0, c->st>>>(ns, S.sptr, S.perm, M.rowptr, M.col, S.col);
   RICH_LAUNCH_CHECK();
-  // the host vectors are read by the copies above before they go out of scope
-  RICH_CUDA(cudaStreamSynchronize(c->st));
   return RICH_OK;
 }
 

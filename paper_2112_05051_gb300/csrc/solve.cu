@@ -27,42 +27,13 @@ __global__ void k_jacobi0(int n, const T* __restrict__ dinv, const T* __restrict
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] = dinv[i] * b[i];
 }
 
-template <class T>
-__global__ void k_jacobi(int n, const int* __restrict__ rp, const int* __restrict__ col, const T* __restrict__ val,
-                         const T* __restrict__ dinv, const T* __restrict__ b, const T* __restrict__ x,
-                         T* __restrict__ xo) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    T s = b[i];
-    for (int e = rp[i]; e < rp[i + 1]; ++e) s -= val[e] * x[col[e]];
-    xo[i] = x[i] + dinv[i] * s;
-  }
-}
-
-template <class T>
-__global__ void k_resid(int n, const int* __restrict__ rp, const int* __restrict__ col, const T* __restrict__ val,
-                        const T* __restrict__ b, const T* __restrict__ x, T* __restrict__ r) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    T s = b[i];
-    for (int e = rp[i]; e < rp[i + 1]; ++e) s -= val[e] * x[col[e]];
-    r[i] = s;
-  }
-}
-
-template <class T>
-__global__ void k_spmv(int n, const int* __restrict__ rp, const int* __restrict__ col, const T* __restrict__ val,
-                       const T* __restrict__ x, T* __restrict__ y, int add) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    T s = add ? y[i] : T(0);
-    for (int e = rp[i]; e < rp[i + 1]; ++e) s += val[e] * x[col[e]];
-    y[i] = s;
-  }
-}
-
 // CSR row operation with G lanes per row (G = 4..32), for levels whose rows are
 // long (coarse Galerkin operators carry tens to hundreds of entries per row).
-// MODE 0: y = A x; 1: y += A x; 2: y = x + dinv (b - A x); 3: y = b - A x.
-// U = 4: each lane keeps four partial sums over entries e, e+G, e+2G, e+3G, so four
-// independent gathers of x are in flight (the coarse levels are gather-latency bound).
+// MODE 0: y = A x; 1: y += A x; 2: y = x + dinv (b - A x); 3: y = b - A x; 4: y = b + dinv (A x).
+// U = 4: a lane takes entries e, e+G, e+2G, e+3G at a time, absent ones predicated off, so
+// that a batch costs one round of loads (columns and values, then the gathers) whatever
+// the row's length, and the row's own operands are in flight meanwhile; the coarse levels
+// are bound by that latency (8876 rows of 101 entries, FP64: 9.1 us in rounds of one).
 template <class T, int MODE, int G, int U = 1>
 __global__ void k_csr_grp(int n, const int* __restrict__ rp, const int* __restrict__ col, const T* __restrict__ val,
                           const T* __restrict__ dinv, const T* __restrict__ b, const T* __restrict__ x,
@@ -74,26 +45,43 @@ __global__ void k_csr_grp(int n, const int* __restrict__ rp, const int* __restri
     T s = 0;
     int e = rp[row] + lane;
     const int end = rp[row + 1];
-    if (U == 4) {
-      T s1 = 0, s2 = 0, s3 = 0;
-      for (; e + 3 * G < end; e += 4 * G) {
-        const int c0 = col[e], c1 = col[e + G], c2 = col[e + 2 * G], c3 = col[e + 3 * G];
-        const T v0 = val[e], v1 = val[e + G], v2 = val[e + 2 * G], v3 = val[e + 3 * G];
-        s += v0 * x[c0];
-        s1 += v1 * x[c1];
-        s2 += v2 * x[c2];
-        s3 += v3 * x[c3];
-      }
-      s = (s + s1) + (s2 + s3);
+    T bi = 0, xi = 0, di = 0;  // the row's own operands
+    if (lane == 0) {
+      if (MODE >= 2) bi = b[row];
+      if (MODE == 2) xi = x[row];
+      if (MODE == 1) xi = y[row];
+      if (MODE == 2 || MODE == 4) di = dinv[row];
     }
-    for (; e < end; e += G) s += val[e] * x[col[e]];
+    if (U == 4) {
+      T s1 = 0;
+      for (; e < end; e += 4 * G) {
+        int c[4];
+        T v[4], xx[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const bool in = e + u * G < end;
+          c[u] = in ? col[e + u * G] : -1;
+          v[u] = in ? val[e + u * G] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) xx[u] = c[u] >= 0 ? x[c[u]] : T(0);
+        s += v[0] * xx[0];
+        s1 += v[1] * xx[1];
+        s += v[2] * xx[2];
+        s1 += v[3] * xx[3];
+      }
+      s += s1;
+    } else {
+      for (; e < end; e += G) s += val[e] * x[col[e]];
+    }
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) s += __shfl_down_sync(mask, s, o, G);
     if (lane == 0) {
       if (MODE == 0) y[row] = s;
-      else if (MODE == 1) y[row] += s;
-      else if (MODE == 2) y[row] = x[row] + dinv[row] * (b[row] - s);
-      else y[row] = b[row] - s;
+      else if (MODE == 1) y[row] = xi + s;
+      else if (MODE == 2) y[row] = xi + di * (bi - s);
+      else if (MODE == 3) y[row] = bi - s;
+      else y[row] = bi + di * s;
     }
   }
 }
@@ -104,7 +92,7 @@ __global__ void k_csr_grp(int n, const int* __restrict__ rp, const int* __restri
 // shuffle-add reductions and the idle lanes of ragged rows cost as much as the
 // products themselves).  Past a row's end the slots hold zeros.
 template <class T, int MODE, int U>
-__global__ void __launch_bounds__(kBlock) k_sell(int nslice, const int* __restrict__ sptr,
+__global__ void __launch_bounds__(U == 4 ? kSellSigma : kBlock) k_sell(int nslice, const int* __restrict__ sptr,
                                                  const int* __restrict__ perm, const int* __restrict__ col,
                                                  const T* __restrict__ val, const T* __restrict__ dinv,
                                                  const T* __restrict__ b, const T* __restrict__ x,
@@ -131,13 +119,32 @@ __global__ void __launch_bounds__(kBlock) k_sell(int nslice, const int* __restri
         s1 += vv[u + 1] * xx[u + 1];
       }
     }
-    for (; e < end; e += kSellC) s0 += val[e] * x[col[e]];
+    if (U == 8) {  // (the batched form below takes 64 registers here and costs 2 us of 21)
+      for (; e < end; e += kSellC) s0 += val[e] * x[col[e]];
+    } else {  // the last columns, one round of loads for all of them (warp-uniform tests)
+      const int rem = (end - e + lane) / kSellC;
+      int cc[U - 1];
+      T vv[U - 1], xx[U - 1];
+#pragma unroll
+      for (int u = 0; u < U - 1; ++u)
+        if (u < rem) {
+          cc[u] = col[e + u * kSellC];
+          vv[u] = val[e + u * kSellC];
+        }
+#pragma unroll
+      for (int u = 0; u < U - 1; ++u)
+        if (u < rem) xx[u] = x[cc[u]];
+#pragma unroll
+      for (int u = 0; u < U - 1; ++u)
+        if (u < rem) s0 += vv[u] * xx[u];
+    }
     const T a = s0 + s1;
     if (row >= 0) {
       if (MODE == 0) y[row] = a;
       else if (MODE == 1) y[row] += a;
       else if (MODE == 2) y[row] = x[row] + dinv[row] * (b[row] - a);
-      else y[row] = b[row] - a;
+      else if (MODE == 3) y[row] = b[row] - a;
+      else y[row] = b[row] + dinv[row] * a;
     }
   }
 }
@@ -209,7 +216,8 @@ __global__ void __launch_bounds__(kBlock) k_sellp(int nslice, const int* __restr
       if (MODE == 0) y[row] = a;
       else if (MODE == 1) y[row] += a;
       else if (MODE == 2) y[row] = x[row] + dinv[row] * (b[row] - a);
-      else y[row] = b[row] - a;
+      else if (MODE == 3) y[row] = b[row] - a;
+      else y[row] = b[row] + dinv[row] * a;
     }
   }
 }
@@ -251,7 +259,8 @@ __global__ void __launch_bounds__(kBlock) k_sell2(int nslice, const int* __restr
       if (MODE == 0) y[row] = a;
       else if (MODE == 1) y[row] += a;
       else if (MODE == 2) y[row] = x[row] + dinv[row] * (b[row] - a);
-      else y[row] = b[row] - a;
+      else if (MODE == 3) y[row] = b[row] - a;
+      else y[row] = b[row] + dinv[row] * a;
     }
   }
 }
@@ -271,6 +280,8 @@ static void csr_launch(cudaStream_t st, int v, int n, const int* rp, const int* 
                        const T* b, const T* x, T* y, const Sell* sl = nullptr, const T* sval = nullptr) {
   if (is_sell(v)) {
     const int g = grid_for((long long)sl->nslice * kSellC);
+    // a block per window of the sort: its vectors' accesses, in sorted order, share L1 lines
+    const int gw = grid_for((long long)sl->nslice * kSellC, kSellSigma);
     if (v == kSellVariant8)
       k_sell<T, MODE, 8><<<g, kBlock, 0, st>>>(sl->nslice, sl->sptr, sl->perm, sl->col, sval, dinv, b, x, y);
     else if (v == kSellVariant2)
@@ -279,7 +290,7 @@ static void csr_launch(cudaStream_t st, int v, int n, const int* rp, const int* 
     else if (v == kSellVariantP)
       k_sellp<T, MODE><<<g, kBlock, 0, st>>>(sl->nslice, sl->sptr, sl->perm, sl->col, sval, dinv, b, x, y);
     else
-      k_sell<T, MODE, 4><<<g, kBlock, 0, st>>>(sl->nslice, sl->sptr, sl->perm, sl->col, sval, dinv, b, x, y);
+      k_sell<T, MODE, 4><<<gw, kSellSigma, 0, st>>>(sl->nslice, sl->sptr, sl->perm, sl->col, sval, dinv, b, x, y);
     return;
   }
   const int G = v & 0xff;
@@ -290,7 +301,9 @@ static void csr_launch(cudaStream_t st, int v, int n, const int* rp, const int* 
       case 1: k_csr_grp<T, MODE, 1, 4><<<gr, kBlock, 0, st>>>(n, rp, col, val, dinv, b, x, y); break;
       case 2: k_csr_grp<T, MODE, 2, 4><<<gr, kBlock, 0, st>>>(n, rp, col, val, dinv, b, x, y); break;
       case 4: k_csr_grp<T, MODE, 4, 4><<<gr, kBlock, 0, st>>>(n, rp, col, val, dinv, b, x, y); break;
-      default: k_csr_grp<T, MODE, 8, 4><<<gr, kBlock, 0, st>>>(n, rp, col, val, dinv, b, x, y); break;
+      case 8: k_csr_grp<T, MODE, 8, 4><<<gr, kBlock, 0, st>>>(n, rp, col, val, dinv, b, x, y); break;
+      case 16: k_csr_grp<T, MODE, 16, 4><<<gr, kBlock, 0, st>>>(n, rp, col, val, dinv, b, x, y); break;
+      default: k_csr_grp<T, MODE, 32, 4><<<gr, kBlock, 0, st>>>(n, rp, col, val, dinv, b, x, y); break;
     }
     return;
   }
@@ -409,7 +422,8 @@ static int csr_op(rich_ctx* c, int n, long long nnz, const int* rp, const int* c
       int best_csr = v;
       const Sell* sl = sell_ok ? src->s : nullptr;
       const T* sval = sell_ok ? (sizeof(T) == 8 ? (const T*)sl->val : (const T*)sl->val32) : nullptr;
-      for (int g : {1, 2, 4, 8, 16, 32, 1 | kUnroll, 2 | kUnroll, 4 | kUnroll, 8 | kUnroll, kSellVariant,
+      for (int g : {1, 2, 4, 8, 16, 32, 1 | kUnroll, 2 | kUnroll, 4 | kUnroll, 8 | kUnroll, 16 | kUnroll,
+                    32 | kUnroll, kSellVariant,
                     kSellVariant8, kSellVariant2, kSellVariantP}) {
         if (is_sell(g) && !sell_ok) continue;
         csr_launch<T, MODE>(c->st, g, n, rp, col, val, dinv, b, x, scratch, sl, sval);
@@ -470,8 +484,7 @@ int autotune_load(const char* text) {
     if (v == kSellVariant || v == kSellVariant8 || v == kSellVariant2 || v == kSellVariantP) return true;
     const int g = v & 0xff, u = v & ~0xff;
     if (u != 0 && u != kUnroll) return false;
-    if (g != 1 && g != 2 && g != 4 && g != 8 && g != 16 && g != 32) return false;
-    return u == 0 || g <= 8;
+    return g == 1 || g == 2 || g == 4 || g == 8 || g == 16 || g == 32;
   };
   std::vector<std::pair<TuneKey, TuneVal>> rows;
   const char* p = text;
@@ -482,7 +495,7 @@ int autotune_load(const char* text) {
     if (sscanf(p, "%d %d %d %lld %d %d %f %d%n", &mode, &tsize, &n, &nnz, &sell, &variant, &us, &best_csr, &used) !=
         8)
       return RICH_EINVAL;
-    if (mode < 0 || mode > 3 || (tsize != 4 && tsize != 8) || (sell != 0 && sell != 1) || !valid(variant) ||
+    if (mode < 0 || mode > 4 || (tsize != 4 && tsize != 8) || (sell != 0 && sell != 1) || !valid(variant) ||
         !valid(best_csr) || best_csr >= kSellVariant || (!sell && variant >= kSellVariant))
       return RICH_EINVAL;
     rows.push_back({TuneKey{mode, tsize, n, nnz, sell}, TuneVal{variant, us, best_csr}});
@@ -494,13 +507,29 @@ int autotune_load(const char* text) {
   return RICH_OK;
 }
 
-// x = M b for a dense row-major n x n matrix; one warp per row.
+// x = M b for a dense row-major n x n matrix; one warp per row, 8 loads of either in
+// flight per lane (n = 362 in FP64: 10 us with one at a time).
 template <class T>
 __global__ void k_gemv(int n, const T* __restrict__ M, const T* __restrict__ b, T* __restrict__ x) {
   int lane = threadIdx.x & 31;
   for (int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < n; row += (gridDim.x * blockDim.x) >> 5) {
-    T s = 0;
-    for (int j = lane; j < n; j += 32) s += M[(long long)row * n + j] * b[j];
+    const T* m = M + (long long)row * n;
+    T s = 0, s1 = 0;
+    for (int j = lane; j < n; j += 256) {
+      T a[8], v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const bool in = j + 32 * u < n;
+        a[u] = in ? m[j + 32 * u] : T(0);
+        v[u] = in ? b[j + 32 * u] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        s += a[u] * v[u];
+        s1 += a[u + 1] * v[u + 1];
+      }
+    }
+    s += s1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) x[row] = s;
@@ -516,12 +545,9 @@ __global__ void k_f2d(long long n, const float* __restrict__ a, double* __restri
     b[i] = (double)a[i];
 }
 
-// Finest-level l1-Jacobi sweep and residual on the stencil form.  The l1 row norm
-// is diag + sum of the six face weights (all couplings are -w with w >= 0).
-// mode 1: xo = x + D_l1^-1 (b - A x); 2: xo = b - A x (residual).  The first
-// sweep from x = 0 (x = D_l1^-1 b) is the elementwise k_jacobi0.
-template <class T, int MODE>
-__global__ void __launch_bounds__(kLineThreads) k_st_smooth(GridP g, Stencil4<T> A, const T* __restrict__ b,
+// Finest-level residual xo = b - A x on the stencil form (hybrid Gauss-Seidel's).
+template <class T>
+__global__ void __launch_bounds__(kLineThreads) k_st_resid(GridP g, Stencil4<T> A, const T* __restrict__ b,
                                                             const T* __restrict__ x, T* __restrict__ xo) {
   int i = blockIdx.y * kLineThreads + threadIdx.x;
   if (i >= g.nx) return;
@@ -540,41 +566,75 @@ __global__ void __launch_bounds__(kLineThreads) k_st_smooth(GridP g, Stencil4<T>
   if (j < g.ny - 1) ax -= wyp * x[c + nx];
   if (k > 0) ax -= A.wz[c - sxy] * x[c - sxy];
   if (k < g.nz - 1) ax -= wzp * x[c + sxy];
-  if (MODE == 2) xo[c] = b[c] - ax;
-  else xo[c] = xc + A.dinv[c] * (b[c] - ax);
+  xo[c] = b[c] - ax;
 }
 
-// The first l1-Jacobi sweep from zero, y = D_l1^-1 b, folded into the next stencil
-// pass on the finest level: y is recomputed from b and the l1 scaling wherever the
-// next pass reads it (own cell and the six neighbours, all cache hits), so it is
-// never written and read back.  MODE 1: out = y + D_l1^-1 (b - A y), the second
-// sweep; MODE 2: x1 = y and out = b - A y, the residual after a single sweep.
+// Sweep (MODE 1: out = b' + (I - A') y) and residual (MODE 2: out = q (b' - A' y), the
+// unscaled residual, with A's own diagonal -gd) of the scaled finest level (ScaledSt).  A thread marches zc layers with
+// its column's y and vertical weight in registers.
+// Bound: FP64, one multiply-add per entry; FP32, HBM (28 bytes per cell: g, 3 weights, b, y
+// in, y out).  128^3 FP64: the unscaled sweep, 9 operations and 64 bytes, took 36 us, and
+// the first sweep from zero, a pass of its own (9 us), is gone.
 template <class T, int MODE>
-__global__ void __launch_bounds__(kLineThreads) k_st_first(GridP g, Stencil4<T> A, const T* __restrict__ b,
-                                                           T* __restrict__ x1, T* __restrict__ out) {
-  int i = blockIdx.y * kLineThreads + threadIdx.x;
+__global__ void __launch_bounds__(kLineThreads) k_sc(GridP g, ScaledSt<T> A, int zc, const T* __restrict__ b,
+                                                     const T* __restrict__ y, T* __restrict__ out) {
+  const int i = blockIdx.y * blockDim.x + threadIdx.x;
   if (i >= g.nx) return;
-  int r = blockIdx.x;
-  int j = r % g.ny;
-  int k = r / g.ny;
-  int nx = g.nx;
-  int sxy = g.nx * g.ny;
-  int c = r * nx + i;
-  T bc = b[c];
-  T yc = A.dinv[c] * bc;
-  T ay = A.diag[c] * yc;
-  if (i > 0) ay -= A.wx[c - 1] * (A.dinv[c - 1] * b[c - 1]);
-  if (i < nx - 1) ay -= A.wx[c] * (A.dinv[c + 1] * b[c + 1]);
-  if (j > 0) ay -= A.wy[c - nx] * (A.dinv[c - nx] * b[c - nx]);
-  if (j < g.ny - 1) ay -= A.wy[c] * (A.dinv[c + nx] * b[c + nx]);
-  if (k > 0) ay -= A.wz[c - sxy] * (A.dinv[c - sxy] * b[c - sxy]);
-  if (k < g.nz - 1) ay -= A.wz[c] * (A.dinv[c + sxy] * b[c + sxy]);
-  if (MODE == 2) {
-    x1[c] = yc;
-    out[c] = bc - ay;
-  } else {
-    out[c] = yc + A.dinv[c] * (bc - ay);
+  const int j = blockIdx.x % g.ny, k0 = blockIdx.x / g.ny * zc, k1 = min(g.nz, k0 + zc);
+  const int nx = g.nx, sxy = g.nx * g.ny;
+  int c = (k0 * g.ny + j) * nx + i;
+  T ym = T(0), wm = T(0), yc = y[c];
+  if (k0 > 0) {
+    ym = y[c - sxy];
+    wm = A.wz[c - sxy];
   }
+  for (int k = k0; k < k1; ++k, c += sxy) {
+    const T wz = A.wz[c];  // 0 in the top layer
+    const T yp = k < g.nz - 1 ? y[c + sxy] : T(0);
+    T t = b[c] + (MODE == 2 ? A.gd[c] : A.g[c]) * yc;
+    if (i > 0) t += A.wx[c - 1] * y[c - 1];
+    if (i < nx - 1) t += A.wx[c] * y[c + 1];
+    if (j > 0) t += A.wy[c - nx] * y[c - nx];
+    if (j < g.ny - 1) t += A.wy[c] * y[c + nx];
+    t += wm * ym;
+    t += wz * yp;
+    out[c] = MODE == 2 ? A.q[c] * t : t;
+    ym = yc;
+    wm = wz;
+    yc = yp;
+  }
+}
+
+// Launch shape of k_sc: lines as wide as the grid needs (up to 4 warps), and as many layers
+// per thread (up to 4) as leave the SMs twice the threads they hold.
+struct ScShape {
+  dim3 grid;
+  int threads, zc;
+};
+static ScShape sc_shape(const GridP& g) {
+  ScShape s;
+  s.threads = std::min(kLineThreads, (g.nx + 31) / 32 * 32);
+  s.zc = 1;
+  while (s.zc < 4 && g.n / (2 * s.zc) >= 2LL * kNumSM * 2048) s.zc *= 2;
+  s.grid = dim3((unsigned)(g.ny * ((g.nz + s.zc - 1) / s.zc)), (unsigned)((g.nx + s.threads - 1) / s.threads), 1);
+  return s;
+}
+
+// b = s r on the way in, z = s y on the way out, and without a pre-sweep r = q b.
+template <class T>
+__global__ void k_sc_in(long long n, const T* __restrict__ s, const double* __restrict__ r, T* __restrict__ b) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    b[i] = s[i] * (T)r[i];
+}
+template <class T>
+__global__ void k_sc_out(long long n, const T* __restrict__ s, const T* __restrict__ y, double* __restrict__ z) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    z[i] = (double)(s[i] * y[i]);
+}
+template <class T>
+__global__ void k_sc_mul(long long n, const T* __restrict__ q, const T* __restrict__ b, T* __restrict__ r) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    r[i] = q[i] * b[i];
 }
 
 // Hybrid Gauss-Seidel (the paper's smoother, Sec. 5.2 / Sec. 6): Gauss-Seidel inside
@@ -685,6 +745,13 @@ template <>
 const Stencil4<float>& fine<float>(rich_ctx* c) { return c->H.st32; }
 
 template <class T>
+static const ScaledSt<T>& scaled(rich_ctx* c);
+template <>
+const ScaledSt<double>& scaled<double>(rich_ctx* c) { return c->H.sc64; }
+template <>
+const ScaledSt<float>& scaled<float>(rich_ctx* c) { return c->H.sc32; }
+
+template <class T>
 struct LevelView {
   int n;
   const int *rp, *col;
@@ -769,7 +836,7 @@ static int vcycle_level_hgs(rich_ctx* c, int l, const T* b, T** xres) {
   {
     ProfScope ps(st0 ? "resid_l0" : "csr_resid", c->st,
                  st0 ? (double)n * 7.0 * es : (double)n * (4.0 + 3.0 * es) + (double)L.A.nnz * (4.0 + es));
-    if (st0) k_st_smooth<T, 2><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, fine<T>(c), b, x, (T*)L.r);
+    if (st0) k_st_resid<T><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, fine<T>(c), b, x, (T*)L.r);
     else RICH_CHECK(csr_op<T, 3>(c, n, L.A.nnz, v.rp, v.col, v.val, (const T*)nullptr, b, x, (T*)L.r, &v.sa));
   }
   RICH_LAUNCH_CHECK();
@@ -831,54 +898,51 @@ static int vcycle_level(rich_ctx* c, int l, const T* b, T** xres) {
     return RICH_OK;
   }
   int nu1 = H.opts.nu1, nu2 = H.opts.nu2;
-  // finest level: stencil form (4 coefficient arrays + b + x in, x out)
-  const bool st0 = (l == 0);
   if (H.opts.smoother == RICH_SMOOTH_HYBRID_GS) return vcycle_level_hgs<T>(c, l, b, xres);
-  // warp-per-row CSR kernels where rows are long
-  const double st_bytes = (double)n * 8.0 * es;  // diag, 3 face weights, dinv, b, x in; x out
-  // In FP32 the first sweep from zero is folded into the next stencil pass (one pass
-  // over the finest level less); in FP64 the fold's extra products (D^-1 b at the six
-  // neighbours) cost more on GB300's narrow FP64 pipe than the pass it saves (ncu:
-  // 88-91 % FP64-pipe utilisation in these sweeps), so FP64 keeps separate passes.
-  constexpr bool kFold = sizeof(T) == 4;
-  if (kFold && st0 && nu1 == 1) {
-    // finest level, one pre-sweep: the sweep from zero and the residual in one pass
-    ProfScope ps("resid_l0", c->st, (double)n * 8.0 * es, 17.0 * n);
-    k_st_first<T, 2><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, fine<T>(c), b, x, (T*)L.r);
+  // the finest level in scaled form (H.scaled holds here: l1-Jacobi, more than one level)
+  const bool st0 = (l == 0);
+  const ScaledSt<T>& S = scaled<T>(c);
+  const ScShape sh = sc_shape(c->g);
+  const double st_bytes = (double)n * 7.0 * es;  // g, 3 face weights, b, y in; y out
+  auto sweep = [&](const T* from, T* to) -> int {
+    {
+      ProfScope ps(st0 ? "l1jacobi_l0" : "l1jacobi", c->st, st0 ? st_bytes : sweep_bytes,
+                   st0 ? 14.0 * n : 2.0 * L.A.nnz + 3.0 * n);
+      if (st0) k_sc<T, 1><<<sh.grid, sh.threads, 0, c->st>>>(c->g, S, sh.zc, b, from, to);
+      else RICH_CHECK(csr_op<T, 2>(c, n, L.A.nnz, v.rp, v.col, v.val, v.dinv, b, from, to, &v.sa));
+    }
     RICH_LAUNCH_CHECK();
-  } else if (nu1 > 0) {
-    int s0 = 1;
-    if (kFold && st0) {
-      // finest level: the first two sweeps from zero in one pass
-      ProfScope ps("l1jacobi_l0", c->st, (double)n * 7.0 * es, 20.0 * n);
-      k_st_first<T, 1><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, fine<T>(c), b, nullptr, x);
-      RICH_LAUNCH_CHECK();
-      s0 = 2;
-    } else {
-      // first sweep from x = 0: x = D_l1^-1 b, elementwise (on the finest level the
-      // stencil copy's 1/l1 array)
-      k_jacobi0<T><<<g, kBlock, 0, c->st>>>(n, st0 ? fine<T>(c).dinv : v.dinv, b, x);
+    return RICH_OK;
+  };
+  const T* cur = x;  // where the iterate is: on the finest level the first sweep's is b itself
+  if (nu1 > 0) {
+    if (st0) {
+      cur = b;
+    } else {  // first sweep from x = 0: x = D_l1^-1 b, elementwise
+      k_jacobi0<T><<<g, kBlock, 0, c->st>>>(n, v.dinv, b, x);
       RICH_LAUNCH_CHECK();
     }
-    for (int s = s0; s < nu1; ++s) {
-      {
-        ProfScope ps(l == 0 ? "l1jacobi_l0" : "l1jacobi", c->st, st0 ? st_bytes : sweep_bytes,
-                     st0 ? 16.0 * n : 2.0 * L.A.nnz + 3.0 * n);
-        if (st0) k_st_smooth<T, 1><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, fine<T>(c), b, x, t);
-        else RICH_CHECK(csr_op<T, 2>(c, n, L.A.nnz, v.rp, v.col, v.val, v.dinv, b, x, t, &v.sa));
-      }
-      RICH_LAUNCH_CHECK();
-      std::swap(x, t);
+    for (int s = 1; s < nu1; ++s) {
+      T* to = cur == x ? t : x;
+      RICH_CHECK(sweep(cur, to));
+      if (to == t) std::swap(x, t);
+      cur = x;
     }
     {
-      ProfScope ps(st0 ? "resid_l0" : "csr_resid", c->st, st0 ? st_bytes : sweep_bytes - (double)n * es);
-      if (st0) k_st_smooth<T, 2><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, fine<T>(c), b, x, (T*)L.r);
-      else RICH_CHECK(csr_op<T, 3>(c, n, L.A.nnz, v.rp, v.col, v.val, (const T*)nullptr, b, x, (T*)L.r, &v.sa));
+      ProfScope ps(st0 ? "resid_l0" : "csr_resid", c->st, st0 ? st_bytes + (double)n * es : sweep_bytes - (double)n * es,
+                   st0 ? 16.0 * n : 0.0);
+      if (st0) k_sc<T, 2><<<sh.grid, sh.threads, 0, c->st>>>(c->g, S, sh.zc, b, cur, (T*)L.r);
+      else RICH_CHECK(csr_op<T, 3>(c, n, L.A.nnz, v.rp, v.col, v.val, (const T*)nullptr, b, cur, (T*)L.r, &v.sa));
     }
     RICH_LAUNCH_CHECK();
   } else {
     RICH_CUDA(cudaMemsetAsync(x, 0, sizeof(T) * n, c->st));
-    RICH_CUDA(cudaMemcpyAsync(L.r, b, sizeof(T) * n, cudaMemcpyDeviceToDevice, c->st));
+    if (st0) {
+      k_sc_mul<T><<<g, kBlock, 0, c->st>>>(n, S.q, b, (T*)L.r);
+      RICH_LAUNCH_CHECK();
+    } else {
+      RICH_CUDA(cudaMemcpyAsync(L.r, b, sizeof(T) * n, cudaMemcpyDeviceToDevice, c->st));
+    }
   }
   Level& C = H.lv[l + 1];
   {
@@ -891,18 +955,15 @@ static int vcycle_level(rich_ctx* c, int l, const T* b, T** xres) {
   RICH_CHECK(vcycle_level<T>(c, l + 1, (const T*)C.b, &xc));
   {
     ProfScope ps("prolong", c->st, (double)n * (4.0 + 2.0 * es) + (double)L.P.nnz * (4.0 + es) + (double)C.n * es);
-    RICH_CHECK(csr_op<T, 1>(c, n, L.P.nnz, v.prp, v.pcol, v.pval, (const T*)nullptr, (const T*)nullptr, xc, x,
-                            &v.sp));
+    if (st0)  // y = cur + q (P xc)
+      RICH_CHECK(csr_op<T, 4>(c, n, L.P.nnz, v.prp, v.pcol, v.pval, S.q, cur, xc, x, &v.sp));
+    else
+      RICH_CHECK(csr_op<T, 1>(c, n, L.P.nnz, v.prp, v.pcol, v.pval, (const T*)nullptr, (const T*)nullptr, xc, x,
+                              &v.sp));
   }
   RICH_LAUNCH_CHECK();
   for (int s = 0; s < nu2; ++s) {
-    {
-      ProfScope ps(l == 0 ? "l1jacobi_l0" : "l1jacobi", c->st, st0 ? st_bytes : sweep_bytes,
-                   st0 ? 16.0 * n : 2.0 * L.A.nnz + 3.0 * n);
-      if (st0) k_st_smooth<T, 1><<<line_grid(c->g), kLineThreads, 0, c->st>>>(c->g, fine<T>(c), b, x, t);
-      else RICH_CHECK(csr_op<T, 2>(c, n, L.A.nnz, v.rp, v.col, v.val, v.dinv, b, x, t, &v.sa));
-    }
-    RICH_LAUNCH_CHECK();
+    RICH_CHECK(sweep(x, t));
     std::swap(x, t);
   }
   // keep the level's buffer pointers consistent with where the result lives
@@ -971,10 +1032,16 @@ static int vcycle_capture(rich_ctx* c) {
 
 // The level-0 right-hand side from r, and the result x into z.
 static int vcycle_in(rich_ctx* c, const double* r) {
-  Level& L0 = c->H.lv[0];
+  const Hierarchy& H = c->H;
+  const Level& L0 = H.lv[0];
   const long long n = c->g.n;
-  if (c->prec == RICH_PREC_MIXED) {
-    k_d2f<<<grid_for(n), kBlock, 0, c->st>>>(n, r, (float*)L0.b);
+  const int g = grid_for(n);
+  if (H.scaled) {
+    if (c->prec == RICH_PREC_MIXED) k_sc_in<float><<<g, kBlock, 0, c->st>>>(n, H.sc32.s, r, (float*)L0.b);
+    else k_sc_in<double><<<g, kBlock, 0, c->st>>>(n, H.sc64.s, r, (double*)L0.b);
+    RICH_LAUNCH_CHECK();
+  } else if (c->prec == RICH_PREC_MIXED) {
+    k_d2f<<<g, kBlock, 0, c->st>>>(n, r, (float*)L0.b);
     RICH_LAUNCH_CHECK();
   } else {
     RICH_CUDA(cudaMemcpyAsync(L0.b, r, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
@@ -982,9 +1049,15 @@ static int vcycle_in(rich_ctx* c, const double* r) {
   return RICH_OK;
 }
 static int vcycle_out(rich_ctx* c, const void* x, double* z) {
+  const Hierarchy& H = c->H;
   const long long n = c->g.n;
-  if (c->prec == RICH_PREC_MIXED) {
-    k_f2d<<<grid_for(n), kBlock, 0, c->st>>>(n, (const float*)x, z);
+  const int g = grid_for(n);
+  if (H.scaled) {
+    if (c->prec == RICH_PREC_MIXED) k_sc_out<float><<<g, kBlock, 0, c->st>>>(n, H.sc32.s, (const float*)x, z);
+    else k_sc_out<double><<<g, kBlock, 0, c->st>>>(n, H.sc64.s, (const double*)x, z);
+    RICH_LAUNCH_CHECK();
+  } else if (c->prec == RICH_PREC_MIXED) {
+    k_f2d<<<g, kBlock, 0, c->st>>>(n, (const float*)x, z);
     RICH_LAUNCH_CHECK();
   } else {
     RICH_CUDA(cudaMemcpyAsync(z, x, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
@@ -1087,6 +1160,7 @@ __global__ void k_fcg_update(long long n, double* __restrict__ x, double* __rest
 // 128^3, FGMRES(30): 667 us per iteration with two explicit projections, 598 with these passes.
 constexpr int kGsThreads = 256;
 constexpr int kGsBlocks = 2 * kNumSM;  // of the dots (fixed: deterministic summation order)
+constexpr int kGsUpdateBlocks = 4 * kNumSM;  // of the update: one wave (8 per SM left a second, 59 us against 46)
 constexpr int kGsTile = 4;             // basis vectors per sweep over a block's elements
 constexpr int kGsLd = 64;              // row length of the Gram matrix
 // Device scalars of an iteration (restart <= 63): h in [0, j], ||w - V h|| and its reciprocal.
@@ -1111,6 +1185,40 @@ __device__ __forceinline__ double warp_sum8(double (&a)[8]) {
   return a[0];
 }
 
+// The block's sums over its elements of M basis vectors (from v0) times w and vj, into
+// a[q] and a[4 + q].
+template <int M>
+__device__ __forceinline__ void gs_tile(long long n, const double* __restrict__ v0, const double* __restrict__ w,
+                                        const double* __restrict__ vj, double (&a)[8]) {
+  const long long stride = (long long)gridDim.x * kGsThreads;
+  long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x;
+  for (; i + stride < n; i += 2 * stride) {
+    const double w0 = w[i], w1 = w[i + stride], x0 = vj[i], x1 = vj[i + stride];
+    double p[M], r[M];
+#pragma unroll
+    for (int q = 0; q < M; ++q) {
+      p[q] = v0[q * n + i];
+      r[q] = v0[q * n + i + stride];
+    }
+#pragma unroll
+    for (int q = 0; q < M; ++q) {
+      a[q] = fma(p[q], w0, a[q]);
+      a[q + 4] = fma(p[q], x0, a[q + 4]);
+      a[q] = fma(r[q], w1, a[q]);
+      a[q + 4] = fma(r[q], x1, a[q + 4]);
+    }
+  }
+  if (i < n) {
+    const double w0 = w[i], x0 = vj[i];
+#pragma unroll
+    for (int q = 0; q < M; ++q) {
+      const double p = v0[q * n + i];
+      a[q] = fma(p, w0, a[q]);
+      a[q + 4] = fma(p, x0, a[q + 4]);
+    }
+  }
+}
+
 // h1 = V^T w and the newest row of G = V^T V (nv vectors, vj = V[nv - 1]); the last block
 // to finish forms h and leaves it at s[0, nv) and in the pinned mirror.
 __global__ void __launch_bounds__(kGsThreads) k_gs_dots(long long n, int nv, const double* __restrict__ V,
@@ -1123,40 +1231,14 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_dots(long long n, int nv, con
   __shared__ bool last;
   const double* vj = V + (long long)(nv - 1) * n;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const long long stride = (long long)gridDim.x * kGsThreads;
   for (int q0 = 0; q0 < nv; q0 += kGsTile) {
     double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const double* v0 = V + (long long)q0 * n;
     const int m = min(kGsTile, nv - q0);
-    long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x;
-    if (m == kGsTile) {
-      for (; i + stride < n; i += 2 * stride) {
-        const double w0 = w[i], w1 = w[i + stride], x0 = vj[i], x1 = vj[i + stride];
-        double p[kGsTile], r[kGsTile];
-#pragma unroll
-        for (int q = 0; q < kGsTile; ++q) {
-          p[q] = v0[q * n + i];
-          r[q] = v0[q * n + i + stride];
-        }
-#pragma unroll
-        for (int q = 0; q < kGsTile; ++q) {
-          a[q] = fma(p[q], w0, a[q]);
-          a[q + 4] = fma(p[q], x0, a[q + 4]);
-          a[q] = fma(r[q], w1, a[q]);
-          a[q + 4] = fma(r[q], x1, a[q + 4]);
-        }
-      }
-    }
-    for (; i < n; i += stride) {
-      const double w0 = w[i], x0 = vj[i];
-#pragma unroll
-      for (int q = 0; q < kGsTile; ++q)
-        if (q < m) {
-          const double p = v0[q * n + i];
-          a[q] = fma(p, w0, a[q]);
-          a[q + 4] = fma(p, x0, a[q + 4]);
-        }
-    }
+    if (m == 4) gs_tile<4>(n, v0, w, vj, a);
+    else if (m == 3) gs_tile<3>(n, v0, w, vj, a);
+    else if (m == 2) gs_tile<2>(n, v0, w, vj, a);
+    else gs_tile<1>(n, v0, w, vj, a);
     const double r = warp_sum8(a);
     if ((lane & 3) == 0) sh[wid][lane >> 2] = r;
     __syncthreads();
@@ -1221,8 +1303,9 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, c
     acc[0] = fma(t, t, acc[0]);
     acc[0] = fma(u, u, acc[0]);
   }
-  for (; i < n; i += stride) {
+  if (i < n) {
     double t = w[i];
+#pragma unroll 4
     for (int q = 0; q < nv; ++q) t = fma(-hs[q], V[(long long)q * n + i], t);
     out[i] = t;
     acc[0] = fma(t, t, acc[0]);
@@ -1247,15 +1330,16 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, c
   }
 }
 
-// V = f src (f from the device if fdev), and the V-cycle's right-hand side with it.
+// V = f src (f from the device if fdev), and the V-cycle's right-hand side with it (scaled
+// by sc, if given).
 template <class T>
 __global__ void k_stage(long long n, const double* src, const double* __restrict__ fdev, double f, double* V,
-                        T* __restrict__ b) {
+                        const T* __restrict__ sc, T* __restrict__ b) {
   if (fdev) f = *fdev;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const double v = f * src[i];
     V[i] = v;
-    if (b) b[i] = (T)v;
+    if (b) b[i] = sc ? sc[i] * (T)v : (T)v;
   }
 }
 
@@ -1473,13 +1557,16 @@ static int fgmres_precondition(rich_ctx* c, const double* src, const double* fde
   const long long n = c->g.n;
   const int g = grid_for(n);
   if (c->H.opts.precond == RICH_PRECOND_AS) {
-    k_stage<double><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, nullptr);
+    k_stage<double><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, nullptr, nullptr);
     RICH_LAUNCH_CHECK();
     return as_apply(c, V, z);
   }
   void* b = c->H.lv[0].b;
-  if (c->prec == RICH_PREC_MIXED) k_stage<float><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, (float*)b);
-  else k_stage<double><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, (double*)b);
+  const Hierarchy& H = c->H;
+  if (c->prec == RICH_PREC_MIXED)
+    k_stage<float><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, H.scaled ? H.sc32.s : nullptr, (float*)b);
+  else
+    k_stage<double><<<g, kBlock, 0, c->st>>>(n, src, fdev, f, V, H.scaled ? H.sc64.s : nullptr, (double*)b);
   RICH_LAUNCH_CHECK();
   return vcycle_staged(c, z);
 }
@@ -1489,7 +1576,7 @@ static int fgmres_precondition(rich_ctx* c, const double* src, const double* fde
 static int gs_pass(rich_ctx* c, int nv, const double* w, double* out) {
   KrylovWork& k = c->kw;
   const long long n = c->g.n;
-  const int g = std::min(grid_for(n), kGsBlocks), gu = std::min(grid_for(n, 2 * kBlock), 8 * kNumSM);
+  const int g = std::min(grid_for(n), kGsBlocks), gu = std::min(grid_for(n, 2 * kBlock), kGsUpdateBlocks);
   {
     ProfScope ps("multidot", c->st, (double)n * 8.0 * (nv + 1), 4.0 * n * nv);
     k_gs_dots<<<g, kGsThreads, 0, c->st>>>(n, nv, k.V, w, c->partials, k.gram, c->ticket, c->dsc, c->hsc);
