@@ -13,9 +13,9 @@
 //
 // What stays per problem is everything with a scalar in it: the Newton iteration
 // (norms, convergence test, line search with its own step length, statistics) and
-// FCG (its own alpha, beta and stopping test).  Dot products are segmented: grid
-// row y of a reduction kernel sums problem y, in the same fixed order for every
-// problem.  A problem that has converged, or failed, is frozen: its Newton
+// FCG (its own alpha, beta and stopping test, kept on the device: solve.cu).  Dot products
+// are segmented: grid row y of a reduction kernel sums problem y, in the same fixed order
+// for every problem.  A problem that has converged, or failed, is frozen: its Newton
 // correction is zero and its Krylov scalars are not applied.  A batch has no
 // FGMRES fallback: a problem whose FCG fails is reported RICH_ENOTCONV_LIN and the
 // server reruns it alone on the ordinary path.
@@ -43,50 +43,6 @@ __global__ void k_seg_dot2(long long ns, const double* __restrict__ a, const dou
     part[(long long)s * gridDim.x + blockIdx.x] = v[0];
     part[((long long)S + s) * gridDim.x + blockIdx.x] = v[1];
   }
-}
-
-// p_s = z_s - (sc[num + s] / sc[den + s]) p_s for active problems
-__global__ void k_seg_fcg_dir(long long ns, const double* __restrict__ z, double* __restrict__ p,
-                              const double* __restrict__ sc, int num, int den, const int* __restrict__ act) {
-  const int s = blockIdx.y;
-  if (!act[s]) return;
-  const long long base = (long long)s * ns;
-  const double beta = sc[num + s] / sc[den + s];
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ns; i += (long long)gridDim.x * blockDim.x)
-    p[base + i] = z[base + i] - beta * p[base + i];
-}
-
-// b_s = a_s for active problems
-__global__ void k_seg_copy(long long ns, const double* __restrict__ a, double* __restrict__ b,
-                           const int* __restrict__ act) {
-  const int s = blockIdx.y;
-  if (!act[s]) return;
-  const long long base = (long long)s * ns;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ns; i += (long long)gridDim.x * blockDim.x)
-    b[base + i] = a[base + i];
-}
-
-// active problems: alpha = sc[num + s] / sc[den + s]; x += alpha p; r -= alpha q;
-// partials of ||r_s||^2 (zero for frozen problems)
-__global__ void k_seg_fcg_update(long long ns, double* __restrict__ x, double* __restrict__ r,
-                                 const double* __restrict__ p, const double* __restrict__ q,
-                                 const double* __restrict__ sc, int num, int den, const int* __restrict__ act,
-                                 double* __restrict__ part) {
-  const int s = blockIdx.y;
-  const long long base = (long long)s * ns;
-  double v[1] = {0.0};
-  if (act[s]) {
-    const double alpha = sc[num + s] / sc[den + s];
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ns;
-         i += (long long)gridDim.x * blockDim.x) {
-      x[base + i] += alpha * p[base + i];
-      double ri = r[base + i] - alpha * q[base + i];
-      r[base + i] = ri;
-      v[0] += ri * ri;
-    }
-  }
-  block_sum<1>(v);
-  if (threadIdx.x == 0) part[(long long)s * gridDim.x + blockIdx.x] = v[0];
 }
 
 // y_s = a_s + lam[s] d_s
@@ -155,89 +111,6 @@ static int upload_flags(rich_ctx* c, BatchWork& w, const std::vector<int>& a) {
   return RICH_OK;
 }
 
-// Segmented FCG (Notay, truncation 1) for J x = b with x0 = 0.  Problems with
-// active[s] == 0 on entry keep x_s = 0.  On return fail[s] = 1 where FCG stopped
-// on (p, q) <= 0, on residual growth, on stagnation (krylov.stall) or at maxit;
-// its[s] counts the iterations.
-static int batch_fcg(rich_ctx* c, BatchWork& w, int S, const double* b, double* x, const rich_krylov_opts* o,
-                     std::vector<int> active, std::vector<int>& fail, std::vector<int>& its) {
-  KrylovWork& k = c->kw;
-  const long long ns = c->g.n / S;
-  const int nb = red_grid(ns);
-  const dim3 grid(nb, S), vgrid(grid_for(ns), S);
-  double* sc = w.dsc;  // [0] rr, [1] zq, [2] pq, [3] pr, [4] pq_prev (each S wide)
-  fail.assign(S, 0);
-  its.assign(S, 0);
-  RICH_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * c->g.n, c->st));
-  RICH_CUDA(cudaMemcpyAsync(k.r, b, sizeof(double) * c->g.n, cudaMemcpyDeviceToDevice, c->st));
-  k_seg_dot2<<<grid, kBlock, 0, c->st>>>(ns, b, b, nullptr, nullptr, c->partials);
-  RICH_LAUNCH_CHECK();
-  RICH_CHECK(seg_finish(c, c->partials, nb, 1, S, sc, w.hsc));
-  std::vector<double> target(S), best(S), window_start(S);
-  for (int s = 0; s < S; ++s) {
-    double bn = sqrt(w.hsc[s]);
-    if (!std::isfinite(bn)) return RICH_ENONFINITE;
-    if (!(bn > 0)) active[s] = 0;
-    target[s] = o->eta * bn;
-    best[s] = bn;
-    window_start[s] = bn;
-  }
-  double* q = k.q;
-  double* qprev = k.qprev;
-  for (int it = 1; it <= o->maxit; ++it) {
-    if (std::none_of(active.begin(), active.end(), [](int a) { return a != 0; })) break;
-    RICH_CHECK(upload_flags(c, w, active));
-    RICH_CHECK(vcycle_apply(c, k.r, k.z));
-    if (it == 1) {
-      k_seg_copy<<<vgrid, kBlock, 0, c->st>>>(ns, k.z, k.p, w.dact);
-    } else {
-      k_seg_dot2<<<grid, kBlock, 0, c->st>>>(ns, k.z, qprev, nullptr, nullptr, c->partials);
-      RICH_LAUNCH_CHECK();
-      RICH_CHECK(finish_sums(c, c->partials, nb, S, sc + 1 * S));
-      k_seg_fcg_dir<<<vgrid, kBlock, 0, c->st>>>(ns, k.z, k.p, sc, 1 * S, 4 * S, w.dact);
-    }
-    RICH_LAUNCH_CHECK();
-    RICH_CHECK(stencil_apply(c, c->J7, k.p, q));
-    k_seg_dot2<<<grid, kBlock, 0, c->st>>>(ns, k.p, q, k.p, k.r, c->partials);
-    RICH_LAUNCH_CHECK();
-    RICH_CHECK(finish_sums(c, c->partials, nb, 2 * S, sc + 2 * S));  // pq at 2S, pr at 3S
-    k_seg_fcg_update<<<grid, kBlock, 0, c->st>>>(ns, x, k.r, k.p, q, sc, 3 * S, 2 * S, w.dact, c->partials);
-    RICH_LAUNCH_CHECK();
-    RICH_CHECK(finish_sums(c, c->partials, nb, S, sc + 0));
-    RICH_CUDA(cudaMemcpyAsync(sc + 4 * S, sc + 2 * S, sizeof(double) * S, cudaMemcpyDeviceToDevice, c->st));
-    RICH_CUDA(cudaMemcpyAsync(w.hsc, sc, sizeof(double) * 4 * S, cudaMemcpyDeviceToHost, c->st));
-    RICH_CUDA(cudaStreamSynchronize(c->st));
-    for (int s = 0; s < S; ++s) {
-      if (!active[s]) continue;
-      double rn = sqrt(w.hsc[s]), pq = w.hsc[2 * S + s];
-      its[s] = it;
-      if (!std::isfinite(rn) || !std::isfinite(pq)) return RICH_ENONFINITE;
-      if (!(pq > 0) || rn > 10.0 * best[s]) {  // the update applied: x is no better than before; stop here
-        fail[s] = 1;
-        active[s] = 0;
-        continue;
-      }
-      if (rn <= target[s]) {
-        active[s] = 0;
-        continue;
-      }
-      if (it % kStallWindow == 0) {  // stagnation over the last window (krylov.stall)
-        if (o->stall > 0 && rn > (1.0 - o->stall) * window_start[s]) {
-          fail[s] = 1;
-          active[s] = 0;
-          continue;
-        }
-        window_start[s] = rn;
-      }
-      best[s] = std::min(best[s], rn);
-    }
-    std::swap(q, qprev);
-  }
-  for (int s = 0; s < S; ++s)
-    if (active[s]) fail[s] = 1;  // maxit
-  return RICH_OK;
-}
-
 static int ensure_newton_batch(rich_ctx* c) {
   if (c->F) return RICH_OK;
   long long n = c->g.n;
@@ -258,7 +131,6 @@ static int ensure_krylov_batch(rich_ctx* c) {
   RICH_CHECK(dalloc(&k.r, n));
   RICH_CHECK(dalloc(&k.p, n));
   RICH_CHECK(dalloc(&k.q, n));
-  RICH_CHECK(dalloc(&k.qprev, n));
   RICH_CHECK(dalloc(&k.z, n));
   RICH_CHECK(dalloc(&k.w, n));
   RICH_CHECK(dalloc(&k.hcoef, 128));
@@ -287,7 +159,8 @@ static int batch_step(rich_ctx* c, BatchWork& w, int S, double* p, double dt, co
     status[s] = RICH_OK;
   }
   std::vector<double> fn(S), tol(S), flo(S), f0(S), slope(S), lam(S), ft(S), flo_t(S);
-  std::vector<int> conv(S, 0), done(S, 0), newton_act(S, 0), search(S, 0), lin_fail, lin_its;
+  std::vector<int> conv(S, 0), done(S, 0), newton_act(S, 0), search(S, 0);
+  FcgResult lin[kMaxBatch];
   RICH_CHECK(residual_eval(c, p, nullptr, dt, c->F, true, true, c->s_old, S));
   RICH_CHECK(wait_scalars(c, 3 * S, w.hsc));
   for (int s = 0; s < S; ++s) {
@@ -328,10 +201,11 @@ static int batch_step(rich_ctx* c, BatchWork& w, int S, double* p, double dt, co
     RICH_CHECK(upload_flags(c, w, newton_act));
     k_seg_neg<<<vgrid, kBlock, 0, c->st>>>(ns, c->F, w.dact, c->rhs);
     RICH_LAUNCH_CHECK();
-    RICH_CHECK(batch_fcg(c, w, S, c->rhs, c->d, &o->krylov, newton_act, lin_fail, lin_its));
+    // segmented FCG: the problems that sit out have a zero right-hand side and keep d = 0
+    RICH_CHECK(fcg_run(c, S, c->rhs, c->d, &o->krylov, lin));
     for (int s = 0; s < S; ++s) {
-      st[s].linear_its += lin_its[s];
-      if (newton_act[s] && lin_fail[s]) {
+      st[s].linear_its += lin[s].it;
+      if (newton_act[s] && lin[s].reason) {
         newton_act[s] = 0;
         done[s] = 1;
         status[s] = RICH_ENOTCONV_LIN;

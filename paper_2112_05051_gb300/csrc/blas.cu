@@ -93,6 +93,8 @@ __global__ void k_prof_delay(long long cycles) {
 }
 constexpr long long kProfDelayCycles = 40000;  // ~20 us at 2 GHz
 
+void gpu_delay(cudaStream_t st, long long cycles) { k_prof_delay<<<1, 32, 0, st>>>(cycles); }
+
 void prof_restart(cudaStream_t st) {
   if (g_prof_open < 0) return;
   k_prof_delay<<<1, 32, 0, st>>>(kProfDelayCycles);

@@ -268,11 +268,9 @@ struct Hierarchy {
   void* vc_out = nullptr;
   int vc_calls = 0;
   bool vc_off = false;            // capture failed: direct launches for this hierarchy
-  // an FCG iteration (it >= 2, V-cycle to the read-back of its scalars) as one graph
-  // per parity of it (q and q_prev alternate), writing the correction fcg_x
-  cudaGraphExec_t fcg_exec[2] = {nullptr, nullptr};
-  long long fcg_nodes[2] = {0, 0};
-  const double* fcg_x = nullptr;
+  // FCG's iterations as one graph (a WHILE loop, solve.cu); kernels per iteration
+  cudaGraphExec_t fcg_exec = nullptr;
+  long long fcg_nodes = 0;
   bool fcg_off = false;
   // one-level additive Schwarz (precond = RICH_PRECOND_AS): ILU(0) diagonals and
   // subdomain solutions (hierarchy precision), FP32 staging of r and z in MIXED
@@ -295,11 +293,12 @@ struct KrylovWork {
   double* r = nullptr;
   double* p = nullptr;
   double* q = nullptr;
-  double* qprev = nullptr;
   double* z = nullptr;
   double* w = nullptr;
   double* hcoef = nullptr;  // device coefficients (m+1)
   double* gram = nullptr;   // V^T V of FGMRES' basis (64 x 64)
+  void* fcg = nullptr;      // FCG's scalars on the device (FcgDev)
+  void* fcg_out = nullptr;  // and what the host reads of them (pinned)
   int fail_reason = 0;      // last failure: 0 none, FCG 1 maxit, 2 (p, J p) <= 0, 3 residual growth;
                             // 4 stagnation (an FCG window or an FGMRES restart cycle, krylov.stall)
 };
@@ -567,6 +566,16 @@ int amg_build(rich_ctx* c, const rich_amg_opts* o);
 int amg_refresh(rich_ctx* c);
 int amg_update_fine(rich_ctx* c);
 void amg_free(rich_ctx* c);
+
+// One problem's outcome of an FCG solve (reason: 0 converged, else KrylovWork::fail_reason).
+struct FcgResult {
+  double rn, bn;
+  int it, reason;
+};
+int fcg_run(rich_ctx* c, int S, const double* b, double* x, const rich_krylov_opts* o, FcgResult* res);
+
+// Keeps the stream busy for a number of GPU clocks (the loop ends by itself).
+void gpu_delay(cudaStream_t st, long long cycles);
 
 // blas.cu: whether a profiling target is set (the autotuner then stays off)
 bool profiling_active();

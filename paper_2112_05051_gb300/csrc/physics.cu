@@ -616,11 +616,15 @@ int rich_destroy(rich_ctx* c) {
   dfree(k.r);
   dfree(k.p);
   dfree(k.q);
-  dfree(k.qprev);
   dfree(k.z);
   dfree(k.w);
   dfree(k.hcoef);
   dfree(k.gram);
+  {
+    char* d = static_cast<char*>(k.fcg);
+    dfree(d);
+    pinned_put(k.fcg_out);
+  }
   pinned_put(c->hsc);
   delete c;
   return RICH_OK;

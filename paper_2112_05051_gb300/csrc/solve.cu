@@ -353,6 +353,7 @@ struct TuneVal {
   float us;      // its time per launch
   int best_csr;  // fastest CSR candidate (used where a matrix of the class has no SELL copy)
 };
+constexpr long long kTuneDelay = 60000;  // ~30 us: longer than the host takes to queue the timed launches
 static std::mutex g_tune_mu;
 static std::map<TuneKey, TuneVal> g_tune;
 
@@ -427,6 +428,7 @@ static int csr_op(rich_ctx* c, int n, long long nnz, const int* rp, const int* c
                     kSellVariant8, kSellVariant2, kSellVariantP}) {
         if (is_sell(g) && !sell_ok) continue;
         csr_launch<T, MODE>(c->st, g, n, rp, col, val, dinv, b, x, scratch, sl, sval);
+        gpu_delay(c->st, kTuneDelay);  // the launches queue up behind it: the events see the GPU alone
         RICH_CUDA(cudaEventRecord(e0, c->st));
         for (int rep = 0; rep < 3; ++rep) csr_launch<T, MODE>(c->st, g, n, rp, col, val, dinv, b, x, scratch, sl, sval);
         RICH_CUDA(cudaEventRecord(e1, c->st));
@@ -1110,44 +1112,6 @@ int vcycle_apply(rich_ctx* c, const double* r, double* z) {
 
 // ---------------------------------------------------------------- Krylov kernels (FP64)
 
-__global__ void k_dot2(long long n, const double* __restrict__ a, const double* __restrict__ b,
-                       const double* __restrict__ cc, const double* __restrict__ d, double* __restrict__ partials) {
-  double v[2] = {0.0, 0.0};
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    v[0] += a[i] * b[i];
-    v[1] += cc[i] * d[i];
-  }
-  block_sum<2>(v);
-  if (threadIdx.x == 0) {
-    partials[blockIdx.x] = v[0];
-    partials[gridDim.x + blockIdx.x] = v[1];
-  }
-}
-
-// p = z - (s[num] / s[den]) p
-__global__ void k_fcg_dir(long long n, const double* __restrict__ z, double* __restrict__ p,
-                          const double* __restrict__ s, int num, int den) {
-  double beta = s[num] / s[den];
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    p[i] = z[i] - beta * p[i];
-}
-
-// alpha = s[num]/s[den]; x += alpha p; r -= alpha q; partial sums of r.r
-__global__ void k_fcg_update(long long n, double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
-                             const double* __restrict__ q, const double* __restrict__ s, int num, int den,
-                             double* __restrict__ partials) {
-  double alpha = s[num] / s[den];
-  double v[1] = {0.0};
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    x[i] += alpha * p[i];
-    double ri = r[i] - alpha * q[i];
-    r[i] = ri;
-    v[0] += ri * ri;
-  }
-  block_sum<1>(v);
-  if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
-}
-
 // ---- Gram-Schmidt of FGMRES, in two passes over the basis (classical Gram-Schmidt with
 // the second projection taken from the basis' Gram matrix: Swirydowicz, Langou, Ananthan,
 // Yang, Thomas, "Low synchronization Gram-Schmidt and generalized minimal residual
@@ -1371,18 +1335,15 @@ __global__ void k_axpby(long long n, const double* __restrict__ a, double lam, c
     y[i] = a[i] + lam * d[i];
 }
 
-__global__ void k_copy_scalar(double* s, int from, int to) { s[to] = s[from]; }
-
 static int ensure_krylov(rich_ctx* c, int m) {
   KrylovWork& k = c->kw;
   long long n = c->g.n;
   if (k.n != n) {
-    dfree(k.x); dfree(k.r); dfree(k.p); dfree(k.q); dfree(k.qprev); dfree(k.z); dfree(k.w);
+    dfree(k.x); dfree(k.r); dfree(k.p); dfree(k.q); dfree(k.z); dfree(k.w);
     RICH_CHECK(dalloc(&k.x, n));
     RICH_CHECK(dalloc(&k.r, n));
     RICH_CHECK(dalloc(&k.p, n));
     RICH_CHECK(dalloc(&k.q, n));
-    RICH_CHECK(dalloc(&k.qprev, n));
     RICH_CHECK(dalloc(&k.z, n));
     RICH_CHECK(dalloc(&k.w, n));
     RICH_CHECK(dalloc(&k.hcoef, 128));
@@ -1399,157 +1360,401 @@ static int ensure_krylov(rich_ctx* c, int m) {
   return RICH_OK;
 }
 
-// Flexible CG (Notay, truncation 1).  Returns RICH_ENOTCONV_LIN on maxit, on
-// (p, q) <= 0, or when ||r|| exceeds 10x the smallest seen.
-// One FCG iteration from the preconditioner application to the copy of its scalars
-// (rr, zq, pq) into the pinned host mirror; `first`: the first iteration (p = z).
-// Under capture the V-cycle's kernels are recorded directly.
-static int fcg_iteration(rich_ctx* c, double* x, double* q, const double* qprev, bool first, bool capturing) {
+// ---------------------------------------------------------------- flexible CG on the device
+// Notay's flexible CG (truncation 1), for one problem or S of them stacked along z, each
+// with its own scalars, tests and iteration count; a problem that has stopped is frozen.
+// An iteration is the V-cycle and four kernels: z and z . q_prev, the direction, q = J p
+// with p . q and p . r, and the update with ||r||^2, whose last block makes the decisions
+// (convergence, (p, q) <= 0, growth, stagnation, maxit) and writes the next right-hand
+// side's scaling in the same pass.  The iterations are the body of a WHILE node of a CUDA
+// graph, which the last block continues or ends: no host turn-round (about 10 us) and no
+// launches (0.75 us per kernel) between iterations, 2.5 us for the loop.
+// 48^3 MIXED, V(1,1): 27 launches and a synchronisation took 78 us per iteration.
+struct FcgSeg {
+  double zq, pq, pr, pq_prev;            // of the iteration under way; (p, q) of the last one
+  double rn, bn, target, best, window;   // ||r||, ||b||, the tests' references
+  int it, reason;                        // iterations; why it stopped (kFcg...), 0 while running
+};
+struct FcgOut {  // pinned mirror
+  double rn, bn;
+  int it, reason;
+};
+constexpr int kFcgMaxSeg = 32;
+struct FcgDev {
+  FcgSeg seg[kFcgMaxSeg];
+  double stall;
+  int maxit;
+};
+// 1..4 are KrylovWork::fail_reason's
+constexpr int kFcgConverged = 10, kFcgZero = 11, kFcgNonfinite = 12;
+constexpr int kFcgThreads = 256;
+static_assert(sizeof(FcgOut) * kFcgMaxSeg <= kPinnedBlock, "the mirror is one pinned block");
+
+// Blocks per problem: two per SM in all, fewer where there are fewer cells.
+static int fcg_blocks(long long ns, int S) {
+  const long long most = std::max(1, 2 * kNumSM / S);
+  return (int)std::min(most, (ns + kFcgThreads - 1) / kFcgThreads);
+}
+
+// Block sums v of this block's problem to the partials; in the last block to finish, the
+// totals of every problem, tot[q * S + s], in block order.
+template <int NQ>
+__device__ __forceinline__ bool fcg_sums(double (&v)[NQ], double* part, unsigned* ticket, double* tot) {
+  constexpr int W = kFcgThreads / 32;
+  __shared__ double sh[W][NQ];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nb = gridDim.x, S = gridDim.y;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+  if (lane == 0)
+    for (int q = 0; q < NQ; ++q) sh[wid][q] = v[q];
+  __syncthreads();
+  if (threadIdx.x < NQ) {
+    double t = 0.0;
+    for (int w = 0; w < W; ++w) t += sh[w][threadIdx.x];
+    part[((long long)threadIdx.x * S + blockIdx.y) * nb + blockIdx.x] = t;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == (unsigned)(nb * S) - 1;
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  for (int i = wid; i < NQ * S; i += W) {
+    double t = 0.0;
+    for (int k = lane; k < nb; k += 32) t += __ldcg(&part[(long long)i * nb + k]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (lane == 0) tot[i] = t;
+  }
+  if (threadIdx.x == 0) *ticket = 0;
+  __syncthreads();
+  return true;
+}
+
+// x = 0, r = b, the V-cycle's right-hand side; ||b|| and the tests' references.
+template <class T>
+__global__ void __launch_bounds__(kFcgThreads) k_fcg_begin(long long ns, const double* __restrict__ b,
+                                                           double* __restrict__ x, double* __restrict__ r,
+                                                           const T* __restrict__ sc, T* __restrict__ vb, double eta,
+                                                           double stall, int maxit, FcgDev* __restrict__ dev,
+                                                           double* __restrict__ part, unsigned* __restrict__ ticket,
+                                                           FcgOut* __restrict__ out) {
+  __shared__ double tot[kFcgMaxSeg];
+  const long long base = blockIdx.y * ns;
+  double v[1] = {0.0};
+  for (long long i = blockIdx.x * (long long)kFcgThreads + threadIdx.x; i < ns;
+       i += (long long)gridDim.x * kFcgThreads) {
+    const double t = b[base + i];
+    x[base + i] = 0.0;
+    r[base + i] = t;
+    if (vb) vb[base + i] = sc[base + i] * (T)t;
+    v[0] = fma(t, t, v[0]);
+  }
+  if (!fcg_sums<1>(v, part, ticket, tot)) return;
+  if (threadIdx.x == 0) {
+    dev->stall = stall;
+    dev->maxit = maxit;
+  }
+  if (threadIdx.x < gridDim.y) {
+    FcgSeg s{};
+    s.bn = s.rn = s.best = s.window = sqrt(tot[threadIdx.x]);
+    s.target = eta * s.bn;
+    if (!isfinite(s.bn)) s.reason = kFcgNonfinite;
+    else if (!(s.bn > 0)) s.reason = kFcgZero;
+    dev->seg[threadIdx.x] = s;
+    out[threadIdx.x] = FcgOut{s.rn, s.bn, 0, s.reason};
+  }
+}
+
+// z = sc y (given y; else z is there already) and z . q_prev.
+template <class T>
+__global__ void __launch_bounds__(kFcgThreads) k_fcg_z(long long ns, const T* __restrict__ sc, const T* __restrict__ y,
+                                                       double* __restrict__ z, const double* __restrict__ q,
+                                                       FcgDev* __restrict__ dev, double* __restrict__ part,
+                                                       unsigned* __restrict__ ticket) {
+  __shared__ double tot[kFcgMaxSeg];
+  const long long base = blockIdx.y * ns;
+  const bool first = dev->seg[blockIdx.y].it == 0;  // no q yet
+  double v[1] = {0.0};
+  for (long long i = base + blockIdx.x * (long long)kFcgThreads + threadIdx.x; i < base + ns;
+       i += (long long)gridDim.x * kFcgThreads) {
+    double t;
+    if (y) {
+      t = (double)(sc[i] * y[i]);
+      z[i] = t;
+    } else {
+      t = z[i];
+    }
+    if (!first) v[0] = fma(t, q[i], v[0]);
+  }
+  if (fcg_sums<1>(v, part, ticket, tot) && threadIdx.x < gridDim.y) dev->seg[threadIdx.x].zq = tot[threadIdx.x];
+}
+
+// p = z - (zq / pq_prev) p; the first direction is z.
+__global__ void k_fcg_dir(long long ns, const double* __restrict__ z, double* __restrict__ p,
+                          const FcgDev* __restrict__ dev) {
+  const FcgSeg& s = dev->seg[blockIdx.y];
+  if (s.reason) return;
+  const bool first = s.it == 0;
+  const double beta = first ? 0.0 : s.zq / s.pq_prev;
+  const long long base = blockIdx.y * ns;
+  for (long long i = base + blockIdx.x * (long long)blockDim.x + threadIdx.x; i < base + ns;
+       i += (long long)gridDim.x * blockDim.x)
+    p[i] = first ? z[i] : z[i] - beta * p[i];
+}
+
+// q = J p, p . q and p . r.
+__global__ void __launch_bounds__(kFcgThreads) k_fcg_apply(GridP g, long long ns, const double* __restrict__ J,
+                                                           const double* __restrict__ p, const double* __restrict__ r,
+                                                           double* __restrict__ q, FcgDev* __restrict__ dev,
+                                                           double* __restrict__ part, unsigned* __restrict__ ticket) {
+  __shared__ double tot[2 * kFcgMaxSeg];
+  const long long n = g.n;
+  const int sxy = g.nx * g.ny, base = (int)(blockIdx.y * ns);
+  double v[2] = {0.0, 0.0};
+  for (int l = blockIdx.x * kFcgThreads + threadIdx.x; l < (int)ns; l += gridDim.x * kFcgThreads) {
+    const int c = base + l, row = c / g.nx, i = c - row * g.nx, k = row / g.ny, j = row - k * g.ny, kl = k % g.nzs;
+    const double pc = p[c];
+    double t = J[c] * pc;
+    if (i > 0) t += J[n + c] * p[c - 1];
+    if (i < g.nx - 1) t += J[2 * n + c] * p[c + 1];
+    if (j > 0) t += J[3 * n + c] * p[c - g.nx];
+    if (j < g.ny - 1) t += J[4 * n + c] * p[c + g.nx];
+    if (kl > 0) t += J[5 * n + c] * p[c - sxy];
+    if (kl < g.nzs - 1) t += J[6 * n + c] * p[c + sxy];
+    q[c] = t;
+    v[0] = fma(pc, t, v[0]);
+    v[1] = fma(pc, r[c], v[1]);
+  }
+  if (fcg_sums<2>(v, part, ticket, tot) && threadIdx.x < gridDim.y) {
+    dev->seg[threadIdx.x].pq = tot[threadIdx.x];
+    dev->seg[threadIdx.x].pr = tot[gridDim.y + threadIdx.x];
+  }
+}
+
+// x += alpha p, r -= alpha q, the V-cycle's next right-hand side; then the tests.
+template <class T>
+__global__ void __launch_bounds__(kFcgThreads) k_fcg_update(long long ns, double* __restrict__ x,
+                                                            double* __restrict__ r, const double* __restrict__ p,
+                                                            const double* __restrict__ q, const T* __restrict__ sc,
+                                                            T* __restrict__ vb, FcgDev* __restrict__ dev,
+                                                            double* __restrict__ part, unsigned* __restrict__ ticket,
+                                                            FcgOut* __restrict__ out,
+                                                            cudaGraphConditionalHandle loop, int looped) {
+  __shared__ double tot[kFcgMaxSeg];
+  __shared__ int running, bad;
+  const long long base = blockIdx.y * ns;
+  double v[1] = {0.0};
+  if (dev->seg[blockIdx.y].reason == 0) {
+    const double alpha = dev->seg[blockIdx.y].pr / dev->seg[blockIdx.y].pq;
+    for (long long i = base + blockIdx.x * (long long)kFcgThreads + threadIdx.x; i < base + ns;
+         i += (long long)gridDim.x * kFcgThreads) {
+      x[i] += alpha * p[i];
+      const double t = r[i] - alpha * q[i];
+      r[i] = t;
+      if (vb) vb[i] = sc[i] * (T)t;
+      v[0] = fma(t, t, v[0]);
+    }
+  }
+  if (threadIdx.x == 0) running = bad = 0;
+  if (!fcg_sums<1>(v, part, ticket, tot)) return;
+  if (threadIdx.x < gridDim.y) {
+    FcgSeg& s = dev->seg[threadIdx.x];
+    if (s.reason == 0) {
+      const double rn = sqrt(tot[threadIdx.x]);
+      ++s.it;
+      s.rn = rn;
+      s.pq_prev = s.pq;
+      if (!isfinite(rn) || !isfinite(s.pq)) s.reason = kFcgNonfinite;
+      else if (!(s.pq > 0)) s.reason = 2;
+      else if (rn <= s.target) s.reason = kFcgConverged;
+      else if (rn > 10.0 * s.best) s.reason = 3;
+      else if (s.it % kStallWindow == 0) {  // stagnation over the last window
+        if (dev->stall > 0 && rn > (1.0 - dev->stall) * s.window) s.reason = 4;
+        s.window = rn;
+      }
+      if (s.reason == 0 && s.it >= dev->maxit) s.reason = 1;
+      s.best = fmin(s.best, rn);
+      out[threadIdx.x] = FcgOut{rn, s.bn, s.it, s.reason};
+    }
+    if (s.reason == 0) atomicOr(&running, 1);
+    if (s.reason == kFcgNonfinite) atomicOr(&bad, 1);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && looped) cudaGraphSetConditional(loop, running && !bad ? 1 : 0);
+}
+
+template <class T>
+static T* vcycle_rhs(rich_ctx* c) { return c->H.scaled ? (T*)c->H.lv[0].b : nullptr; }
+
+// One iteration on S problems, launched or captured as it comes.
+template <class T>
+static int fcg_body(rich_ctx* c, int S, cudaGraphConditionalHandle loop, int looped) {
   KrylovWork& k = c->kw;
-  const long long n = c->g.n;
-  const int g = grid_for(n), nb = red_grid(n);
-  double* s = c->dsc;  // 0 rr, 1 zq, 2 pq, 3 pr, 4 pq_prev
-  if (capturing) {
-    RICH_CHECK(vcycle_in(c, k.r));
-    RICH_CHECK(vcycle_direct(c, k.z));
+  Hierarchy& H = c->H;
+  const long long n = c->g.n, ns = n / S;
+  const dim3 grid(fcg_blocks(ns, S), S);
+  const T* sc = scaled<T>(c).s;
+  FcgDev* dev = static_cast<FcgDev*>(k.fcg);
+  FcgOut* out = static_cast<FcgOut*>(k.fcg_out);
+  const T* y = nullptr;
+  if (H.opts.precond == RICH_PRECOND_AS) {
+    RICH_CHECK(as_apply(c, k.r, k.z));
   } else {
-    RICH_CHECK(vcycle_apply(c, k.r, k.z));
+    if (!H.scaled) RICH_CHECK(vcycle_in(c, k.r));
+    T* res = nullptr;
+    RICH_CHECK(vcycle_level<T>(c, 0, (const T*)H.lv[0].b, &res));
+    if (H.scaled) y = res;
+    else RICH_CHECK(vcycle_out(c, res, k.z));
   }
-  if (first) {
-    RICH_CUDA(cudaMemcpyAsync(k.p, k.z, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
-  } else {
-    RICH_CHECK(dot(c, k.z, qprev, n, s + 1));
-    k_fcg_dir<<<g, kBlock, 0, c->st>>>(n, k.z, k.p, s, 1, 4);
-    RICH_LAUNCH_CHECK();
-  }
-  RICH_CHECK(stencil_apply(c, c->J7, k.p, q));
-  k_dot2<<<nb, kBlock, 0, c->st>>>(n, k.p, q, k.p, k.r, c->partials);
+  k_fcg_z<T><<<grid, kFcgThreads, 0, c->st>>>(ns, sc, y, k.z, k.q, dev, c->partials, c->ticket);
   RICH_LAUNCH_CHECK();
-  RICH_CHECK(finish_sums(c, c->partials, nb, 2, s + 2));
+  k_fcg_dir<<<dim3(grid_for(ns), S), kBlock, 0, c->st>>>(ns, k.z, k.p, dev);
+  RICH_LAUNCH_CHECK();
+  {
+    ProfScope ps("stencil_spmv", c->st, (double)n * 80.0, (double)n * 17.0);
+    k_fcg_apply<<<grid, kFcgThreads, 0, c->st>>>(c->g, ns, c->J7, k.p, k.r, k.q, dev, c->partials, c->ticket);
+  }
+  RICH_LAUNCH_CHECK();
   {
     ProfScope ps("fcg_update", c->st, (double)n * 48.0);
-    k_fcg_update<<<nb, kBlock, 0, c->st>>>(n, x, k.r, k.p, q, s, 3, 2, c->partials);
+    k_fcg_update<T><<<grid, kFcgThreads, 0, c->st>>>(ns, k.x, k.r, k.p, k.q, sc, vcycle_rhs<T>(c), dev, c->partials,
+                                                     c->ticket, out, loop, looped);
   }
   RICH_LAUNCH_CHECK();
-  RICH_CHECK(finish_sums(c, c->partials, nb, 1, s + 0));
-  k_copy_scalar<<<1, 1, 0, c->st>>>(s, 2, 4);
-  RICH_LAUNCH_CHECK();
-  RICH_CUDA(cudaMemcpyAsync(c->hsc, s, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
   return RICH_OK;
 }
 
-// Captures fcg_iteration (not the first) with these q, q_prev and x as graph `par`,
-// as vcycle_capture does; a failed capture leaves direct launches.
-static void fcg_capture(rich_ctx* c, int par, double* x, double* q, const double* qprev) {
+// Captures the loop: a WHILE node whose body is fcg_body.  As for the V-cycle, on a private
+// stream after a direct application; a failure leaves direct launches.
+template <class T>
+static void fcg_capture(rich_ctx* c, int S) {
   Hierarchy& H = c->H;
-  cudaStream_t cs;
-  if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
-    cudaGetLastError();
-    H.fcg_off = true;
-    return;
-  }
+  cudaStream_t cs = nullptr;
+  cudaGraph_t graph = nullptr, body = nullptr;
   cudaStream_t saved = c->st;
-  cudaError_t e = cudaStreamSynchronize(saved);
-  c->st = cs;
   long long before = 0, after = 0;
-  rich_kernel_launches(&before);
-  cudaGraph_t graph = nullptr;
   int rc = RICH_OK;
-  if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+  cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(saved);
+  if (e == cudaSuccess) e = cudaGraphCreate(&graph, 0);
+  cudaGraphConditionalHandle loop;
+  if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&loop, graph, 1, cudaGraphCondAssignDefault);
   if (e == cudaSuccess) {
-    rc = fcg_iteration(c, x, q, qprev, false, true);
-    e = cudaStreamEndCapture(cs, &graph);
+    cudaGraphNodeParams np = {};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = loop;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    cudaGraphNode_t node;
+    e = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &np);
+    if (e == cudaSuccess) body = np.conditional.phGraph_out[0];
   }
-  c->st = saved;
-  rich_kernel_launches(&after);
-  count_launches(before - after);  // recorded, not launched
+  if (e == cudaSuccess)
+    e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    rich_kernel_launches(&before);
+    c->st = cs;
+    rc = fcg_body<T>(c, S, loop, 1);
+    c->st = saved;
+    rich_kernel_launches(&after);
+    count_launches(before - after);  // recorded, not launched
+    cudaGraph_t captured = nullptr;
+    e = cudaStreamEndCapture(cs, &captured);  // the body itself
+  }
   if (e == cudaSuccess && rc == RICH_OK) {
-    e = cudaGraphInstantiate(&H.fcg_exec[par], graph, 0);
-    if (e == cudaSuccess) H.fcg_nodes[par] = after - before;
-    else H.fcg_exec[par] = nullptr;
+    e = cudaGraphInstantiate(&H.fcg_exec, graph, 0);
+    if (e == cudaSuccess) H.fcg_nodes = after - before;
+    else H.fcg_exec = nullptr;
   }
   if (graph) cudaGraphDestroy(graph);
-  cudaStreamDestroy(cs);
-  if (e != cudaSuccess || rc != RICH_OK || !H.fcg_exec[par]) {
+  if (cs) cudaStreamDestroy(cs);
+  if (e != cudaSuccess || rc != RICH_OK || !H.fcg_exec) {
     cudaGetLastError();
+    H.fcg_exec = nullptr;
     H.fcg_off = true;
   }
 }
 
-// Notay's flexible CG (truncation 1).  With o->stall > 0 it gives up when a window
-// of kStallWindow iterations reduced the residual by less than that fraction.
-// From the second iteration on, an iteration is a graph replay where the V-cycle
-// may be (rich_amg_opts.graph): the same kernels on the same buffers.
-static int fcg(rich_ctx* c, const double* b, double* x, const rich_krylov_opts* o, rich_krylov_stats* st) {
+template <class T>
+static int fcg_solve(rich_ctx* c, int S, const double* b, double* x, const rich_krylov_opts* o) {
   KrylovWork& k = c->kw;
   Hierarchy& H = c->H;
-  long long n = c->g.n;
-  double* s = c->dsc;
-  RICH_CHECK(nrm2sq(c, b, n, s + 0));
-  double h[4];
-  RICH_CHECK(fetch_scalars(c, s, 1, h));
-  double bn = sqrt(h[0]);
-  st->res0 = bn;
-  st->res = bn;
-  st->iterations = 0;
-  st->converged = 0;
-  k.fail_reason = 0;
-  RICH_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * n, c->st));
-  if (!(bn > 0)) {
-    st->converged = std::isfinite(bn) ? 1 : 0;
-    return std::isfinite(bn) ? RICH_OK : RICH_ENONFINITE;
+  const long long n = c->g.n, ns = n / S;
+  if (!k.fcg) {
+    FcgDev* d = nullptr;
+    RICH_CHECK(dalloc(&d, 1));
+    k.fcg = d;
   }
-  if (!std::isfinite(bn)) return RICH_ENONFINITE;
-  RICH_CUDA(cudaMemcpyAsync(k.r, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
-  double target = o->eta * bn, best = bn, window_start = bn;
-  double* q = k.q;
-  double* qprev = k.qprev;
-  const bool graphs = vcycle_graphable(c) && !H.fcg_off && (!H.fcg_x || H.fcg_x == x);
-  for (int it = 1; it <= o->maxit; ++it) {
-    bool replayed = false;
-    if (graphs && it >= 2 && H.vc_calls > 0 && !H.fcg_off) {
-      const int par = it & 1;  // it even: q = k.qprev, q_prev = k.q; odd: the other way round
-      if (!H.fcg_exec[par]) {
-        H.fcg_x = x;
-        fcg_capture(c, par, x, q, qprev);
-      }
-      if (H.fcg_exec[par]) {
-        RICH_CUDA(cudaGraphLaunch(H.fcg_exec[par], c->st));
-        count_launches(H.fcg_nodes[par]);
-        replayed = true;
+  if (!k.fcg_out && !(k.fcg_out = pinned_get())) return RICH_ENOMEM;
+  const FcgOut* out = static_cast<const FcgOut*>(k.fcg_out);
+  k_fcg_begin<T><<<dim3(fcg_blocks(ns, S), S), kFcgThreads, 0, c->st>>>(
+      ns, b, k.x, k.r, scaled<T>(c).s, vcycle_rhs<T>(c), o->eta, o->stall, o->maxit, static_cast<FcgDev*>(k.fcg),
+      c->partials, c->ticket, static_cast<FcgOut*>(k.fcg_out));
+  RICH_LAUNCH_CHECK();
+  auto running = [&]() {
+    bool any = false;
+    for (int s = 0; s < S; ++s) {
+      if (out[s].reason == kFcgNonfinite) return false;
+      any = any || out[s].reason == 0;
+    }
+    return any;
+  };
+  const bool graphs = vcycle_graphable(c) && !H.fcg_off;
+  bool waited = false;
+  for (;;) {
+    if (graphs && !H.fcg_off && H.vc_calls > 0) {  // a first application launched directly
+      if (waited && !running()) break;
+      if (!H.fcg_exec) fcg_capture<T>(c, S);
+      if (H.fcg_exec) {
+        const int it0 = waited ? out[0].it : 0;
+        RICH_CUDA(cudaGraphLaunch(H.fcg_exec, c->st));
+        RICH_CUDA(cudaStreamSynchronize(c->st));
+        int most = 1;
+        for (int s = 0; s < S; ++s) most = std::max(most, out[s].it - it0);
+        count_launches(most * H.fcg_nodes);
+        break;
       }
     }
-    if (!replayed) RICH_CHECK(fcg_iteration(c, x, q, qprev, it == 1, false));
+    if (!waited) RICH_CUDA(cudaStreamSynchronize(c->st));
+    waited = true;
+    if (!running()) break;
+    ++H.vc_calls;
+    RICH_CHECK(fcg_body<T>(c, S, cudaGraphConditionalHandle(0), 0));
     RICH_CUDA(cudaStreamSynchronize(c->st));
-    for (int i = 0; i < 3; ++i) h[i] = c->hsc[i];
-    double rn = sqrt(h[0]);
-    st->iterations = it;
-    st->res = rn;
-    if (!std::isfinite(rn) || !std::isfinite(h[2])) return RICH_ENONFINITE;
-    if (!(h[2] > 0)) {
-      k.fail_reason = 2;
-      return RICH_ENOTCONV_LIN;
-    }
-    if (rn <= target) {
-      st->converged = 1;
-      return RICH_OK;
-    }
-    if (rn > 10.0 * best) {
-      k.fail_reason = 3;
-      return RICH_ENOTCONV_LIN;
-    }
-    if (it % kStallWindow == 0) {  // stagnation over the last window
-      if (o->stall > 0 && rn > (1.0 - o->stall) * window_start) {
-        k.fail_reason = 4;
-        return RICH_ENOTCONV_LIN;
-      }
-      window_start = rn;
-    }
-    best = std::min(best, rn);
-    std::swap(q, qprev);
   }
-  k.fail_reason = 1;
-  return RICH_ENOTCONV_LIN;
+  RICH_CUDA(cudaMemcpyAsync(x, k.x, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->st));
+  return RICH_OK;
+}
+
+// S problems' solves of J x = b from x = 0; per problem the iterations, ||b||, the last
+// ||r|| and the reason it stopped (0 converged, else KrylovWork::fail_reason's codes).
+// RICH_ENONFINITE if any problem met a non-finite scalar.
+int fcg_run(rich_ctx* c, int S, const double* b, double* x, const rich_krylov_opts* o, FcgResult* res) {
+  RICH_CHECK(c->prec == RICH_PREC_MIXED ? fcg_solve<float>(c, S, b, x, o) : fcg_solve<double>(c, S, b, x, o));
+  const FcgOut* out = static_cast<const FcgOut*>(c->kw.fcg_out);
+  int rc = RICH_OK;
+  for (int s = 0; s < S; ++s) {
+    res[s] = FcgResult{out[s].rn, out[s].bn, out[s].it,
+                       out[s].reason == kFcgConverged || out[s].reason == kFcgZero ? 0 : out[s].reason};
+    if (out[s].reason == kFcgNonfinite) rc = RICH_ENONFINITE;
+  }
+  return rc;
+}
+
+static int fcg(rich_ctx* c, const double* b, double* x, const rich_krylov_opts* o, rich_krylov_stats* st) {
+  FcgResult r{};
+  const int rc = fcg_run(c, 1, b, x, o, &r);
+  st->res0 = r.bn;
+  st->res = r.rn;
+  st->iterations = r.it;
+  st->converged = rc == RICH_OK && r.reason == 0;
+  if (rc != RICH_OK) return rc;
+  c->kw.fail_reason = r.reason;
+  return r.reason == 0 ? RICH_OK : RICH_ENOTCONV_LIN;
 }
 
 // V = f src (f = *fdev if given), z = M V.
