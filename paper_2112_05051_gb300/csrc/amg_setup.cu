@@ -19,6 +19,8 @@
 // patterns with one thread per row in the same product order.
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace rich {
@@ -93,6 +95,37 @@ __global__ void k_strength(int n, const int* __restrict__ rp, const int* __restr
     }
     if (cnt) cnt[i] = c;
   }
+}
+
+// The same with a warp per row, for rows of more than a few entries (a thread per row walks
+// 100 entries, each with a search in another row, one after another: 590 us for 1400 rows).
+__global__ void k_strength_warp(int n, const int* __restrict__ rp, const int* __restrict__ col,
+                                const double* __restrict__ val, const double* __restrict__ d, double theta2,
+                                const int* __restrict__ srp, int* __restrict__ cnt, int* __restrict__ scol) {
+  const int lane = threadIdx.x & 31;
+  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += (gridDim.x * blockDim.x) >> 5) {
+    const int o = srp ? srp[i] : 0, e1 = rp[i + 1];
+    int c = 0;
+    for (int e0 = rp[i]; e0 < e1; e0 += 32) {
+      const int e = e0 + lane;
+      const bool s = e < e1 && strong_sym(i, e, rp, col, val, d, theta2);
+      const unsigned m = __ballot_sync(0xffffffffu, s);
+      if (s && scol) scol[o + c + __popc(m & ((1u << lane) - 1))] = col[e];
+      c += __popc(m);
+    }
+    if (cnt && lane == 0) cnt[i] = c;
+  }
+}
+
+static int strength(rich_ctx* c, const Csr<double>& A, const double* d, double theta2, const int* srp, int* cnt,
+                    int* scol) {
+  const int n = A.nrows;
+  if (A.nnz > 12LL * n)
+    k_strength_warp<<<grid_for(32LL * n), kBlock, 0, c->st>>>(n, A.rowptr, A.col, A.val, d, theta2, srp, cnt, scol);
+  else
+    k_strength<<<grid_for(n), kBlock, 0, c->st>>>(n, A.rowptr, A.col, A.val, d, theta2, srp, cnt, scol);
+  RICH_LAUNCH_CHECK();
+  return RICH_OK;
 }
 
 // Isolated nodes (no strong neighbour) start OUT: they join no aggregate.
@@ -411,6 +444,135 @@ __global__ void k_spgemm_esc(int nrows, const int* __restrict__ arp, const int* 
   }
 }
 
+// The same for products with fewer than 2^kSortCol columns: keys of 32 bits (column, product
+// index), sorted in registers.  A lane holds K consecutive keys, so that the network's
+// short distances are register exchanges and the long ones shuffles; the products of 32 A
+// entries at a time are spread over the lanes through a scan of their B rows' lengths, so
+// that the loads of a row are in flight together.  Sums, order and results are k_spgemm_esc's.
+// 64^3, A_1 P_1 (29k rows, 210 products on average): 1480 us in shared memory with 64-bit
+// keys, 16 kB per warp and one A entry after another.
+constexpr int kSortCol = 22, kSortIdx = 32 - kSortCol;
+static_assert((1 << kSortIdx) >= kEscCap, "a product index fits beside the column");
+
+template <int K>
+__device__ __forceinline__ void warp_sort_keys(unsigned* keys, int u, int lane) {
+  unsigned a[K];
+#pragma unroll
+  for (int r = 0; r < K; ++r) a[r] = lane * K + r < u ? keys[lane * K + r] : 0xffffffffu;
+#pragma unroll
+  for (int k = 2; k <= 32 * K; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      if (j >= K) {
+        const bool keep_min = ((lane & (j / K)) == 0) == ((lane & (k / K)) == 0);
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+          const unsigned o = __shfl_xor_sync(0xffffffffu, a[r], j / K);
+          a[r] = keep_min ? min(a[r], o) : max(a[r], o);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < K; ++r)
+          if ((r & j) == 0) {
+            const bool asc = k < K ? (r & k) == 0 : (lane & (k / K)) == 0;
+            const unsigned lo = min(a[r], a[r ^ j]), hi = max(a[r], a[r ^ j]);
+            a[r] = asc ? lo : hi;
+            a[r ^ j] = asc ? hi : lo;
+          }
+      }
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int r = 0; r < K; ++r)
+    if (lane * K + r < u) keys[lane * K + r] = a[r];
+  __syncwarp();
+}
+
+// Rows with umin < products <= cap (cap slots of shared memory per warp).
+__global__ void __launch_bounds__(256) k_spgemm_sort(int nrows, const int* __restrict__ arp,
+                                                     const int* __restrict__ acol, const double* __restrict__ aval,
+                                                     const int* __restrict__ brp, const int* __restrict__ bcol,
+                                                     const double* __restrict__ bval, const int* __restrict__ u,
+                                                     int mode, const int* __restrict__ crp,
+                                                     const long long* __restrict__ uoff, int* __restrict__ ccol,
+                                                     double* __restrict__ cval, int* __restrict__ cnt, int umin,
+                                                     int cap) {
+  extern __shared__ __align__(8) unsigned char smem[];
+  __shared__ int pre_all[8][33], bst_all[8][32];
+  __shared__ double av_all[8][32];
+  const int wpb = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* vals = reinterpret_cast<double*>(smem) + (size_t)w * cap;
+  unsigned* keys = reinterpret_cast<unsigned*>(smem + (size_t)wpb * cap * sizeof(double)) + (size_t)w * cap;
+  int *pre = pre_all[w], *bst = bst_all[w];
+  double* av = av_all[w];
+  for (int row = blockIdx.x * wpb + w; row < nrows; row += gridDim.x * wpb) {
+    const int ur = u[row];
+    if (ur > cap || ur <= umin) {
+      if (ur == 0 && umin == 0 && mode != 1 && lane == 0) cnt[row] = 0;
+      continue;
+    }
+    // expand in product order: A entries in column order, then B entries in column order
+    int t0 = 0;
+    const int a1 = arp[row + 1];
+    for (int e0 = arp[row]; e0 < a1; e0 += 32) {
+      const int e = e0 + lane;
+      const bool has = e < a1;
+      const int j = has ? acol[e] : 0;
+      const int b0 = has ? brp[j] : 0, len = has ? brp[j + 1] - b0 : 0;
+      int inc = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      const int total = __shfl_sync(0xffffffffu, inc, 31);
+      pre[lane + 1] = inc;
+      if (lane == 0) pre[0] = 0;
+      bst[lane] = b0;
+      av[lane] = has && aval ? aval[e] : 1.0;
+      __syncwarp();
+      for (int p = lane; p < total; p += 32) {
+        int lo = 0, hi = 32;  // owner q of product p: pre[q] <= p < pre[q+1]
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (pre[mid] <= p) lo = mid; else hi = mid;
+        }
+        const int f = bst[lo] + (p - pre[lo]);
+        keys[t0 + p] = (unsigned)bcol[f] << kSortIdx | (unsigned)(t0 + p);
+        vals[t0 + p] = av[lo] * (bval ? bval[f] : 1.0);
+      }
+      t0 += total;
+      __syncwarp();
+    }
+    if (ur <= 32) warp_sort_keys<1>(keys, ur, lane);
+    else if (ur <= 64) warp_sort_keys<2>(keys, ur, lane);
+    else if (ur <= 128) warp_sort_keys<4>(keys, ur, lane);
+    else if (ur <= 256) warp_sort_keys<8>(keys, ur, lane);
+    else if (ur <= 512) warp_sort_keys<16>(keys, ur, lane);
+    else warp_sort_keys<32>(keys, ur, lane);
+    // segment heads
+    const long long base = mode == 1 ? (long long)crp[row] : (mode == 2 ? uoff[row] : 0);
+    int running = 0;
+    for (int s0 = 0; s0 < ur; s0 += 32) {
+      const int t = s0 + lane;
+      const unsigned c = t < ur ? keys[t] >> kSortIdx : 0u;
+      const bool head = t < ur && (t == 0 || keys[t - 1] >> kSortIdx != c);
+      const unsigned mask = __ballot_sync(0xffffffffu, head);
+      if (mode != 0 && head) {
+        const long long pos = base + running + __popc(mask & ((1u << lane) - 1));
+        double s = 0.0;
+        for (int q = t; q < ur && keys[q] >> kSortIdx == c; ++q) s += vals[keys[q] & ((1u << kSortIdx) - 1)];
+        ccol[pos] = (int)c;
+        cval[pos] = s;
+      }
+      running += __popc(mask);
+    }
+    if (mode != 1 && lane == 0) cnt[row] = running;
+    __syncwarp();
+  }
+}
+
 // Rows with more than kEscCap products: one block per row accumulates the products
 // into a shared-memory hash table keyed by column (linear probing, atomicCAS), then
 // sorts the occupied keys.  The column set is exact; the FP64 sums depend on the
@@ -428,6 +590,8 @@ __global__ void __launch_bounds__(kHashThreads) k_spgemm_hash(
   double* hval = reinterpret_cast<double*>(smem + kHashSlots * sizeof(int));
   __shared__ int nfill;
   __shared__ int fail;
+  __shared__ int pre[kHashThreads + 1], bst[kHashThreads], wsum[kHashThreads / 32];
+  __shared__ double av[kHashThreads];
   for (int row = blockIdx.x; row < nrows; row += gridDim.x) {
     if (u[row] <= kEscCap) continue;
     for (int t = threadIdx.x; t < kHashSlots; t += blockDim.x) {
@@ -439,13 +603,39 @@ __global__ void __launch_bounds__(kHashThreads) k_spgemm_hash(
       fail = 0;
     }
     __syncthreads();
-    // products: A entries of the row in turn, B entries strided over the block
-    for (int e = arp[row]; e < arp[row + 1]; ++e) {
-      int j = acol[e];
-      double a = aval ? aval[e] : 1.0;
-      for (int f = brp[j] + threadIdx.x; f < brp[j + 1]; f += blockDim.x) {
+    // products of 256 A entries at a time, spread over the block through a scan of their B
+    // rows' lengths (one A entry after another left most threads idle: 1270 us for 1400 rows)
+    for (int e0 = arp[row]; e0 < arp[row + 1]; e0 += kHashThreads) {
+      const int e = e0 + threadIdx.x;
+      const bool has = e < arp[row + 1];
+      const int j = has ? acol[e] : 0;
+      const int b0 = has ? brp[j] : 0, len = has ? brp[j + 1] - b0 : 0;
+      const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+      int inc = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      if (lane == 31) wsum[wid] = inc;
+      bst[threadIdx.x] = b0;
+      av[threadIdx.x] = has && aval ? aval[e] : 1.0;
+      __syncthreads();
+      int add = 0;
+      for (int q = 0; q < wid; ++q) add += wsum[q];
+      pre[threadIdx.x + 1] = inc + add;
+      if (threadIdx.x == 0) pre[0] = 0;
+      __syncthreads();
+      const int total = pre[kHashThreads];
+      for (int p = threadIdx.x; p < total; p += blockDim.x) {
+        int lo = 0, hi = kHashThreads;
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (pre[mid] <= p) lo = mid; else hi = mid;
+        }
+        const int f = bst[lo] + (p - pre[lo]);
         int col = bcol[f];
-        double v = a * (bval ? bval[f] : 1.0);
+        double v = av[lo] * (bval ? bval[f] : 1.0);
         unsigned h = ((unsigned)col * 2654435761u) & (kHashSlots - 1);
         int probes = 0;
         for (;;) {
@@ -463,8 +653,8 @@ __global__ void __launch_bounds__(kHashThreads) k_spgemm_hash(
         }
         if (probes < kHashSlots) atomicAdd(&hval[h], v);
       }
+      __syncthreads();
     }
-    __syncthreads();
     if (fail) {
       if (threadIdx.x == 0) atomicOr(overflow, 1);
       __syncthreads();
@@ -750,6 +940,7 @@ __global__ void __launch_bounds__(kNumThreads) k_spgemm_numeric_block(
 // or files each pair into its C entry's segment; k_plist_sort then orders each
 // segment by A entry, which is the order a row-by-row product sums in.
 constexpr int kPlWarps = 8;
+constexpr int kPlCols = 512;  // columns of a C row searched in shared memory
 
 template <bool FILL>
 __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* __restrict__ arp,
@@ -761,12 +952,17 @@ __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* _
                                                          int* __restrict__ pb) {
   __shared__ int pre_all[kPlWarps][33];
   __shared__ int bst_all[kPlWarps][32];
+  __shared__ int col_all[kPlWarps][kPlCols];
   int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int* pre = pre_all[w];
   int* bst = bst_all[w];
+  int* scol = col_all[w];
   int nw = gridDim.x * kPlWarps;
   for (int row = blockIdx.x * kPlWarps + w; row < nrows; row += nw) {
     int c0 = crp[row], c1 = crp[row + 1];
+    const bool staged = c1 - c0 <= kPlCols;  // eight dependent L2 loads per product otherwise
+    if (staged)
+      for (int t = lane; t < c1 - c0; t += 32) scol[t] = ccol[c0 + t];
     int a1 = arp[row + 1];
     for (int e0 = arp[row]; e0 < a1; e0 += 32) {
       int e = e0 + lane;
@@ -792,7 +988,7 @@ __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* _
           if (pre[mid] <= t) lo = mid; else hi = mid;
         }
         int f = bst[lo] + (t - pre[lo]);
-        int q = find_col(ccol, c0, c1, bcol[f]);
+        int q = staged ? c0 + find_col(scol, 0, c1 - c0, bcol[f]) : find_col(ccol, c0, c1, bcol[f]);
         int slot = atomicAdd(&cnt[q], 1);
         if (FILL) {
           long long at = base[q >> kPlShift] + seg[q] + slot;
@@ -1142,6 +1338,7 @@ static int spgemm_symbolic(rich_ctx* c, const Csr<double>& A, const Csr<double>&
   RICH_CUDA(cudaStreamSynchronize(c->st));
   size_t mfree = 0, mtotal = 0;
   RICH_CUDA(cudaMemGetInfo(&mfree, &mtotal));
+  mfree += pool_slack();
   const bool one_pass = (double)nprod * (sizeof(int) + sizeof(double)) <= 0.25 * (double)mfree;
   int* tcol = nullptr;
   double* tval = nullptr;
@@ -1176,9 +1373,20 @@ static int spgemm_symbolic(rich_ctx* c, const Csr<double>& A, const Csr<double>&
     }
     int* ocol = mode == 2 ? tcol : C.col;
     double* oval = mode == 2 ? tval : C.val;
-    k_spgemm_esc<<<nblk, 32 * esc_warps, smem, c->st>>>(n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, u, mode,
-                                                       C.rowptr, uoff, ocol, oval, cnt, cap);
-    RICH_LAUNCH_CHECK();
+    if (B.ncols < (1 << kSortCol)) {
+      // rows of up to 256 products with 3 kB of shared memory per warp, the others apart
+      for (int umin = 0; umin < cap; umin = umin ? cap : 256) {
+        const int cp = umin ? cap : std::min(cap, 256), wpb = cp <= 256 ? 8 : cp <= 512 ? 4 : 2;
+        const int nblk2 = std::min((n + wpb - 1) / wpb, 64 * kNumSM);
+        k_spgemm_sort<<<nblk2, 32 * wpb, (size_t)wpb * cp * (sizeof(double) + sizeof(unsigned)), c->st>>>(
+            n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, u, mode, C.rowptr, uoff, ocol, oval, cnt, umin, cp);
+        RICH_LAUNCH_CHECK();
+      }
+    } else {
+      k_spgemm_esc<<<nblk, 32 * esc_warps, smem, c->st>>>(n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, u, mode,
+                                                         C.rowptr, uoff, ocol, oval, cnt, cap);
+      RICH_LAUNCH_CHECK();
+    }
     if (big) {
       int hb = n < 8 * kNumSM ? n : 8 * kNumSM;
       k_spgemm_hash<<<hb, kHashThreads, hsmem, c->st>>>(n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, u, mode,
@@ -1192,7 +1400,6 @@ static int spgemm_symbolic(rich_ctx* c, const Csr<double>& A, const Csr<double>&
   dfree(tcol);
   dfree(tval);
   dfree(uoff);
-  RICH_CUDA(cudaStreamSynchronize(c->st));
   if (u_keep) *u_keep = u; else dfree(u);
   dfree(cnt);
   return RICH_OK;
@@ -1228,9 +1435,8 @@ static int plist_build(rich_ctx* c, const Csr<double>& A, const Csr<double>& B, 
   RICH_CUDA(cudaMemcpyAsync(&np, dsum, sizeof(np), cudaMemcpyDeviceToHost, c->st));
   RICH_CUDA(cudaStreamSynchronize(c->st));
   size_t fr = 0, tot = 0;
-  RICH_CUDA(cudaStreamSynchronize(c->st));
-  pool_trim();  // blocks freed into the pool count as free here
   RICH_CUDA(cudaMemGetInfo(&fr, &tot));
+  fr += pool_slack();  // blocks freed into the pool count as free here
   double need = 8.0 * (double)np + 24.0 * ((double)C.nnz + 1);  // lists, offsets and the build's scratch
   if (need > 0.5 * (double)fr) return RICH_OK;
   int* cnt = nullptr;
@@ -1257,7 +1463,6 @@ static int plist_build(rich_ctx* c, const Csr<double>& A, const Csr<double>& B, 
   RICH_LAUNCH_CHECK();
   k_plist_sort<<<grid_for(C.nnz), kBlock, 0, c->st>>>(C.nnz, pl.seg, pl.base, pl.pa, pl.pb);
   RICH_LAUNCH_CHECK();
-  RICH_CUDA(cudaStreamSynchronize(c->st));
   dfree(cnt);
   dfree(segll);
   return RICH_OK;
@@ -1768,15 +1973,13 @@ static int coarsen(rich_ctx* c, int l, bool* stop) {
   } else {
     double theta_l = o.theta * std::ldexp(1.0, -l);
     double theta2 = theta_l * theta_l;
-    k_strength<<<grid_for(n), kBlock, 0, c->st>>>(n, L.A.rowptr, L.A.col, L.A.val, d, theta2, nullptr, cnt, nullptr);
-    RICH_LAUNCH_CHECK();
+    RICH_CHECK(strength(c, L.A, d, theta2, nullptr, cnt, nullptr));
     RICH_CHECK(dalloc(&S.rowptr, (long long)n + 1));
     RICH_CHECK(scan_exclusive_int(c, cnt, S.rowptr, n));
     int snnz = 0;
     RICH_CHECK(read_dev_int(c, S.rowptr + n, &snnz));
     RICH_CHECK(dalloc(&S.col, snnz));
-    k_strength<<<grid_for(n), kBlock, 0, c->st>>>(n, L.A.rowptr, L.A.col, L.A.val, d, theta2, S.rowptr, nullptr, S.col);
-    RICH_LAUNCH_CHECK();
+    RICH_CHECK(strength(c, L.A, d, theta2, S.rowptr, nullptr, S.col));
     // MIS-2
     uint64_t *t = nullptr, *m1 = nullptr;
     RICH_CHECK(dalloc(&t, n));

@@ -37,6 +37,17 @@ void pool_trim() {
   cudaMemPoolTrimTo(pool, 0);
 }
 
+size_t pool_slack() {
+  int dev = 0;
+  cudaMemPool_t pool;
+  uint64_t reserved = 0, used = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetDefaultMemPool(&pool, dev) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+    return 0;
+  return reserved > used ? (size_t)(reserved - used) : 0;
+}
+
 static std::mutex g_pinned_mu;
 static std::vector<void*> g_pinned_free;
 
@@ -300,8 +311,7 @@ static int scan_impl(rich_ctx* c, const TI* in, TO* out, long long n) {
   RICH_LAUNCH_CHECK();
   k_scan_apply<TI, TO><<<(int)nt, kBlock, 0, c->st>>>(in, n, sums, out);
   RICH_LAUNCH_CHECK();
-  RICH_CUDA(cudaStreamSynchronize(c->st));
-  dfree(sums);
+  dfree(sums);  // stream-ordered: after the scan
   return RICH_OK;
 }
 

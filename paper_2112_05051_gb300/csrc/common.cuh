@@ -519,6 +519,7 @@ struct AllocStream {
 };
 void pool_setup();         // keeps freed device memory in the current device's pool
 void pool_trim();          // returns the pool's unused memory (before free-memory queries)
+size_t pool_slack();       // bytes the pool holds beyond what is in use
 void* pinned_get();        // a 2 KB pinned host block from a process-wide free list
 void pinned_put(void* b);  // back to the list (never cudaFreeHost: that synchronises the device)
 constexpr size_t kPinnedBlock = 2048;
