@@ -942,7 +942,9 @@ __global__ void __launch_bounds__(kNumThreads) k_spgemm_numeric_block(
 constexpr int kPlWarps = 8;
 constexpr int kPlCols = 512;  // columns of a C row searched in shared memory
 
-template <bool FILL>
+// WIDE: a block per row (rows of thousands of products), its warps taking the row's A
+// entries in turn; the order within a segment is settled by k_plist_sort either way.
+template <bool FILL, bool WIDE>
 __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* __restrict__ arp,
                                                          const int* __restrict__ acol, const int* __restrict__ brp,
                                                          const int* __restrict__ bcol, const int* __restrict__ crp,
@@ -956,15 +958,18 @@ __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* _
   int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int* pre = pre_all[w];
   int* bst = bst_all[w];
-  int* scol = col_all[w];
-  int nw = gridDim.x * kPlWarps;
-  for (int row = blockIdx.x * kPlWarps + w; row < nrows; row += nw) {
+  int* scol = WIDE ? col_all[0] : col_all[w];
+  int nw = WIDE ? gridDim.x : gridDim.x * kPlWarps;
+  for (int row = WIDE ? blockIdx.x : blockIdx.x * kPlWarps + w; row < nrows; row += nw) {
     int c0 = crp[row], c1 = crp[row + 1];
-    const bool staged = c1 - c0 <= kPlCols;  // eight dependent L2 loads per product otherwise
+    // eight dependent L2 loads per product otherwise
+    const bool staged = c1 - c0 <= (WIDE ? kPlCols * kPlWarps : kPlCols);
+    if (WIDE) __syncthreads();  // the row before this one is done with the columns
     if (staged)
-      for (int t = lane; t < c1 - c0; t += 32) scol[t] = ccol[c0 + t];
+      for (int t = WIDE ? threadIdx.x : lane; t < c1 - c0; t += WIDE ? 32 * kPlWarps : 32) scol[t] = ccol[c0 + t];
+    if (WIDE) __syncthreads();
     int a1 = arp[row + 1];
-    for (int e0 = arp[row]; e0 < a1; e0 += 32) {
+    for (int e0 = arp[row] + (WIDE ? 32 * w : 0); e0 < a1; e0 += WIDE ? 32 * kPlWarps : 32) {
       int e = e0 + lane;
       bool has = e < a1;
       int j = has ? acol[e] : 0;
@@ -1035,6 +1040,49 @@ __global__ void k_plist_sort(int nnz, const int* __restrict__ seg, const long lo
   }
 }
 
+// The same for long segments, a warp each: up to kPlSort pairs are ranked in shared memory
+// (an A entry contributes one product to an entry of C, so the keys are distinct).
+constexpr int kPlSort = 512;
+__global__ void __launch_bounds__(32 * kPlWarps) k_plist_rank(int nnz, const int* __restrict__ seg,
+                                                              const long long* __restrict__ base,
+                                                              int* __restrict__ pa, int* __restrict__ pb) {
+  __shared__ int a_all[kPlWarps][kPlSort], b_all[kPlWarps][kPlSort];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int *a = a_all[w], *b = b_all[w];
+  for (int q = blockIdx.x * kPlWarps + w; q < nnz; q += gridDim.x * kPlWarps) {
+    const long long s0 = plist_start(seg, base, q);
+    const int len = (int)(plist_start(seg, base, q + 1) - s0);
+    if (len < 2) continue;
+    if (len > kPlSort) {
+      if (lane == 0)
+        for (long long t = s0 + 1; t < s0 + len; ++t) {
+          const int ka = pa[t], kb = pb[t];
+          long long v = t - 1;
+          for (; v >= s0 && pa[v] > ka; --v) {
+            pa[v + 1] = pa[v];
+            pb[v + 1] = pb[v];
+          }
+          pa[v + 1] = ka;
+          pb[v + 1] = kb;
+        }
+      continue;
+    }
+    for (int t = lane; t < len; t += 32) {
+      a[t] = pa[s0 + t];
+      b[t] = pb[s0 + t];
+    }
+    __syncwarp();
+    for (int t = lane; t < len; t += 32) {
+      const int k = a[t];
+      int r = 0;
+      for (int v = 0; v < len; ++v) r += a[v] < k;
+      pa[s0 + r] = k;
+      pb[s0 + r] = b[t];
+    }
+    __syncwarp();
+  }
+}
+
 __global__ void k_sum_rows_ll(int n, const int* __restrict__ u, unsigned long long* __restrict__ out) {
   unsigned long long s = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) s += (unsigned)u[i];
@@ -1063,58 +1111,96 @@ __global__ void __launch_bounds__(256) k_galerkin_lists(int nnz, const int* __re
 
 // ---------------------------------------------------------------- coarsest level: dense inverse
 
+// Entries of a CSR matrix into a zeroed dense one, a warp per row.
 template <class T>
 __global__ void k_csr_to_dense(int n, const int* __restrict__ rp, const int* __restrict__ col,
                                const T* __restrict__ val, double* __restrict__ dense) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    for (int j = 0; j < n; ++j) dense[(long long)i * n + j] = 0.0;
-    for (int e = rp[i]; e < rp[i + 1]; ++e) dense[(long long)i * n + col[e]] = (double)val[e];
-  }
+  const int lane = threadIdx.x & 31;
+  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += (gridDim.x * blockDim.x) >> 5)
+    for (int e = rp[i] + lane; e < rp[i + 1]; e += 32) dense[(long long)i * n + col[e]] = (double)val[e];
 }
 
 // Blocked Gauss-Jordan inversion in place (no pivoting: the matrix is SPD).
 // For a panel P of kGjB consecutive pivots and the other indices O, one block
 // step turns [[A_PP, A_PO], [A_OP, A_OO]] into
 //   [[A_PP^-1, A_PP^-1 A_PO], [-A_OP A_PP^-1, A_OO - A_OP A_PP^-1 A_PO]];
-// after every panel the matrix holds A^-1.  Three launches per panel:
-// k_gj_panel inverts A_PP in shared memory; k_gj_rows forms the new panel rows
-// and saves the old panel columns; k_gj_update applies the rank-kGjB update as
-// a shared-memory tiled product.  Work buffer (2 kGjB n + kGjB^2 doubles):
-// R[p][j] (new panel rows; for j in P the panel inverse), C[p][i] (old panel
-// columns), Pinv (kGjB x kGjB).
+// after every panel the matrix holds A^-1.  The matrix being symmetric, every step leaves
+// a_ij = a_ji where both indices or neither has been a pivot and a_ij = -a_ji otherwise, so
+// only the tiles on and above the diagonal are computed (n^3 / 2 multiply-adds instead of
+// n^3) and mirrored; the upper triangle is what is inverted.  Two launches per panel:
+// k_gj_rows forms the new panel rows (and their mirror), k_gj_update applies the rank-kGjB
+// update, and its block on the next diagonal tile inverts that tile while the others are
+// still at work.  Work buffer (2 kGjB n + kGjB^2 doubles): R[p][j] (new panel rows),
+// C[p][i] (old panel columns), Pinv (kGjB x kGjB).
+// Bound: FP64 multiply-adds for large n, the chain of pivots for small n.  n = 362: 713 us
+// with full tiles, three launches per panel and a 42 us panel inversion.
 constexpr int kGjB = 32;
+constexpr int kGjInvWarps = 8;
 
-__global__ void __launch_bounds__(kGjB* kGjB) k_gj_panel(int n, int K, int bs, double* __restrict__ a,
-                                                        double* __restrict__ pinv) {
-  __shared__ double m[kGjB][kGjB + 1];
-  __shared__ double rowk[kGjB], colk[kGjB];  // pivot row, and pivot column scaled by 1/pivot
-  __shared__ double inv;
-  const int r = threadIdx.y, q = threadIdx.x;  // element (r, q) of the bs x bs panel block
-  const bool in = r < bs && q < bs;
-  if (in) m[r][q] = a[(long long)(K + r) * n + K + q];
-  __syncthreads();
-  for (int k = 0; k < bs; ++k) {
-    if (r == 0 && q == 0) inv = 1.0 / m[k][k];  // the step's one division
-    if (in && r == k) rowk[q] = m[k][q];
-    __syncthreads();
-    if (in && q == k) colk[r] = m[r][k] * inv;
-    __syncthreads();
-    if (in) {
-      double v;
-      if (r == k) v = (q == k) ? inv : rowk[q] * inv;
-      else if (q == k) v = -colk[r];
-      else v = fma(-colk[r], rowk[q], m[r][q]);
-      m[r][q] = v;
-    }
-    __syncthreads();
+// Inverse of the bs x bs block m by Gauss-Jordan in registers, by the first 8 warps of a
+// block: warp w holds rows w, w + 8, w + 16, w + 24, a lane per column.  Per pivot the
+// owner scales its row, one barrier publishes it (double buffer), and every other row takes
+// one multiply-add; a column's factor comes from the pivot's lane by a shuffle.
+__device__ __forceinline__ void gj_invert(double (*m)[kGjB + 1], int bs, double (*rk)[kGjB]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double v[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int r = w + 8 * t;
+    v[t] = r < bs && lane < bs ? m[r][lane] : (r == lane ? 1.0 : 0.0);
   }
-  if (in) a[(long long)(K + r) * n + K + q] = m[r][q];
-  pinv[r * kGjB + q] = in ? m[r][q] : 0.0;  // zeros outside a partial last panel
+#pragma unroll
+  for (int t0 = 0; t0 < 4; ++t0) {
+    for (int kk = 0; kk < 8; ++kk) {
+      const int k = 8 * t0 + kk;
+      if (k >= bs) break;
+      double* row = rk[k & 1];
+      if (w == kk) {
+        const double inv = safe_rcp(__shfl_sync(0xffffffffu, v[t0], k));
+        v[t0] = lane == k ? inv : v[t0] * inv;
+        row[lane] = v[t0];
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      const double q = row[lane];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const double f = __shfl_sync(0xffffffffu, v[t], k);
+        if (w + 8 * t != k) v[t] = fma(-f, q, lane == k ? 0.0 : v[t]);
+      }
+    }
+  }
+  asm volatile("bar.sync 1, 256;" ::: "memory");
+#pragma unroll
+  for (int t = 0; t < 4; ++t) m[w + 8 * t][lane] = v[t];
+  asm volatile("bar.sync 1, 256;" ::: "memory");
 }
 
-// Columns j0 .. j0+7 per block, thread (p, jj): R[p][j] = (Pinv A_P,j)_p written
-// back to panel row p (j outside P), or the panel inverse's entry (j in P); the
-// same thread saves row i = j's old panel entry C[p][i] = a_i,K+p (i outside P).
+// Inverse of the panel block at K: into the matrix and Pinv (zeros outside a partial block).
+__device__ __forceinline__ void gj_store_panel(double (*m)[kGjB + 1], int n, int K, int bs, double* __restrict__ a,
+                                               double* __restrict__ pinv) {
+  for (int t = threadIdx.x; t < kGjB * kGjB; t += 32 * kGjInvWarps) {
+    const int r = t / kGjB, q = t % kGjB;
+    const bool in = r < bs && q < bs;
+    if (in) a[(long long)(K + r) * n + K + q] = m[r][q];
+    pinv[t] = in ? m[r][q] : 0.0;
+  }
+}
+
+__global__ void __launch_bounds__(32 * kGjInvWarps) k_gj_panel(int n, int bs, double* __restrict__ a,
+                                                              double* __restrict__ pinv) {
+  __shared__ double m[kGjB][kGjB + 1], rk[2][kGjB];
+  for (int t = threadIdx.x; t < kGjB * kGjB; t += 32 * kGjInvWarps) {
+    const int r = t / kGjB, q = t % kGjB;
+    m[r][q] = r < bs && q < bs ? a[(long long)min(r, q) * n + max(r, q)] : 0.0;
+  }
+  __syncthreads();
+  gj_invert(m, bs, rk);
+  gj_store_panel(m, n, 0, bs, a, pinv);
+}
+
+// Columns j0 .. j0+7 per block, thread (p, jj): R[p][j] = (Pinv A_P,j)_p to panel row p and,
+// mirrored, to column p; C[p][j] = a_j,K+p before the step (a_K+p,j, negated for an earlier
+// pivot j).  Columns in P take zeros (the panel itself is done).
 constexpr int kGjCols = 8;
 
 __global__ void __launch_bounds__(kGjB* kGjCols) k_gj_rows(int n, int K, int bs, double* __restrict__ a,
@@ -1122,45 +1208,80 @@ __global__ void __launch_bounds__(kGjB* kGjCols) k_gj_rows(int n, int K, int bs,
                                                           double* __restrict__ C) {
   __shared__ double ps[kGjB][kGjB + 1];
   __shared__ double cs[kGjB][kGjCols];
+  __shared__ double out[kGjB][kGjCols + 1];
   const int p = threadIdx.x, jj = threadIdx.y;
   for (int t = jj; t < kGjB; t += kGjCols) ps[t][p] = pinv[t * kGjB + p];
+  const int t = jj * kGjB + p, lr = t / kGjCols, lj = blockIdx.x * kGjCols + t % kGjCols;  // coalesced in j
+  cs[lr][t % kGjCols] = (lj < n && lr < bs) ? a[(long long)(K + lr) * n + lj] : 0.0;
+  __syncthreads();
   const int j = blockIdx.x * kGjCols + jj;
   const bool inP = j >= K && j < K + bs;
-  cs[p][jj] = (j < n && p < bs && !inP) ? a[(long long)(K + p) * n + j] : 0.0;
-  __syncthreads();
-  if (j >= n || p >= bs) return;
-  if (inP) {
-    R[(long long)p * n + j] = ps[p][j - K];
-    return;
-  }
   double v = 0.0;
 #pragma unroll
   for (int q = 0; q < kGjB; ++q) v = fma(ps[p][q], cs[q][jj], v);
-  R[(long long)p * n + j] = v;
-  a[(long long)(K + p) * n + j] = v;
-  C[(long long)p * n + j] = a[(long long)j * n + K + p];
+  out[p][jj] = v;
+  if (j < n && p < bs && !inP) a[(long long)j * n + K + p] = j < K ? v : -v;
+  __syncthreads();
+  if (lj >= n) return;
+  const bool lp = lj >= K && lj < K + bs;
+  const double w = out[lr][t % kGjCols], old = cs[lr][t % kGjCols];
+  R[(long long)lr * n + lj] = lp ? 0.0 : w;
+  C[(long long)lr * n + lj] = lp ? 0.0 : (lj < K ? -old : old);
+  if (lr < bs && !lp) a[(long long)(K + lr) * n + lj] = w;
 }
 
-// a_ij <- (j in P ? 0 : a_ij) - sum_p C[p][i] R[p][j] for rows i outside P; one
-// kGjB x kGjB tile of (i, j) per block.
-__global__ void __launch_bounds__(kGjB* kGjB) k_gj_update(int n, int K, int bs, double* __restrict__ a,
-                                                         const double* __restrict__ R, const double* __restrict__ C) {
-  __shared__ double cs[kGjB][kGjB + 1];  // cs[p][ti]
+// a_ij -= sum_p C[p][i] R[p][j] for one kGjB x kGjB tile on or above the diagonal per
+// block, outside the panel's row and column, and its mirror image; the block on the next
+// diagonal tile inverts it.
+__global__ void __launch_bounds__(kGjB* kGjB) k_gj_update(int n, int K, int bs, int nt, double* __restrict__ a,
+                                                         const double* __restrict__ R, const double* __restrict__ C,
+                                                         double* __restrict__ pinv) {
+  __shared__ double cs[kGjB][kGjB + 1];  // cs[p][ti], then the tile
   __shared__ double rs[kGjB][kGjB + 1];  // rs[p][tj]
-  const int ti = threadIdx.y, tj = threadIdx.x;
-  const int i0 = blockIdx.y * kGjB, j0 = blockIdx.x * kGjB;
-  for (int p = ti; p < kGjB; p += blockDim.y) {
+  __shared__ double rk[2][kGjB];
+  // tile (I, J), I <= J, from the block number, rows of tiles in order; block 0 takes the
+  // next diagonal tile, so that its inversion starts first
+  const int kt = K / kGjB, next = kt + 1;
+  int b = blockIdx.x, I = 0, J;
+  if (next < nt) {  // number of (next, next) in the order
+    const int nn = next * nt - next * (next - 1) / 2;
+    if (b == 0) b = nn;
+    else if (b <= nn) --b;
+  }
+  while (b >= nt - I) b -= nt - I++;
+  J = I + b;
+  if (I == kt || J == kt) return;
+  const int tj = threadIdx.x & 31, ti = threadIdx.x >> 5;
+  const int i0 = I * kGjB, j0 = J * kGjB;
+  {
     const int i = i0 + tj, j = j0 + tj;
-    cs[p][tj] = (p < bs && i < n) ? C[(long long)p * n + i] : 0.0;
-    rs[p][tj] = (p < bs && j < n) ? R[(long long)p * n + j] : 0.0;
+    cs[ti][tj] = (ti < bs && i < n) ? C[(long long)ti * n + i] : 0.0;
+    rs[ti][tj] = (ti < bs && j < n) ? R[(long long)ti * n + j] : 0.0;
   }
   __syncthreads();
   const int i = i0 + ti, j = j0 + tj;
-  if (i >= n || j >= n || (i >= K && i < K + bs)) return;
-  double acc = (j >= K && j < K + bs) ? 0.0 : a[(long long)i * n + j];
+  const bool in = i < n && j < n;
+  double acc = in ? a[(long long)i * n + j] : 0.0;
 #pragma unroll 8
   for (int p = 0; p < kGjB; ++p) acc = fma(-cs[p][ti], rs[p][tj], acc);
-  a[(long long)i * n + j] = acc;
+  if (in) a[(long long)i * n + j] = acc;
+  __syncthreads();
+  cs[ti][tj] = acc;
+  __syncthreads();
+  if (I < J) {
+    // pivots so far: tiles up to kt; the sign of the mirror image where only one has been
+    const double s = (I <= kt) == (J <= kt) ? 1.0 : -1.0;
+    const int mi = j0 + ti, mj = i0 + tj;
+    if (mi < n && mj < n) a[(long long)mi * n + mj] = s * cs[tj][ti];
+  } else if (I == next) {
+    if (tj < ti) cs[ti][tj] = cs[tj][ti];
+    __syncthreads();
+    if (threadIdx.x < 32 * kGjInvWarps) {
+      const int nbs = min(kGjB, n - i0);
+      gj_invert(cs, nbs, rk);
+      gj_store_panel(cs, n, i0, nbs, a, pinv);
+    }
+  }
 }
 
 // ---------------------------------------------------------------- matching aggregation
@@ -1448,20 +1569,30 @@ static int plist_build(rich_ctx* c, const Csr<double>& A, const Csr<double>& B, 
   RICH_CHECK(dalloc(&pl.pa, (long long)np + 1));
   RICH_CHECK(dalloc(&pl.pb, (long long)np + 1));
   pl.np = (long long)np;
-  int nwb = (A.nrows + kPlWarps - 1) / kPlWarps;
+  const bool wide = (double)np > 512.0 * A.nrows;
+  int nwb = wide ? A.nrows : (A.nrows + kPlWarps - 1) / kPlWarps;
   if (nwb > 64 * kNumSM) nwb = 64 * kNumSM;
+  auto list = [&](auto kernel, const int* seg, const long long* base, int* pa, int* pb) {
+    kernel<<<nwb, 32 * kPlWarps, 0, c->st>>>(A.nrows, A.rowptr, A.col, B.rowptr, B.col, C.rowptr, C.col, cnt, seg,
+                                             base, pa, pb);
+  };
   RICH_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * ((size_t)C.nnz + 1), c->st));
-  k_plist<false><<<nwb, 32 * kPlWarps, 0, c->st>>>(A.nrows, A.rowptr, A.col, B.rowptr, B.col, C.rowptr, C.col, cnt,
-                                                   nullptr, nullptr, nullptr, nullptr);
+  if (wide) list(k_plist<false, true>, nullptr, nullptr, nullptr, nullptr);
+  else list(k_plist<false, false>, nullptr, nullptr, nullptr, nullptr);
   RICH_LAUNCH_CHECK();
   RICH_CHECK(scan_exclusive_int_ll(c, cnt, segll, C.nnz));
   k_plist_split<<<grid_for((long long)C.nnz + 1), kBlock, 0, c->st>>>(C.nnz, segll, pl.seg, pl.base);
   RICH_LAUNCH_CHECK();
   RICH_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * ((size_t)C.nnz + 1), c->st));
-  k_plist<true><<<nwb, 32 * kPlWarps, 0, c->st>>>(A.nrows, A.rowptr, A.col, B.rowptr, B.col, C.rowptr, C.col, cnt,
-                                                  pl.seg, pl.base, pl.pa, pl.pb);
+  if (wide) list(k_plist<true, true>, pl.seg, pl.base, pl.pa, pl.pb);
+  else list(k_plist<true, false>, pl.seg, pl.base, pl.pa, pl.pb);
   RICH_LAUNCH_CHECK();
-  k_plist_sort<<<grid_for(C.nnz), kBlock, 0, c->st>>>(C.nnz, pl.seg, pl.base, pl.pa, pl.pb);
+  // short segments filed by one warp per row are almost in order already
+  if (wide || (double)np > 8.0 * (double)C.nnz)
+    k_plist_rank<<<std::min((int)((C.nnz + kPlWarps - 1) / kPlWarps), 64 * kNumSM), 32 * kPlWarps, 0, c->st>>>(
+        (int)C.nnz, pl.seg, pl.base, pl.pa, pl.pb);
+  else
+    k_plist_sort<<<grid_for(C.nnz), kBlock, 0, c->st>>>(C.nnz, pl.seg, pl.base, pl.pa, pl.pb);
   RICH_LAUNCH_CHECK();
   dfree(cnt);
   dfree(segll);
@@ -1625,25 +1756,25 @@ static int coarse_inverse_launches(rich_ctx* c) {
   Hierarchy& H = c->H;
   Level& L = H.lv[H.nlev - 1];
   int n = L.n;
+  long long nn = (long long)n * n;
+  RICH_CUDA(cudaMemsetAsync(H.cdense, 0, sizeof(double) * (size_t)nn, c->st));
   // in MIXED precision the refreshed coarse values are the FP32 ones
   if (c->prec == RICH_PREC_MIXED && H.nlev > 1)
-    k_csr_to_dense<float><<<grid_for(n), kBlock, 0, c->st>>>(n, L.A.rowptr, L.A.col, L.A32, H.cdense);
+    k_csr_to_dense<float><<<grid_for(32LL * n), kBlock, 0, c->st>>>(n, L.A.rowptr, L.A.col, L.A32, H.cdense);
   else
-    k_csr_to_dense<double><<<grid_for(n), kBlock, 0, c->st>>>(n, L.A.rowptr, L.A.col, L.A.val, H.cdense);
+    k_csr_to_dense<double><<<grid_for(32LL * n), kBlock, 0, c->st>>>(n, L.A.rowptr, L.A.col, L.A.val, H.cdense);
   RICH_LAUNCH_CHECK();
-  long long nn = (long long)n * n;
   double* R = H.cwork;
   double* C = R + (long long)kGjB * n;
   double* pinv = C + (long long)kGjB * n;
-  const dim3 tile(kGjB, kGjB);
-  const dim3 tiles((unsigned)((n + kGjB - 1) / kGjB), (unsigned)((n + kGjB - 1) / kGjB));
-  for (int K = 0; K < n; K += kGjB) {
+  const int nt = (n + kGjB - 1) / kGjB;
+  k_gj_panel<<<1, 32 * kGjInvWarps, 0, c->st>>>(n, std::min(kGjB, n), H.cdense, pinv);
+  RICH_LAUNCH_CHECK();
+  for (int K = 0; K < n && nt > 1; K += kGjB) {
     const int bs = n - K < kGjB ? n - K : kGjB;
-    k_gj_panel<<<1, tile, 0, c->st>>>(n, K, bs, H.cdense, pinv);
-    RICH_LAUNCH_CHECK();
     k_gj_rows<<<(n + kGjCols - 1) / kGjCols, dim3(kGjB, kGjCols), 0, c->st>>>(n, K, bs, H.cdense, pinv, R, C);
     RICH_LAUNCH_CHECK();
-    k_gj_update<<<tiles, tile, 0, c->st>>>(n, K, bs, H.cdense, R, C);
+    k_gj_update<<<nt * (nt + 1) / 2, kGjB * kGjB, 0, c->st>>>(n, K, bs, nt, H.cdense, R, C, pinv);
     RICH_LAUNCH_CHECK();
   }
   if (H.cinv32) {
