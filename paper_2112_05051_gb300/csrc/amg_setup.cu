@@ -489,8 +489,11 @@ __device__ __forceinline__ void warp_sort_keys(unsigned* keys, int u, int lane) 
   __syncwarp();
 }
 
-// Rows with umin < products <= cap (cap slots of shared memory per warp).
-__global__ void __launch_bounds__(256) k_spgemm_sort(int nrows, const int* __restrict__ arp,
+// Rows with umin < products <= cap (cap slots of shared memory per warp), cap <= 32 KMAX.
+// The kernel waits on loads, so the classes are compiled apart: registers for short keys
+// only let twice the warps in (262k rows of 24 products: 340 us with all sizes in one).
+template <int KMAX>
+__global__ void __launch_bounds__(256, KMAX <= 2 ? 6 : KMAX <= 8 ? 5 : 2) k_spgemm_sort(int nrows, const int* __restrict__ arp,
                                                      const int* __restrict__ acol, const double* __restrict__ aval,
                                                      const int* __restrict__ brp, const int* __restrict__ bcol,
                                                      const double* __restrict__ bval, const int* __restrict__ u,
@@ -545,12 +548,16 @@ __global__ void __launch_bounds__(256) k_spgemm_sort(int nrows, const int* __res
       t0 += total;
       __syncwarp();
     }
-    if (ur <= 32) warp_sort_keys<1>(keys, ur, lane);
-    else if (ur <= 64) warp_sort_keys<2>(keys, ur, lane);
-    else if (ur <= 128) warp_sort_keys<4>(keys, ur, lane);
-    else if (ur <= 256) warp_sort_keys<8>(keys, ur, lane);
-    else if (ur <= 512) warp_sort_keys<16>(keys, ur, lane);
-    else warp_sort_keys<32>(keys, ur, lane);
+    if (KMAX <= 2) {
+      if (ur <= 32) warp_sort_keys<1>(keys, ur, lane);
+      else warp_sort_keys<2>(keys, ur, lane);
+    } else if (KMAX <= 8) {
+      if (ur <= 128) warp_sort_keys<4>(keys, ur, lane);
+      else warp_sort_keys<8>(keys, ur, lane);
+    } else {
+      if (ur <= 512) warp_sort_keys<16>(keys, ur, lane);
+      else warp_sort_keys<32>(keys, ur, lane);
+    }
     // segment heads
     const long long base = mode == 1 ? (long long)crp[row] : (mode == 2 ? uoff[row] : 0);
     int running = 0;
@@ -937,21 +944,22 @@ __global__ void __launch_bounds__(kNumThreads) k_spgemm_numeric_block(
 // the same every time.  k_plist enumerates the products of each row (one warp
 // per row, A entries 32 at a time, a warp scan of their B-row lengths spreads
 // the products over the lanes) and either counts the products of every C entry
-// or files each pair into its C entry's segment; k_plist_sort then orders each
-// segment by A entry, which is the order a row-by-row product sums in.
+// or files each pair into its C entry's slots (ProdList), which k_pl_shape lays out from
+// the counts; k_pl_sort or k_pl_rank then orders each entry's pairs by A entry, which is
+// the order a row-by-row product sums in.
 constexpr int kPlWarps = 8;
 constexpr int kPlCols = 512;  // columns of a C row searched in shared memory
 
 // WIDE: a block per row (rows of thousands of products), its warps taking the row's A
-// entries in turn; the order within a segment is settled by k_plist_sort either way.
+// entries in turn; the order within a segment is settled by k_pl_rank either way.
 template <bool FILL, bool WIDE>
 __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* __restrict__ arp,
                                                          const int* __restrict__ acol, const int* __restrict__ brp,
                                                          const int* __restrict__ bcol, const int* __restrict__ crp,
                                                          const int* __restrict__ ccol, int* __restrict__ cnt,
-                                                         const int* __restrict__ seg,
-                                                         const long long* __restrict__ base, int* __restrict__ pa,
-                                                         int* __restrict__ pb) {
+                                                         const int* __restrict__ place,
+                                                         const long long* __restrict__ sptr,
+                                                         int2* __restrict__ pairs) {
   __shared__ int pre_all[kPlWarps][33];
   __shared__ int bst_all[kPlWarps][32];
   __shared__ int col_all[kPlWarps][kPlCols];
@@ -996,9 +1004,8 @@ __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* _
         int q = staged ? c0 + find_col(scol, 0, c1 - c0, bcol[f]) : find_col(ccol, c0, c1, bcol[f]);
         int slot = atomicAdd(&cnt[q], 1);
         if (FILL) {
-          long long at = base[q >> kPlShift] + seg[q] + slot;
-          pa[at] = e0 + lo;
-          pb[at] = f;
+          const int at = place[q];
+          pairs[sptr[at / kSellC] + (long long)slot * kSellC + at % kSellC] = make_int2(e0 + lo, f);
         }
       }
       __syncwarp();
@@ -1006,78 +1013,97 @@ __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* _
   }
 }
 
-// 64-bit segment starts -> chunk bases and 32-bit remainders.
-__global__ void k_plist_split(int nnz, const long long* __restrict__ segll, int* __restrict__ seg,
-                              long long* __restrict__ base) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q <= nnz; q += gridDim.x * blockDim.x) {
-    long long b = segll[(q >> kPlShift) << kPlShift];
-    seg[q] = (int)(segll[q] - b);
-    if ((q & ((1 << kPlShift) - 1)) == 0) base[q >> kPlShift] = b;
+// The lists' layout from the entries' counts: a window of kSellSigma entries per block,
+// bucketed by decreasing count (ties in any order: an entry's sum does not depend on its
+// place).  place[q] is q's position, perm its inverse, slots the slices' sizes.
+constexpr int kPlBuckets = 512;  // longer entries share the first bucket
+__global__ void __launch_bounds__(kSellSigma) k_pl_shape(int nnz, const int* __restrict__ cnt, int nslice,
+                                                         int* __restrict__ perm, int* __restrict__ place,
+                                                         int* __restrict__ slots) {
+  __shared__ int first[kPlBuckets], wsum[kPlBuckets / 32], wide[kSellSigma / kSellC];
+  const int t = threadIdx.x, w0 = blockIdx.x * kSellSigma, q = w0 + t;
+  const int l = q < nnz ? cnt[q] : 0, b = kPlBuckets - 1 - min(l, kPlBuckets - 1);
+  if (t < kPlBuckets) first[t] = 0;
+  if (t < kSellSigma / kSellC) wide[t] = 0;
+  __syncthreads();
+  const int rank = q < nnz ? atomicAdd(&first[b], 1) : 0;
+  __syncthreads();
+  int v = 0, inc = 0;
+  if (t < kPlBuckets) {
+    inc = v = first[t];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, inc, o);
+      if ((t & 31) >= o) inc += u;
+    }
+    if ((t & 31) == 31) wsum[t >> 5] = inc;
   }
+  __syncthreads();
+  if (t < kPlBuckets) {
+    for (int u = 0; u < (t >> 5); ++u) inc += wsum[u];
+    first[t] = inc - v;
+  }
+  __syncthreads();
+  if (q < nnz) {
+    const int r = first[b] + rank;
+    perm[w0 + r] = q;
+    place[q] = w0 + r;
+    atomicMax(&wide[r / kSellC], l);
+  } else if (q < nslice * kSellC) {
+    perm[q] = -1;  // entries fill the window's front: the places past them are the ones past nnz
+  }
+  __syncthreads();
+  if (t < kSellSigma / kSellC && w0 / kSellC + t < nslice) slots[w0 / kSellC + t] = kSellC * wide[t];
 }
 
-__device__ __forceinline__ long long plist_start(const int* __restrict__ seg, const long long* __restrict__ base,
-                                                 int q) {
-  return base[q >> kPlShift] + seg[q];
-}
-
-// Insertion sort of each segment by A entry (segments hold tens of pairs).
-__global__ void k_plist_sort(int nnz, const int* __restrict__ seg, const long long* __restrict__ base,
-                             int* __restrict__ pa, int* __restrict__ pb) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nnz; q += gridDim.x * blockDim.x) {
-    long long s0 = plist_start(seg, base, q), s1 = plist_start(seg, base, q + 1);
-    for (long long t = s0 + 1; t < s1; ++t) {
-      int ka = pa[t], kb = pb[t];
-      long long v = t - 1;
-      while (v >= s0 && pa[v] > ka) {
-        pa[v + 1] = pa[v];
-        pb[v + 1] = pb[v];
-        --v;
-      }
-      pa[v + 1] = ka;
-      pb[v + 1] = kb;
+// Insertion sort of each entry's pairs by A entry, a thread per entry in slot order.
+__global__ void k_pl_sort(int nslice, const long long* __restrict__ sptr, int2* __restrict__ pairs) {
+  const int lane = threadIdx.x & 31;
+  for (int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslice; s += (gridDim.x * blockDim.x) >> 5) {
+    int2* p = pairs + sptr[s] + lane;
+    const int w = (int)((sptr[s + 1] - sptr[s]) / kSellC);
+    for (int t = 1; t < w; ++t) {
+      const int2 k = p[(long long)t * kSellC];
+      if (k.x < 0) break;  // past the entry's end
+      int v = t - 1;
+      for (; v >= 0 && p[(long long)v * kSellC].x > k.x; --v) p[(long long)(v + 1) * kSellC] = p[(long long)v * kSellC];
+      p[(long long)(v + 1) * kSellC] = k;
     }
   }
 }
 
-// The same for long segments, a warp each: up to kPlSort pairs are ranked in shared memory
+// The same for long entries, a warp each: up to kPlSort pairs are ranked in shared memory
 // (an A entry contributes one product to an entry of C, so the keys are distinct).
 constexpr int kPlSort = 512;
-__global__ void __launch_bounds__(32 * kPlWarps) k_plist_rank(int nnz, const int* __restrict__ seg,
-                                                              const long long* __restrict__ base,
-                                                              int* __restrict__ pa, int* __restrict__ pb) {
-  __shared__ int a_all[kPlWarps][kPlSort], b_all[kPlWarps][kPlSort];
+__global__ void __launch_bounds__(32 * kPlWarps) k_pl_rank(int nnz, const int* __restrict__ cnt,
+                                                           const int* __restrict__ place,
+                                                           const long long* __restrict__ sptr,
+                                                           int2* __restrict__ pairs) {
+  __shared__ int2 a_all[kPlWarps][kPlSort];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int *a = a_all[w], *b = b_all[w];
+  int2* a = a_all[w];
   for (int q = blockIdx.x * kPlWarps + w; q < nnz; q += gridDim.x * kPlWarps) {
-    const long long s0 = plist_start(seg, base, q);
-    const int len = (int)(plist_start(seg, base, q + 1) - s0);
+    const int len = cnt[q], at = place[q];
     if (len < 2) continue;
+    int2* p = pairs + sptr[at / kSellC] + at % kSellC;
     if (len > kPlSort) {
       if (lane == 0)
-        for (long long t = s0 + 1; t < s0 + len; ++t) {
-          const int ka = pa[t], kb = pb[t];
-          long long v = t - 1;
-          for (; v >= s0 && pa[v] > ka; --v) {
-            pa[v + 1] = pa[v];
-            pb[v + 1] = pb[v];
-          }
-          pa[v + 1] = ka;
-          pb[v + 1] = kb;
+        for (int t = 1; t < len; ++t) {
+          const int2 k = p[(long long)t * kSellC];
+          int v = t - 1;
+          for (; v >= 0 && p[(long long)v * kSellC].x > k.x; --v)
+            p[(long long)(v + 1) * kSellC] = p[(long long)v * kSellC];
+          p[(long long)(v + 1) * kSellC] = k;
         }
       continue;
     }
-    for (int t = lane; t < len; t += 32) {
-      a[t] = pa[s0 + t];
-      b[t] = pb[s0 + t];
-    }
+    for (int t = lane; t < len; t += 32) a[t] = p[(long long)t * kSellC];
     __syncwarp();
     for (int t = lane; t < len; t += 32) {
-      const int k = a[t];
+      const int2 k = a[t];
       int r = 0;
-      for (int v = 0; v < len; ++v) r += a[v] < k;
-      pa[s0 + r] = k;
-      pb[s0 + r] = b[t];
+      for (int v = 0; v < len; ++v) r += a[v].x < k.x;
+      p[(long long)r * kSellC] = k;
     }
     __syncwarp();
   }
@@ -1090,22 +1116,41 @@ __global__ void k_sum_rows_ll(int n, const int* __restrict__ u, unsigned long lo
   if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
 }
 
-// c[q] = sum over the segment of q of a[pa] * b[pb], in segment order: no
-// search, no atomics, the same sum every refresh.  One thread per entry keeps
-// the threads of a warp on neighbouring entries of one C row, whose pairs read
-// neighbouring B entries (a lane group per entry was measured slower: its
-// gathers from B, too large for L2, lose that locality).
+// c[q] = sum of a[x] * b[y] over q's pairs, in their order: no search, no atomics, the same
+// sum every refresh.  A warp per slice, a thread per entry, four pairs in flight.
+// Bound: FP64 one FMA per pair, FP32 HBM (8 bytes per pair).  128^3 FP64, 176M pairs over
+// three levels: 1270 us with the pairs entry by entry (a thread's own run, 32 sectors per
+// warp and load, and as many steps as the longest of 32 neighbours).
 template <class T>
-__global__ void __launch_bounds__(256) k_galerkin_lists(int nnz, const int* __restrict__ seg,
-                                                        const long long* __restrict__ base,
-                                                        const int* __restrict__ pa, const int* __restrict__ pb,
-                                                        const T* __restrict__ aval, const T* __restrict__ bval,
-                                                        T* __restrict__ cval) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nnz; q += gridDim.x * blockDim.x) {
-    long long s0 = plist_start(seg, base, q), s1 = plist_start(seg, base, q + 1);
+__global__ void __launch_bounds__(256) k_galerkin_lists(int nslice, const int* __restrict__ perm,
+                                                        const long long* __restrict__ sptr,
+                                                        const int2* __restrict__ pairs, const T* __restrict__ aval,
+                                                        const T* __restrict__ bval, T* __restrict__ cval) {
+  const int lane = threadIdx.x & 31;
+  for (int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslice; s += (gridDim.x * blockDim.x) >> 5) {
+    const int q = perm[s * kSellC + lane];
+    long long e = sptr[s] + lane;
+    const long long end = sptr[s + 1];
     T acc = T(0);
-    for (long long t = s0; t < s1; ++t) acc += aval[pa[t]] * bval[pb[t]];
-    cval[q] = acc;
+    for (; e + 3 * kSellC < end; e += 4 * kSellC) {  // warp-uniform
+      int2 p[4];
+      T a[4], b[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) p[u] = __ldcs(&pairs[e + u * kSellC]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        a[u] = p[u].x >= 0 ? aval[p[u].x] : T(0);
+        b[u] = p[u].x >= 0 ? bval[p[u].y] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (p[u].x >= 0) acc += a[u] * b[u];
+    }
+    for (; e < end; e += kSellC) {
+      const int2 p = __ldcs(&pairs[e]);
+      if (p.x >= 0) acc += aval[p.x] * bval[p.y];
+    }
+    if (q >= 0) cval[q] = acc;
   }
 }
 
@@ -1495,14 +1540,18 @@ static int spgemm_symbolic(rich_ctx* c, const Csr<double>& A, const Csr<double>&
     int* ocol = mode == 2 ? tcol : C.col;
     double* oval = mode == 2 ? tval : C.val;
     if (B.ncols < (1 << kSortCol)) {
-      // rows of up to 256 products with 3 kB of shared memory per warp, the others apart
-      for (int umin = 0; umin < cap; umin = umin ? cap : 256) {
-        const int cp = umin ? cap : std::min(cap, 256), wpb = cp <= 256 ? 8 : cp <= 512 ? 4 : 2;
+      auto run = [&](auto kernel, int umin, int cp, int wpb) -> int {
+        if (umin >= cap) return RICH_OK;
+        cp = std::min(cap, cp);
         const int nblk2 = std::min((n + wpb - 1) / wpb, 64 * kNumSM);
-        k_spgemm_sort<<<nblk2, 32 * wpb, (size_t)wpb * cp * (sizeof(double) + sizeof(unsigned)), c->st>>>(
+        kernel<<<nblk2, 32 * wpb, (size_t)wpb * cp * (sizeof(double) + sizeof(unsigned)), c->st>>>(
             n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, u, mode, C.rowptr, uoff, ocol, oval, cnt, umin, cp);
         RICH_LAUNCH_CHECK();
-      }
+        return RICH_OK;
+      };
+      RICH_CHECK(run(k_spgemm_sort<2>, 0, 64, 8));
+      RICH_CHECK(run(k_spgemm_sort<8>, 64, 256, 8));
+      RICH_CHECK(run(k_spgemm_sort<32>, 256, 1024, cap <= 512 ? 4 : 2));
     } else {
       k_spgemm_esc<<<nblk, 32 * esc_warps, smem, c->st>>>(n, A.rowptr, A.col, A.val, B.rowptr, B.col, B.val, u, mode,
                                                          C.rowptr, uoff, ocol, oval, cnt, cap);
@@ -1535,10 +1584,10 @@ static const char* kNumericName[2][16] = {
      "galerkin_rap", "galerkin_rap", "galerkin_rap", "galerkin_rap", "galerkin_rap"}};
 
 static void plist_free(ProdList& pl) {
-  dfree(pl.seg);
-  dfree(pl.base);
-  dfree(pl.pa);
-  dfree(pl.pb);
+  dfree(pl.perm);
+  dfree(pl.sptr);
+  dfree(pl.pairs);
+  pl.nslice = 0;
   pl.np = 0;
 }
 
@@ -1560,42 +1609,52 @@ static int plist_build(rich_ctx* c, const Csr<double>& A, const Csr<double>& B, 
   fr += pool_slack();  // blocks freed into the pool count as free here
   double need = 8.0 * (double)np + 24.0 * ((double)C.nnz + 1);  // lists, offsets and the build's scratch
   if (need > 0.5 * (double)fr) return RICH_OK;
-  int* cnt = nullptr;
-  long long* segll = nullptr;
-  RICH_CHECK(dalloc(&cnt, (long long)C.nnz + 1));
-  RICH_CHECK(dalloc(&segll, (long long)C.nnz + 1));
-  RICH_CHECK(dalloc(&pl.seg, (long long)C.nnz + 1));
-  RICH_CHECK(dalloc(&pl.base, ((long long)C.nnz >> kPlShift) + 1));
-  RICH_CHECK(dalloc(&pl.pa, (long long)np + 1));
-  RICH_CHECK(dalloc(&pl.pb, (long long)np + 1));
+  const int nnz = (int)C.nnz;
+  pl.nslice = (nnz + kSellC - 1) / kSellC;
+  int *cnt = nullptr, *place = nullptr, *slots = nullptr;
+  RICH_CHECK(dalloc(&cnt, nnz + 1LL));
+  RICH_CHECK(dalloc(&place, nnz + 1LL));
+  RICH_CHECK(dalloc(&slots, pl.nslice));
+  RICH_CHECK(dalloc(&pl.perm, (long long)pl.nslice * kSellC));
+  RICH_CHECK(dalloc(&pl.sptr, pl.nslice + 1LL));
   pl.np = (long long)np;
   const bool wide = (double)np > 512.0 * A.nrows;
   int nwb = wide ? A.nrows : (A.nrows + kPlWarps - 1) / kPlWarps;
   if (nwb > 64 * kNumSM) nwb = 64 * kNumSM;
-  auto list = [&](auto kernel, const int* seg, const long long* base, int* pa, int* pb) {
-    kernel<<<nwb, 32 * kPlWarps, 0, c->st>>>(A.nrows, A.rowptr, A.col, B.rowptr, B.col, C.rowptr, C.col, cnt, seg,
-                                             base, pa, pb);
+  auto list = [&](auto kernel) {
+    kernel<<<nwb, 32 * kPlWarps, 0, c->st>>>(A.nrows, A.rowptr, A.col, B.rowptr, B.col, C.rowptr, C.col, cnt, place,
+                                             pl.sptr, pl.pairs);
   };
-  RICH_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * ((size_t)C.nnz + 1), c->st));
-  if (wide) list(k_plist<false, true>, nullptr, nullptr, nullptr, nullptr);
-  else list(k_plist<false, false>, nullptr, nullptr, nullptr, nullptr);
+  RICH_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * ((size_t)nnz + 1), c->st));
+  if (wide) list(k_plist<false, true>);
+  else list(k_plist<false, false>);
   RICH_LAUNCH_CHECK();
-  RICH_CHECK(scan_exclusive_int_ll(c, cnt, segll, C.nnz));
-  k_plist_split<<<grid_for((long long)C.nnz + 1), kBlock, 0, c->st>>>(C.nnz, segll, pl.seg, pl.base);
+  k_pl_shape<<<(nnz + kSellSigma - 1) / kSellSigma, kSellSigma, 0, c->st>>>(nnz, cnt, pl.nslice, pl.perm, place, slots);
   RICH_LAUNCH_CHECK();
-  RICH_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * ((size_t)C.nnz + 1), c->st));
-  if (wide) list(k_plist<true, true>, pl.seg, pl.base, pl.pa, pl.pb);
-  else list(k_plist<true, false>, pl.seg, pl.base, pl.pa, pl.pb);
-  RICH_LAUNCH_CHECK();
-  // short segments filed by one warp per row are almost in order already
-  if (wide || (double)np > 8.0 * (double)C.nnz)
-    k_plist_rank<<<std::min((int)((C.nnz + kPlWarps - 1) / kPlWarps), 64 * kNumSM), 32 * kPlWarps, 0, c->st>>>(
-        (int)C.nnz, pl.seg, pl.base, pl.pa, pl.pb);
-  else
-    k_plist_sort<<<grid_for(C.nnz), kBlock, 0, c->st>>>(C.nnz, pl.seg, pl.base, pl.pa, pl.pb);
-  RICH_LAUNCH_CHECK();
+  RICH_CHECK(scan_exclusive_int_ll(c, slots, pl.sptr, pl.nslice));
+  long long total = 0;
+  RICH_CUDA(cudaMemcpyAsync(&total, pl.sptr + pl.nslice, sizeof(total), cudaMemcpyDeviceToHost, c->st));
+  RICH_CUDA(cudaStreamSynchronize(c->st));
+  if (dalloc(&pl.pairs, total) != RICH_OK) {  // padding beyond what was free: the refresh searches
+    cudaGetLastError();
+    plist_free(pl);
+  } else {
+    RICH_CUDA(cudaMemsetAsync(pl.pairs, 0xff, sizeof(int2) * (size_t)total, c->st));  // x = -1: no pair
+    RICH_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * ((size_t)nnz + 1), c->st));
+    if (wide) list(k_plist<true, true>);
+    else list(k_plist<true, false>);
+    RICH_LAUNCH_CHECK();
+    // short entries filed by one warp per row are almost in order already
+    if (wide || (double)np > 8.0 * (double)nnz)
+      k_pl_rank<<<std::min((nnz + kPlWarps - 1) / kPlWarps, 64 * kNumSM), 32 * kPlWarps, 0, c->st>>>(nnz, cnt, place,
+                                                                                                   pl.sptr, pl.pairs);
+    else
+      k_pl_sort<<<grid_for(32LL * pl.nslice), kBlock, 0, c->st>>>(pl.nslice, pl.sptr, pl.pairs);
+    RICH_LAUNCH_CHECK();
+  }
   dfree(cnt);
-  dfree(segll);
+  dfree(place);
+  dfree(slots);
   return RICH_OK;
 }
 
@@ -1605,13 +1664,13 @@ template <class T>
 static int spgemm_numeric_t(rich_ctx* c, const Csr<double>& A, const T* aval, const Csr<double>& B, const T* bval,
                             const Csr<double>& C, T* cval, const int* u, int which, int level,
                             const ProdList* pl = nullptr) {
-  if (pl && pl->seg) {
+  if (pl && pl->built()) {
     ProfScope ps(kNumericName[which][level & 15], c->st,
                  4.0 * ((double)C.nnz + 1) + 8.0 * (double)pl->np +
                      (double)sizeof(T) * ((double)A.nnz + (double)B.nnz + (double)C.nnz),
                  2.0 * (double)pl->np);
-    k_galerkin_lists<T><<<grid_for(C.nnz, 256), 256, 0, c->st>>>(C.nnz, pl->seg, pl->base, pl->pa, pl->pb, aval,
-                                                                  bval, cval);
+    k_galerkin_lists<T><<<(pl->nslice + 7) / 8, 256, 0, c->st>>>(pl->nslice, pl->perm, pl->sptr, pl->pairs, aval, bval,
+                                                                cval);
     RICH_LAUNCH_CHECK();
     return RICH_OK;
   }
@@ -2247,8 +2306,8 @@ static int coarsen(rich_ctx* c, int l, bool* stop) {
     // refresh would build), so that a setup does not depend on the order of atomics.
     L.pl_tried = true;
     RICH_CHECK(plist_build(c, L.A, L.P, L.AP, L.u_ap, L.pl_ap));
-    if (L.pl_ap.seg) RICH_CHECK(plist_build(c, L.R, L.AP, nxt.A, L.u_rap, L.pl_rap));
-    if (L.pl_ap.seg && L.pl_rap.seg) {
+    if (L.pl_ap.built()) RICH_CHECK(plist_build(c, L.R, L.AP, nxt.A, L.u_rap, L.pl_rap));
+    if (L.pl_ap.built() && L.pl_rap.built()) {
       RICH_CHECK(spgemm_numeric(c, L.A, L.P, L.AP, L.u_ap, 0, l, &L.pl_ap));
       RICH_CHECK(spgemm_numeric(c, L.R, L.AP, nxt.A, L.u_rap, 1, l, &L.pl_rap));
     }
@@ -2341,7 +2400,7 @@ int amg_refresh(rich_ctx* c) {
     if (L.pl_tried || !H.opts.product_lists) continue;
     L.pl_tried = true;
     RICH_CHECK(plist_build(c, L.A, L.P, L.AP, L.u_ap, L.pl_ap));
-    if (L.pl_ap.seg) RICH_CHECK(plist_build(c, L.R, L.AP, H.lv[l + 1].A, L.u_rap, L.pl_rap));
+    if (L.pl_ap.built()) RICH_CHECK(plist_build(c, L.R, L.AP, H.lv[l + 1].A, L.u_rap, L.pl_rap));
   }
   if (c->prec == RICH_PREC_MIXED) {
     // The V-cycle runs in FP32, so the Galerkin products do too: A32_{l+1} =

@@ -169,21 +169,22 @@ struct Sell {
   bool built() const { return sptr != nullptr; }
 };
 
-// One level of the AMG hierarchy.  Level 0 holds the diffusion matrix of the
-// finest grid; levels 1.. hold Galerkin products.  FP32 copies exist in MIXED mode.
-// Galerkin refresh by product lists: entry q of C = A B is the sum over
-// t in [start(q), start(q+1)) of a[pa[t]] * b[pb[t]], the pairs sorted by A
-// entry; start(q) = base[q >> kPlShift] + seg[q] (64-bit pair offsets stored as
-// one base per 2^kPlShift entries plus a 32-bit remainder).
-constexpr int kPlShift = 10;
+// Galerkin refresh by product lists: entry q of C = A B is the sum of a[x] * b[y] over
+// its pairs (x, y), in A-entry order.  Entries are ranked by their number of pairs within
+// windows of kSellSigma and cut into slices of 32, the pairs of a slice stored column by
+// column as in Sell (slot sptr[s] + 32 j + t: pair j of entry perm[32 s + t], x = -1 past its
+// end), so that a warp reads its pairs coalesced and its threads end together.
 struct ProdList {
-  int* seg = nullptr;        // nnz(C) + 1 offsets within the entry's chunk
-  long long* base = nullptr; // (nnz(C) >> kPlShift) + 1 chunk offsets
-  int* pa = nullptr;         // A entry of each pair
-  int* pb = nullptr;         // B entry of each pair
-  long long np = 0;          // pairs (= scalar products of C = A B)
+  long long np = 0;            // pairs (= scalar products of C = A B)
+  int nslice = 0;
+  int* perm = nullptr;         // 32 nslice entries of C, -1 past the last
+  long long* sptr = nullptr;   // nslice + 1 slot offsets
+  int2* pairs = nullptr;
+  bool built() const { return pairs != nullptr; }
 };
 
+// One level of the AMG hierarchy.  Level 0 holds the diffusion matrix of the
+// finest grid; levels 1.. hold Galerkin products.  FP32 copies exist in MIXED mode.
 struct Level {
   int n = 0;
   Csr<double> A;
