@@ -1136,12 +1136,14 @@ int vcycle_apply(rich_ctx* c, const double* r, double* z) {
 // algorithms", 2021).  With G = V^T V, whose last row is the new vector's dots, the
 // coefficients of two projections are h = h1 + (I - G) h1, h1 = V^T w, so the basis is read
 // once for the dots (with w and with the newest vector) and once for w - V h; V stays
-// orthogonal to about ten units of rounding.  Bound: the FP64 pipe, three operations per
-// basis element (explicit second projections take four and read the basis four times).
-// Where w - V h loses more than 1e-2 of w's norm, the host asks for one explicit pass more.
-// 128^3, FGMRES(30): 667 us per iteration with two explicit projections, 598 with these passes.
+// orthogonal to about ten units of rounding.  Bound: the FP64 pipe, two operations per basis
+// element, one in either pass (explicit second projections take four and read the basis four
+// times), and in the dots the loads.  Where w - V h loses more than 1e-2 of w's norm, the host
+// asks for one explicit pass more.
+// 128^3, FGMRES(30): 667 us per iteration with two explicit projections, 545 with a Gram matrix
+// summed in FP64, 518 with one summed in integers (dots at ten vectors: 101 -> 75 us).
 constexpr int kGsThreads = 256;
-constexpr int kGsBlocks = 2 * kNumSM;  // of the dots (fixed: deterministic summation order)
+constexpr int kGsBlocks = 3 * kNumSM;  // of the dots: one wave at 80 registers (4 per SM, 64 registers: 93 us against 83)
 constexpr int kGsUpdateBlocks = 4 * kNumSM;  // of the update: one wave (8 per SM left a second, 59 us against 46)
 constexpr int kGsTile = 4;             // basis vectors per sweep over a block's elements
 constexpr int kGsLd = 64;              // row length of the Gram matrix
@@ -1167,49 +1169,116 @@ __device__ __forceinline__ double warp_sum8(double (&a)[8]) {
   return a[0];
 }
 
+// G's entries are summed in integers.  The basis is normalised, |v| <= 1, so an entry in
+// units of 2^-60 is h 2^30 + l with |h| <= 2^30 and |l| <= 2^29, and a product is four 32-bit
+// multiply-adds into three 64-bit sums; those and the split (20 integer instructions) run
+// beside the FP64 pipe, which is left with the dots with w alone.  An entry's rounding, at
+// most 2^-61, is all the error: |G - V^T V| measured 7e-19 on random and smooth vectors of
+// 300k entries and 1.4e-16 at worst (a constant against one cell with a tail of 1e-18),
+// where FP64 sums leave up to 8e-17, the rounding of a diagonal entry.
+struct UnitFixed {
+  int h, l;
+};
+__device__ __forceinline__ UnitFixed unit_fixed(double v) {
+  const int hi = __double2hiint(v), sg = hi >> 31;
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu, s = min(1023u - e, 63u);
+  // twice the magnitude in units of 2^-60, shifted, then rounded to nearest
+  unsigned long long m = (unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(v);
+  m = (((m << 9) >> s) + 1) >> 1;
+  const int h = (int)((m + (1u << 29)) >> 30), l = (int)((unsigned)m - ((unsigned)h << 30));
+  return {(h ^ sg) - sg, (l ^ sg) - sg};
+}
+// Sums of products: hh 2^-60 + x 2^-90 + ll 2^-120, carried after every kUnitRun of
+// them.  |ll| grows by 2^58 a product; |x| stays below 2 2^29 sqrt(16) 2^30 and |hh| below
+// 2^60 because sum h^2 <= 2^60 over a whole vector.
+constexpr int kUnitRun = 16;
+struct UnitSum {
+  long long hh = 0, x = 0, ll = 0;
+  __device__ __forceinline__ void add(UnitFixed a, UnitFixed b) {
+    hh += (long long)a.h * b.h;
+    x += (long long)a.h * b.l;
+    x += (long long)a.l * b.h;
+    ll += (long long)a.l * b.l;
+  }
+  __device__ __forceinline__ void carry() {
+    x += ll >> 30;
+    ll &= (1 << 30) - 1;
+    hh += x >> 30;
+    x &= (1 << 30) - 1;
+  }
+  // The sum in units of 2^-62, rounded to one of them (a thread's; one conversion).
+  __device__ __forceinline__ double value() {
+    carry();
+    return (double)(4 * hh + ((x + (1 << 27)) >> 28));
+  }
+};
+
+// Copies of 8 bytes into the thread's own words of shared memory, kGsStages elements deep:
+// the loads of the next elements run under this one's arithmetic and hold no registers
+// (with plain loads the warps waited for memory two thirds of the time: 147 us, ten vectors).
+constexpr int kGsStages = 3;
+typedef double GsStage[kGsTile + 2][kGsThreads];
+__device__ __forceinline__ void copy8(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
 // The block's sums over its elements of M basis vectors (from v0) times w and vj, into
 // a[q] and a[4 + q].
 template <int M>
-__device__ __forceinline__ void gs_tile(long long n, const double* __restrict__ v0, const double* __restrict__ w,
-                                        const double* __restrict__ vj, double (&a)[8]) {
+__device__ __forceinline__ void gs_tile(long long n, const double* v0, const double* w, const double* vj,
+                                        GsStage (&st)[kGsStages], double (&a)[8]) {
   const long long stride = (long long)gridDim.x * kGsThreads;
-  long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x;
-  for (; i + stride < n; i += 2 * stride) {
-    const double w0 = w[i], w1 = w[i + stride], x0 = vj[i], x1 = vj[i + stride];
-    double p[M], r[M];
+  const int t = threadIdx.x;
+  auto fetch = [&](int slot, long long i) {
+    if (i < n) {
 #pragma unroll
-    for (int q = 0; q < M; ++q) {
-      p[q] = v0[q * n + i];
-      r[q] = v0[q * n + i + stride];
+      for (int q = 0; q < M; ++q) copy8(&st[slot][q][t], v0 + q * n + i);
+      copy8(&st[slot][kGsTile][t], w + i);
+      copy8(&st[slot][kGsTile + 1][t], vj + i);
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  long long i = blockIdx.x * (long long)kGsThreads + t;
+#pragma unroll
+  for (int k = 0; k < kGsStages; ++k) fetch(k, i + k * stride);
+  UnitSum g[M];
+  int run = 0, slot = 0;
+#pragma unroll 1
+  for (; i < n; i += stride) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kGsStages - 1) : "memory");
+    double p[M];
+    const double w0 = st[slot][kGsTile][t], x0 = st[slot][kGsTile + 1][t];
+#pragma unroll
+    for (int q = 0; q < M; ++q) p[q] = st[slot][q][t];
+    const UnitFixed f = unit_fixed(x0);
 #pragma unroll
     for (int q = 0; q < M; ++q) {
       a[q] = fma(p[q], w0, a[q]);
-      a[q + 4] = fma(p[q], x0, a[q + 4]);
-      a[q] = fma(r[q], w1, a[q]);
-      a[q + 4] = fma(r[q], x1, a[q + 4]);
+      g[q].add(unit_fixed(p[q]), f);
     }
-  }
-  if (i < n) {
-    const double w0 = w[i], x0 = vj[i];
+    if (++run == kUnitRun) {
 #pragma unroll
-    for (int q = 0; q < M; ++q) {
-      const double p = v0[q * n + i];
-      a[q] = fma(p, w0, a[q]);
-      a[q + 4] = fma(p, x0, a[q + 4]);
+      for (int q = 0; q < M; ++q) g[q].carry();
+      run = 0;
     }
+    fetch(slot, i + kGsStages * stride);  // into the words just read
+    slot = slot == kGsStages - 1 ? 0 : slot + 1;
   }
+#pragma unroll
+  for (int q = 0; q < M; ++q) a[4 + q] = g[q].value();
 }
 
 // h1 = V^T w and the newest row of G = V^T V (nv vectors, vj = V[nv - 1]); the last block
 // to finish forms h and leaves it at s[0, nv) and in the pinned mirror.
-__global__ void __launch_bounds__(kGsThreads) k_gs_dots(long long n, int nv, const double* __restrict__ V,
+__global__ void __launch_bounds__(kGsThreads, 3) k_gs_dots(long long n, int nv, const double* __restrict__ V,
                                                         const double* __restrict__ w, double* __restrict__ part,
                                                         double* __restrict__ gram, unsigned* __restrict__ ticket,
                                                         double* __restrict__ s, double* __restrict__ mirror) {
   constexpr int W = kGsThreads / 32;
   __shared__ double sh[W][2 * kGsTile];
   __shared__ double tot[2 * kGsLd];
+  __shared__ GsStage st[kGsStages];
   __shared__ bool last;
   const double* vj = V + (long long)(nv - 1) * n;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1217,10 +1286,10 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_dots(long long n, int nv, con
     double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const double* v0 = V + (long long)q0 * n;
     const int m = min(kGsTile, nv - q0);
-    if (m == 4) gs_tile<4>(n, v0, w, vj, a);
-    else if (m == 3) gs_tile<3>(n, v0, w, vj, a);
-    else if (m == 2) gs_tile<2>(n, v0, w, vj, a);
-    else gs_tile<1>(n, v0, w, vj, a);
+    if (m == 4) gs_tile<4>(n, v0, w, vj, st, a);
+    else if (m == 3) gs_tile<3>(n, v0, w, vj, st, a);
+    else if (m == 2) gs_tile<2>(n, v0, w, vj, st, a);
+    else gs_tile<1>(n, v0, w, vj, st, a);
     const double r = warp_sum8(a);
     if ((lane & 3) == 0) sh[wid][lane >> 2] = r;
     __syncthreads();
@@ -1244,7 +1313,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_dots(long long n, int nv, con
     for (int k = lane; k < (int)gridDim.x; k += 32) a += __ldcg(&part[(long long)q * gridDim.x + k]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if (lane == 0) tot[q] = a;
+    if (lane == 0) tot[q] = t < nv ? a : a * 0x1p-62;
   }
   __syncthreads();
   if (threadIdx.x < nv) gram[(nv - 1) * kGsLd + threadIdx.x] = gram[threadIdx.x * kGsLd + nv - 1] = tot[kGsLd + threadIdx.x];
