@@ -59,11 +59,7 @@ FALLBACK_HBM_GBS = 6800.0
 # ncu dram__bytes_read.sum + dram__bytes_write.sum per launch of a kernel on a
 # workload, from the profiles/ summaries of the same kernel and workload (None:
 # no capture of the current kernel).
-# DRAM bytes per launch from ncu captures of the same workload: the finest FP64
-# sweep measured whole; the batched dots measured over their first 60 launches
-# (DRAM / algorithmic = 1.037) and scaled to the profile pass's 241.2 MB per launch
-NCU_TRAFFIC_BYTES = {("richards128_fp64", "l1jacobi_l0"): 125.615616e6,
-                     ("richards128_fp64", "multidot"): 1.037 * 241.2e6}
+NCU_TRAFFIC_BYTES = {}
 # the oracle's reduced grid for the host-core samples (cells per side)
 CPU_SAMPLE_N = {"richards128_fp64": 48, "richards16_fp64": 16, "richards256_mixed": 32, "richards512_mixed": 32,
                 "paper_infiltration": 96}
@@ -567,7 +563,7 @@ def roofline_of(name, ms, launches, nbytes, flops, fp64, peak_gbs, fp64_tflops, 
 
 # kernel name prefix -> (profile names that make it, runs in FP64 in the FP64 mode)
 def _is_fp64_kernel(name, prec_fp64):
-    if name in ("residual", "assemble", "stencil_spmv", "multidot", "orth_axpy", "orth_final", "fcg_update"):
+    if name in ("residual", "assemble", "stencil_spmv", "multidot", "orth_axpy", "fcg_update"):
         return True
     return prec_fp64
 

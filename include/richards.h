@@ -116,7 +116,8 @@ extern "C" {
 #define RICH_PREC_MIXED  1
 
 #define RICH_KRYLOV_FCG     0  /* Notay's flexible CG, truncation 1 */
-#define RICH_KRYLOV_FGMRES  1  /* Saad's flexible GMRES(m), CGS2, Givens */
+#define RICH_KRYLOV_FGMRES  1  /* Saad's flexible GMRES(m); classical Gram-Schmidt whose second
+                                  projection comes from the basis' Gram matrix; Givens */
 
 /* AMG reuse across Newton iterations.
  *  REFRESH      aggregates, P and R from the first setup of the run are kept;
@@ -195,7 +196,7 @@ typedef struct {
   int autotune;            /* 1 (default): the first time a CSR row operation of the V-cycle (sweep,
                               residual, restriction, prolongation) meets a shape class (rows in
                               quarter-octave bins, mean row length), every lane-group width (1..32 lanes
-                              per row, and 1..8 with four-way unrolled rows) is timed on it and the
+                              per row, each also with four-way unrolled rows) is timed on it and the
                               fastest is kept for the process
                               (rich_autotune_table lists the choices); 0: a fixed rule by the mean row
                               length */
@@ -491,7 +492,7 @@ int rich_kernel_launches(long long* out);
 /* Time every launch of the kernel called name (NULL disables) with CUDA events
  * on its launching stream, from now until the next call.  Names: "residual",
  * "assemble", "stencil_spmv", "l1jacobi_l0", "l1jacobi", "csr_resid",
- * "restrict", "prolong", "coarse_gemv", "multidot", "multiaxpy", "fcg_update",
+ * "resid_l0", "restrict", "prolong", "coarse_gemv", "multidot", "orth_axpy", "fcg_update",
  * "spgemm_numeric". */
 int rich_profile_kernel(const char* name);
 /* Time only every stride-th launch of the profiling target (1 = every launch,

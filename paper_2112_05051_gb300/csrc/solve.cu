@@ -1143,7 +1143,8 @@ int vcycle_apply(rich_ctx* c, const double* r, double* z) {
 // 128^3, FGMRES(30): 667 us per iteration with two explicit projections, 545 with a Gram matrix
 // summed in FP64, 518 with one summed in integers (dots at ten vectors: 101 -> 75 us).
 constexpr int kGsThreads = 256;
-constexpr int kGsBlocks = 3 * kNumSM;  // of the dots: one wave at 80 registers (4 per SM, 64 registers: 93 us against 83)
+// Of the dots: one wave at 80 registers (4 per SM with 64 registers: 93 us against 83).
+constexpr int kGsBlocks = 3 * kNumSM;
 constexpr int kGsUpdateBlocks = 4 * kNumSM;  // of the update: one wave (8 per SM left a second, 59 us against 46)
 constexpr int kGsTile = 4;             // basis vectors per sweep over a block's elements
 constexpr int kGsLd = 64;              // row length of the Gram matrix
@@ -1183,7 +1184,8 @@ __device__ __forceinline__ UnitFixed unit_fixed(double v) {
   const int hi = __double2hiint(v), sg = hi >> 31;
   const unsigned e = ((unsigned)hi >> 20) & 0x7ffu, s = min(1023u - e, 63u);
   // twice the magnitude in units of 2^-60, shifted, then rounded to nearest
-  unsigned long long m = (unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(v);
+  unsigned long long m = (unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32;
+  m |= (unsigned)__double2loint(v);
   m = (((m << 9) >> s) + 1) >> 1;
   const int h = (int)((m + (1u << 29)) >> 30), l = (int)((unsigned)m - ((unsigned)h << 30));
   return {(h ^ sg) - sg, (l ^ sg) - sg};
@@ -1316,7 +1318,8 @@ __global__ void __launch_bounds__(kGsThreads, 3) k_gs_dots(long long n, int nv, 
     if (lane == 0) tot[q] = t < nv ? a : a * 0x1p-62;
   }
   __syncthreads();
-  if (threadIdx.x < nv) gram[(nv - 1) * kGsLd + threadIdx.x] = gram[threadIdx.x * kGsLd + nv - 1] = tot[kGsLd + threadIdx.x];
+  if (threadIdx.x < nv)
+    gram[(nv - 1) * kGsLd + threadIdx.x] = gram[threadIdx.x * kGsLd + nv - 1] = tot[kGsLd + threadIdx.x];
   __syncthreads();
   for (int i = wid; i < nv; i += W) {  // h_i = h1_i + sum_q (I - G)_iq h1_q
     double d = 0.0;
@@ -1870,7 +1873,7 @@ static int gs_pass(rich_ctx* c, int nv, const double* w, double* out) {
   const long long n = c->g.n;
   const int g = std::min(grid_for(n), kGsBlocks), gu = std::min(grid_for(n, 2 * kBlock), kGsUpdateBlocks);
   {
-    ProfScope ps("multidot", c->st, (double)n * 8.0 * (nv + 1), 4.0 * n * nv);
+    ProfScope ps("multidot", c->st, (double)n * 8.0 * (nv + 1), 2.0 * n * nv);  // FP64 operations; G is integer
     k_gs_dots<<<g, kGsThreads, 0, c->st>>>(n, nv, k.V, w, c->partials, k.gram, c->ticket, c->dsc, c->hsc);
   }
   RICH_LAUNCH_CHECK();
