@@ -2041,9 +2041,11 @@ void amg_free(rich_ctx* c) {
   H.vc_out = nullptr;
   H.vc_calls = 0;
   H.vc_off = false;
-  if (H.fcg_exec) cudaGraphExecDestroy(H.fcg_exec);
-  H.fcg_exec = nullptr;
-  H.fcg_nodes = 0;
+  for (int q = 0; q < 2; ++q) {
+    if (H.fcg_exec[q]) cudaGraphExecDestroy(H.fcg_exec[q]);
+    H.fcg_exec[q] = nullptr;
+    H.fcg_nodes[q] = 0;
+  }
   H.fcg_off = false;
   as_free(c);
   H.built = false;

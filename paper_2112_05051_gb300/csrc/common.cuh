@@ -269,9 +269,11 @@ struct Hierarchy {
   void* vc_out = nullptr;
   int vc_calls = 0;
   bool vc_off = false;            // capture failed: direct launches for this hierarchy
-  // FCG's iterations as one graph (a WHILE loop, solve.cu); kernels per iteration
-  cudaGraphExec_t fcg_exec = nullptr;
-  long long fcg_nodes = 0;
+  // FCG's iterations as one graph (a WHILE loop, solve.cu); kernels per iteration.  The number
+  // of stacked problems is part of a captured loop: [0] one problem, [1] the batch's nbatch
+  // (a batch context reaches both: its own step, and a lone solve or step over the stack).
+  cudaGraphExec_t fcg_exec[2] = {nullptr, nullptr};
+  long long fcg_nodes[2] = {0, 0};
   bool fcg_off = false;
   // one-level additive Schwarz (precond = RICH_PRECOND_AS): ILU(0) diagonals and
   // subdomain solutions (hierarchy precision), FP32 staging of r and z in MIXED

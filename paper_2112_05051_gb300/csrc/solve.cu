@@ -1718,6 +1718,9 @@ static int fcg_body(rich_ctx* c, int S, cudaGraphConditionalHandle loop, int loo
   return RICH_OK;
 }
 
+// Which of the hierarchy's loops serves S problems (S is 1 or the context's nbatch).
+static int fcg_slot(int S) { return S > 1; }
+
 // Captures the loop: a WHILE node whose body is fcg_body.  As for the V-cycle, on a private
 // stream after a direct application; a failure leaves direct launches.
 template <class T>
@@ -1755,16 +1758,17 @@ static void fcg_capture(rich_ctx* c, int S) {
     cudaGraph_t captured = nullptr;
     e = cudaStreamEndCapture(cs, &captured);  // the body itself
   }
+  cudaGraphExec_t& exec = H.fcg_exec[fcg_slot(S)];
   if (e == cudaSuccess && rc == RICH_OK) {
-    e = cudaGraphInstantiate(&H.fcg_exec, graph, 0);
-    if (e == cudaSuccess) H.fcg_nodes = after - before;
-    else H.fcg_exec = nullptr;
+    e = cudaGraphInstantiate(&exec, graph, 0);
+    if (e == cudaSuccess) H.fcg_nodes[fcg_slot(S)] = after - before;
+    else exec = nullptr;
   }
   if (graph) cudaGraphDestroy(graph);
   if (cs) cudaStreamDestroy(cs);
-  if (e != cudaSuccess || rc != RICH_OK || !H.fcg_exec) {
+  if (e != cudaSuccess || rc != RICH_OK || !exec) {
     cudaGetLastError();
-    H.fcg_exec = nullptr;
+    exec = nullptr;
     H.fcg_off = true;
   }
 }
@@ -1798,14 +1802,14 @@ static int fcg_solve(rich_ctx* c, int S, const double* b, double* x, const rich_
   for (;;) {
     if (graphs && !H.fcg_off && H.vc_calls > 0) {  // a first application launched directly
       if (waited && !running()) break;
-      if (!H.fcg_exec) fcg_capture<T>(c, S);
-      if (H.fcg_exec) {
+      if (!H.fcg_exec[fcg_slot(S)]) fcg_capture<T>(c, S);
+      if (H.fcg_exec[fcg_slot(S)]) {
         const int it0 = waited ? out[0].it : 0;
-        RICH_CUDA(cudaGraphLaunch(H.fcg_exec, c->st));
+        RICH_CUDA(cudaGraphLaunch(H.fcg_exec[fcg_slot(S)], c->st));
         RICH_CUDA(cudaStreamSynchronize(c->st));
         int most = 1;
         for (int s = 0; s < S; ++s) most = std::max(most, out[s].it - it0);
-        count_launches(most * H.fcg_nodes);
+        count_launches(most * H.fcg_nodes[fcg_slot(S)]);
         break;
       }
     }
@@ -1828,8 +1832,8 @@ int fcg_run(rich_ctx* c, int S, const double* b, double* x, const rich_krylov_op
   const FcgOut* out = static_cast<const FcgOut*>(c->kw.fcg_out);
   int rc = RICH_OK;
   for (int s = 0; s < S; ++s) {
-    res[s] = FcgResult{out[s].rn, out[s].bn, out[s].it,
-                       out[s].reason == kFcgConverged || out[s].reason == kFcgZero ? 0 : out[s].reason};
+    const int r = out[s].reason;  // 0: the loop left the problem unfinished
+    res[s] = FcgResult{out[s].rn, out[s].bn, out[s].it, r == kFcgConverged || r == kFcgZero ? 0 : r ? r : 1};
     if (out[s].reason == kFcgNonfinite) rc = RICH_ENONFINITE;
   }
   return rc;

@@ -1,0 +1,50 @@
+"""One batch context used both ways: step_batch (FCG over nbatch problems, each with its own
+scalars) and the lone calls it inherits, krylov_solve and step (one problem over the whole
+stack), in both orders and with the iterations as a graph (graph = 1) or launched singly
+(graph = 0).  The same kernels run either way, so iterates, counts and statuses agree bit for
+bit; a lone solve also meets its own tolerance on the whole stack."""
+import numpy as np
+import pytest
+
+from paper_2112_05051_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _run(order, graph, prec, nbatch):
+    from paper_2112_05051_gb300 import richards as rb
+    rb.load()
+    grid = synth.Grid(14, 13, 12)
+    ks = np.concatenate([synth.ks_field(grid, 40 + b, 0.5, (4.0, 4.0, 2.0)) for b in range(nbatch)])
+    ctx = rb.BatchContext(grid, nbatch, synth.Soil(), synth.infiltration_bc(), synth.KMEAN_ARITH, ks, precision=prec)
+    opts = rb.default_newton_opts(kind=rb.KRYLOV_FCG, seed=3, coarse_max=100, smooth_levels=2, graph=graph)
+    p = torch.full((ctx.n,), synth.P_INITIAL, dtype=torch.float64, device="cuda")
+    b = torch.randn(ctx.n, generator=torch.Generator().manual_seed(5), dtype=torch.float64).cuda()
+    ctx.jacobian(p - 1.0, 0.25)
+    ctx.amg_setup(opts.amg)
+    out = []
+    for op in order:
+        if op == "batch":
+            status, st = ctx.step_batch(p, 0.25, opts)
+            out.append((status, [s.linear_its for s in st], [s.newton_its for s in st], p.cpu().numpy()))
+        elif op == "step":
+            status, st = ctx.step(p, 0.25, opts, check_status=False)
+            out.append((status, st.linear_its, st.newton_its, p.cpu().numpy()))
+        else:
+            x, y = torch.full_like(b, float("nan")), torch.empty_like(b)
+            status, st = ctx.krylov_solve(b, x, kind=rb.KRYLOV_FCG, check_status=False)
+            ctx.jacobian_apply(x, y)
+            assert status == 0 and float((y - b).norm()) <= 1.01e-7 * float(b.norm())
+            out.append((status, st.iterations, st.res, x.cpu().numpy()))
+    ctx.close()
+    return out
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("order,nbatch", [(("batch", "solve", "batch", "solve"), 3), (("solve", "batch", "solve"), 3),
+                                          (("step", "batch", "step"), 2), (("batch", "solve"), 1)])
+def test_batch_and_lone_solves_on_one_context(order, nbatch, prec):
+    for a, b in zip(_run(order, 0, prec, nbatch), _run(order, 1, prec, nbatch)):
+        assert a[:3] == b[:3]
+        np.testing.assert_array_equal(a[3], b[3])
