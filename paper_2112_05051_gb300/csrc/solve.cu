@@ -1554,6 +1554,7 @@ __global__ void __launch_bounds__(kFcgThreads) k_fcg_begin(long long ns, const d
     s.target = eta * s.bn;
     if (!isfinite(s.bn)) s.reason = kFcgNonfinite;
     else if (!(s.bn > 0)) s.reason = kFcgZero;
+    else if (maxit < 1) s.reason = 1;  // a batch's limit of no iterations at all: x = 0, not converged
     dev->seg[threadIdx.x] = s;
     out[threadIdx.x] = FcgOut{s.rn, s.bn, 0, s.reason};
   }

@@ -48,3 +48,22 @@ def test_batch_and_lone_solves_on_one_context(order, nbatch, prec):
     for a, b in zip(_run(order, 0, prec, nbatch), _run(order, 1, prec, nbatch)):
         assert a[:3] == b[:3]
         np.testing.assert_array_equal(a[3], b[3])
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+def test_batch_without_iterations(graph):
+    """maxit = 0: no iteration is made, also not by a loop captured before, and no problem moves."""
+    from paper_2112_05051_gb300 import richards as rb
+    rb.load()
+    grid = synth.Grid(9, 8, 7)
+    ctx = rb.BatchContext(grid, 2, synth.Soil(), synth.infiltration_bc(), synth.KMEAN_ARITH, None)
+    kw = dict(kind=rb.KRYLOV_FCG, seed=3, coarse_max=100, graph=graph)
+    p = torch.full((ctx.n,), synth.P_INITIAL, dtype=torch.float64, device="cuda")
+    for warm in (False, True):
+        if warm:  # a step whose solves run (and capture) the loop, wherever it ends
+            assert max(s.linear_its for s in ctx.step_batch(p, 0.25, rb.default_newton_opts(**kw))[1]) > 2
+        before = p.clone()
+        status, st = ctx.step_batch(p, 0.25, rb.default_newton_opts(maxit=0, **kw))
+        assert status == [-4, -4] and [s.linear_its for s in st] == [0, 0]
+        assert torch.equal(p, before)
+    ctx.close()
