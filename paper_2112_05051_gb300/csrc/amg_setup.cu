@@ -1072,11 +1072,18 @@ __global__ void k_pl_sort(int nslice, const long long* __restrict__ sptr, int2* 
   }
 }
 
-// The same for long entries, a warp each: up to kPlSort pairs are ranked in shared memory
-// (an A entry contributes one product to an entry of C, so the keys are distinct).
+// The same for the entries of wide rows, which a block's warps file out of order: a warp
+// per entry, up to kPlSort pairs ranked in shared memory (an A entry contributes one product
+// to an entry of C, so the keys are distinct).  A longer entry is written anew, in order:
+// the row's A entries 32 at a time, each looking for the entry's column in its B row.
+// (64^3, setup with matching aggregates of 8 / of 1024 cells, those entries sorted by one
+// lane: 110 / 48 ms, 67 and 22 of them here; 49 / 25 ms so.)
 constexpr int kPlSort = 512;
-__global__ void __launch_bounds__(32 * kPlWarps) k_pl_rank(int nnz, const int* __restrict__ cnt,
-                                                           const int* __restrict__ place,
+__global__ void __launch_bounds__(32 * kPlWarps) k_pl_rank(int nrows, const int* __restrict__ arp,
+                                                           const int* __restrict__ acol, const int* __restrict__ brp,
+                                                           const int* __restrict__ bcol, const int* __restrict__ crp,
+                                                           const int* __restrict__ ccol, int nnz,
+                                                           const int* __restrict__ cnt, const int* __restrict__ place,
                                                            const long long* __restrict__ sptr,
                                                            int2* __restrict__ pairs) {
   __shared__ int2 a_all[kPlWarps][kPlSort];
@@ -1087,14 +1094,25 @@ __global__ void __launch_bounds__(32 * kPlWarps) k_pl_rank(int nnz, const int* _
     if (len < 2) continue;
     int2* p = pairs + sptr[at / kSellC] + at % kSellC;
     if (len > kPlSort) {
-      if (lane == 0)
-        for (int t = 1; t < len; ++t) {
-          const int2 k = p[(long long)t * kSellC];
-          int v = t - 1;
-          for (; v >= 0 && p[(long long)v * kSellC].x > k.x; --v)
-            p[(long long)(v + 1) * kSellC] = p[(long long)v * kSellC];
-          p[(long long)(v + 1) * kSellC] = k;
+      int row = 0, end = nrows;  // crp[row] <= q < crp[row + 1]
+      while (end - row > 1) {
+        const int mid = (row + end) >> 1;
+        if (crp[mid] <= q) row = mid; else end = mid;
+      }
+      const int c = ccol[q], a1 = arp[row + 1];
+      int t = 0;
+      for (int e0 = arp[row]; e0 < a1; e0 += 32) {
+        const int e = e0 + lane;
+        int f = -1;
+        if (e < a1) {
+          const int b1 = brp[acol[e] + 1];
+          f = find_col(bcol, brp[acol[e]], b1, c);
+          if (f == b1 || bcol[f] != c) f = -1;
         }
+        const unsigned m = __ballot_sync(0xffffffffu, f >= 0);
+        if (f >= 0) p[(long long)(t + __popc(m & ((1u << lane) - 1))) * kSellC] = make_int2(e, f);
+        t += __popc(m);
+      }
       continue;
     }
     for (int t = lane; t < len; t += 32) a[t] = p[(long long)t * kSellC];
@@ -1644,10 +1662,10 @@ static int plist_build(rich_ctx* c, const Csr<double>& A, const Csr<double>& B, 
     if (wide) list(k_plist<true, true>);
     else list(k_plist<true, false>);
     RICH_LAUNCH_CHECK();
-    // short entries filed by one warp per row are almost in order already
-    if (wide || (double)np > 8.0 * (double)nnz)
-      k_pl_rank<<<std::min((nnz + kPlWarps - 1) / kPlWarps, 64 * kNumSM), 32 * kPlWarps, 0, c->st>>>(nnz, cnt, place,
-                                                                                                   pl.sptr, pl.pairs);
+    // entries filed by one warp per row are almost in order already
+    if (wide)
+      k_pl_rank<<<std::min((nnz + kPlWarps - 1) / kPlWarps, 64 * kNumSM), 32 * kPlWarps, 0, c->st>>>(
+          A.nrows, A.rowptr, A.col, B.rowptr, B.col, C.rowptr, C.col, nnz, cnt, place, pl.sptr, pl.pairs);
     else
       k_pl_sort<<<grid_for(32LL * pl.nslice), kBlock, 0, c->st>>>(pl.nslice, pl.sptr, pl.pairs);
     RICH_LAUNCH_CHECK();
