@@ -1016,13 +1016,20 @@ __global__ void __launch_bounds__(32 * kPlWarps) k_plist(int nrows, const int* _
 // The lists' layout from the entries' counts: a window of kSellSigma entries per block,
 // bucketed by decreasing count (ties in any order: an entry's sum does not depend on its
 // place).  place[q] is q's position, perm its inverse, slots the slices' sizes.
-constexpr int kPlBuckets = 512;  // longer entries share the first bucket
+// Buckets: one per count below 256, above it 32 per power of two, so that a slice's padding
+// stays within a 32nd of its entries; counts from 2^16 on share the first bucket.
+constexpr int kPlBuckets = 512;
+__device__ __forceinline__ int pl_bucket(int l) {
+  if (l < 256) return kPlBuckets - 1 - l;
+  const int e = 31 - __clz(l);
+  return kPlBuckets - 1 - min(256 + ((e - 8) << 5) + ((l >> (e - 5)) & 31), kPlBuckets - 1);
+}
 __global__ void __launch_bounds__(kSellSigma) k_pl_shape(int nnz, const int* __restrict__ cnt, int nslice,
                                                          int* __restrict__ perm, int* __restrict__ place,
                                                          int* __restrict__ slots) {
   __shared__ int first[kPlBuckets], wsum[kPlBuckets / 32], wide[kSellSigma / kSellC];
   const int t = threadIdx.x, w0 = blockIdx.x * kSellSigma, q = w0 + t;
-  const int l = q < nnz ? cnt[q] : 0, b = kPlBuckets - 1 - min(l, kPlBuckets - 1);
+  const int l = q < nnz ? cnt[q] : 0, b = pl_bucket(l);
   if (t < kPlBuckets) first[t] = 0;
   if (t < kSellSigma / kSellC) wide[t] = 0;
   __syncthreads();
@@ -1134,42 +1141,63 @@ __global__ void k_sum_rows_ll(int n, const int* __restrict__ u, unsigned long lo
   if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
 }
 
-// c[q] = sum of a[x] * b[y] over q's pairs, in their order: no search, no atomics, the same
-// sum every refresh.  A warp per slice, a thread per entry, four pairs in flight.
+// acc + the products of U columns of a slice from p on, all loads in flight together; of
+// the first `left` of them if PRED (warp-uniform).  The multiply-add is explicit: a sum may
+// not depend on which of these forms its pairs fall into (the slice's width decides).
+template <class T, int U, bool PRED>
+__device__ __forceinline__ T pl_sum(const int2* __restrict__ p, int left, const T* __restrict__ aval,
+                                    const T* __restrict__ bval, T acc) {
+  int2 k[U];
+  T a[U], b[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) k[u] = !PRED || u < left ? __ldcs(&p[u * kSellC]) : make_int2(-1, 0);
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    a[u] = k[u].x >= 0 ? aval[k[u].x] : T(0);
+    b[u] = k[u].x >= 0 ? bval[k[u].y] : T(0);
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (k[u].x >= 0) acc = fma(a[u], b[u], acc);
+  return acc;
+}
+
+// c[q] = sum of a[x] * b[y] over q's pairs: no search, no atomics, the same sum every
+// refresh.  A warp per slice, a thread per entry, four pairs in flight, summed in their order.
 // Bound: FP64 one FMA per pair, FP32 HBM (8 bytes per pair).  128^3 FP64, 176M pairs over
 // three levels: 1270 us with the pairs entry by entry (a thread's own run, 32 sectors per
-// warp and load, and as many steps as the longest of 32 neighbours).
-template <class T>
-__global__ void __launch_bounds__(256) k_galerkin_lists(int nslice, const int* __restrict__ perm,
-                                                        const long long* __restrict__ sptr,
-                                                        const int2* __restrict__ pairs, const T* __restrict__ aval,
-                                                        const T* __restrict__ bval, T* __restrict__ cval) {
-  const int lane = threadIdx.x & 31;
-  for (int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslice; s += (gridDim.x * blockDim.x) >> 5) {
-    const int q = perm[s * kSellC + lane];
-    long long e = sptr[s] + lane;
-    const long long end = sptr[s + 1];
-    T acc = T(0);
-    for (; e + 3 * kSellC < end; e += 4 * kSellC) {  // warp-uniform
-      int2 p[4];
-      T a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) p[u] = __ldcs(&pairs[e + u * kSellC]);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = p[u].x >= 0 ? aval[p[u].x] : T(0);
-        b[u] = p[u].x >= 0 ? bval[p[u].y] : T(0);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (p[u].x >= 0) acc += a[u] * b[u];
-    }
-    for (; e < end; e += kSellC) {
-      const int2 p = __ldcs(&pairs[e]);
-      if (p.x >= 0) acc += aval[p.x] * bval[p.y];
-    }
-    if (q >= 0) cval[q] = acc;
+// warp and load, and as many steps as the longest of 32 neighbours), 880 us so.
+// SPLIT: a block per slice, for products whose slices are few and long, where a warp's chain
+// of loads would be the time: its warps take the columns eight at a time in turn (an entry's
+// split is its own, whatever slice it shares) and their sums are added in order.  48^3 FP64,
+// all products: 328 us without, 112 us so; matching aggregates of 1024 cells on 64^3: 657
+// and 227 us.
+template <class T, bool SPLIT>
+__global__ void __launch_bounds__(32 * kPlWarps) k_galerkin_lists(int nslice, const int* __restrict__ perm,
+                                                                  const long long* __restrict__ sptr,
+                                                                  const int2* __restrict__ pairs,
+                                                                  const T* __restrict__ aval,
+                                                                  const T* __restrict__ bval, T* __restrict__ cval) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, s = SPLIT ? blockIdx.x : blockIdx.x * kPlWarps + w;
+  if (s >= nslice) return;  // (SPLIT: no block of the grid)
+  const int2* p = pairs + sptr[s] + lane;
+  const int width = (int)((sptr[s + 1] - sptr[s]) / kSellC);
+  T acc = T(0);
+  if (SPLIT) {
+    __shared__ T part[kPlWarps][kSellC];
+    for (int c = 8 * w; c < width; c += 8 * kPlWarps)
+      acc = pl_sum<T, 8, true>(p + (long long)c * kSellC, width - c, aval, bval, acc);
+    part[w][lane] = acc;
+    __syncthreads();
+    if (w > 0) return;
+    for (int v = 1; v < kPlWarps; ++v) acc += part[v][lane];
+  } else {
+    int c = 0;
+    for (; c + 4 <= width; c += 4) acc = pl_sum<T, 4, false>(p + (long long)c * kSellC, 4, aval, bval, acc);
+    for (; c < width; ++c) acc = pl_sum<T, 1, false>(p + (long long)c * kSellC, 1, aval, bval, acc);
   }
+  const int q = perm[s * kSellC + lane];
+  if (q >= 0) cval[q] = acc;
 }
 
 // ---------------------------------------------------------------- coarsest level: dense inverse
@@ -1687,8 +1715,15 @@ static int spgemm_numeric_t(rich_ctx* c, const Csr<double>& A, const T* aval, co
                  4.0 * ((double)C.nnz + 1) + 8.0 * (double)pl->np +
                      (double)sizeof(T) * ((double)A.nnz + (double)B.nnz + (double)C.nnz),
                  2.0 * (double)pl->np);
-    k_galerkin_lists<T><<<(pl->nslice + 7) / 8, 256, 0, c->st>>>(pl->nslice, pl->perm, pl->sptr, pl->pairs, aval, bval,
-                                                                cval);
+    auto run = [&](auto kernel, int blocks) {
+      kernel<<<blocks, 32 * kPlWarps, 0, c->st>>>(pl->nslice, pl->perm, pl->sptr, pl->pairs, aval, bval, cval);
+    };
+    // a warp per slice below 48 of them per SM does not hide its loads' latency (64^3, entries
+    // of 40 products in 3146 slices: 3 times longer); a pair or two per warp is not worth it
+    if (pl->nslice < 48 * kNumSM && (double)pl->np > 8.0 * (double)C.nnz)
+      run(k_galerkin_lists<T, true>, pl->nslice);
+    else
+      run(k_galerkin_lists<T, false>, (pl->nslice + kPlWarps - 1) / kPlWarps);
     RICH_LAUNCH_CHECK();
     return RICH_OK;
   }
