@@ -22,6 +22,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "plist_limit.h"
 
 namespace rich {
 
@@ -1653,8 +1654,7 @@ static int plist_build(rich_ctx* c, const Csr<double>& A, const Csr<double>& B, 
   size_t fr = 0, tot = 0;
   RICH_CUDA(cudaMemGetInfo(&fr, &tot));
   fr += pool_slack();  // blocks freed into the pool count as free here
-  double need = 8.0 * (double)np + 24.0 * ((double)C.nnz + 1);  // lists, offsets and the build's scratch
-  if (need > 0.5 * (double)fr) return RICH_OK;
+  if (!plist_fits((double)np, (double)C.nnz, (double)fr)) return RICH_OK;
   const int nnz = (int)C.nnz;
   pl.nslice = (nnz + kSellC - 1) / kSellC;
   int *cnt = nullptr, *place = nullptr, *slots = nullptr;
@@ -1681,7 +1681,9 @@ static int plist_build(rich_ctx* c, const Csr<double>& A, const Csr<double>& B, 
   long long total = 0;
   RICH_CUDA(cudaMemcpyAsync(&total, pl.sptr + pl.nslice, sizeof(total), cudaMemcpyDeviceToHost, c->st));
   RICH_CUDA(cudaStreamSynchronize(c->st));
-  if (dalloc(&pl.pairs, total) != RICH_OK) {  // padding beyond what was free: the refresh searches
+  if (!plist_fits((double)total, (double)C.nnz, (double)fr)) {  // padded beyond the limit: the refresh searches
+    plist_free(pl);
+  } else if (dalloc(&pl.pairs, total) != RICH_OK) {  // or beyond what is left
     cudaGetLastError();
     plist_free(pl);
   } else {
