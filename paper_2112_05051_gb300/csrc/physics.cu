@@ -159,15 +159,16 @@ __device__ __forceinline__ void asm_face(int kmean, int axis, const GridP& g, do
 
 // J (7 planes) and A_aux (7 planes) at the pressure K, K' and s' belong to.  A thread
 // marches upward through its cell of every layer of its block's range (blocks take equal
-// ranges of the units (chunk of the plane, layer)), so a vertical face is computed once;
-// J7b / A7b, if not NULL, receive the caller's copies in the same pass.
+// ranges of the units (chunk of the columns, layer)), so a vertical face is computed once;
+// J7b / A7b, if not NULL, receive the caller's copies in the same pass.  The columns are
+// those of the plane cut into runs of `len` layers (nz, or 1 for planes that fill no warp).
 // Bound: the FP64 pipe (35 to 45 operations per cell) until the 112 bytes per cell it
 // writes bind.  399 x 401 x 19 cells, upstream: one cell per thread with every mean's
 // general form took 700 us, and 105 to copy both stencils out; law, assembly and copies
 // together went from 829 to 456 us.
 constexpr int kAsmThreads = 128;
 template <int KM>
-__global__ void __launch_bounds__(kAsmThreads, 5) k_assemble(GridP g, SoilP so, BCP bc, int kmean, int units,
+__global__ void __launch_bounds__(kAsmThreads, 5) k_assemble(GridP g, SoilP so, BCP bc, int kmean, int units, int len,
                                                           const double* __restrict__ p, const double* __restrict__ K,
                                                           const double* __restrict__ dK,
                                                           const double* __restrict__ dS,
@@ -184,10 +185,11 @@ __global__ void __launch_bounds__(kAsmThreads, 5) k_assemble(GridP g, SoilP so, 
   };
   const int u1 = (int)((blockIdx.x + 1LL) * units / gridDim.x);
   for (int u = (int)((long long)blockIdx.x * units / gridDim.x), run; u < u1; u += run) {
-    const int ch = u / g.nz, k0 = u - ch * g.nz;
-    run = min(u1 - u, g.nz - k0);
-    const int r = ch * (int)blockDim.x + threadIdx.x;
-    if (r >= plane) continue;
+    const int ch = u / len, l0 = u - ch * len;
+    run = min(u1 - u, len - l0);
+    const int col = ch * (int)blockDim.x + threadIdx.x, seg = col / plane, r = col - seg * plane;
+    const int k0 = seg * len + l0;
+    if (k0 >= g.nz) continue;
     const int j = r / g.nx, i = r - j * g.nx;
     long long c = r + (long long)plane * k0;
     int kl = k0 % g.nzs;  // layer within its problem: a batch's problems meet at boundaries
@@ -360,16 +362,21 @@ int jacobian_eval(rich_ctx* c, const double* p, double dt, bool constit_current,
   if (!constit_current) RICH_CHECK(constit_eval(c, p));
   const GridP& g = c->g;
   // chunks of a warp where chunks of kAsmThreads cells would leave SMs without a block
+  // and, so that narrow planes fill their warps, a thread per cell below 32 columns (every
+  // vertical face twice: upstream, 1 x 1 x 100000 cells 155 us marched and 21 so, 4 x 4 x 20000
+  // 101 and 62, 7 x 9 x 2000 29 and 35)
   const long long plane = (long long)g.nx * g.ny;
-  const int threads = (plane + kAsmThreads - 1) / kAsmThreads * g.nz < 2 * kNumSM ? 32 : kAsmThreads;
-  const int units = (int)((plane + threads - 1) / threads * g.nz);
+  const int len = plane < 32 ? 1 : g.nz;
+  const long long cols = plane * (g.nz / len);
+  const int threads = (cols + kAsmThreads - 1) / kAsmThreads * len < 2 * kNumSM ? 32 : kAsmThreads;
+  const int units = (int)((cols + threads - 1) / threads * len);
   const int nb = std::min(units, 20 * kNumSM * 32 / threads);  // 20 warps per SM (registers)
   const double rdt = c->soil.rho_phi / dt;
   {
     const int copies = 1 + (J7b != nullptr) + (A7b != nullptr);
     ProfScope ps("assemble", c->st, (double)g.n * (32.0 + (c->ks ? 8.0 : 0.0) + (copies + 1) * 7 * 8.0));
     auto run = [&](auto kernel) {
-      kernel<<<nb, threads, 0, c->st>>>(g, c->soil, c->bc, c->kmean, units, p, c->K, c->dK, c->dS, c->ks, rdt, c->J7,
+      kernel<<<nb, threads, 0, c->st>>>(g, c->soil, c->bc, c->kmean, units, len, p, c->K, c->dK, c->dS, c->ks, rdt, c->J7,
                                         c->A7, J7b, A7b);
     };
     switch (c->kmean) {
