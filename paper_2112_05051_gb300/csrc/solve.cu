@@ -16,7 +16,7 @@
 #include <mutex>
 #include <vector>
 
-#include "common.cuh"
+#include "gram.cuh"
 
 namespace rich {
 
@@ -1129,273 +1129,6 @@ int vcycle_apply(rich_ctx* c, const double* r, double* z) {
 }
 
 // ---------------------------------------------------------------- Krylov kernels (FP64)
-
-// ---- Gram-Schmidt of FGMRES, in two passes over the basis (classical Gram-Schmidt with
-// the second projection taken from the basis' Gram matrix: Swirydowicz, Langou, Ananthan,
-// Yang, Thomas, "Low synchronization Gram-Schmidt and generalized minimal residual
-// algorithms", 2021).  With G = V^T V, whose last row is the new vector's dots, the
-// coefficients of two projections are h = h1 + (I - G) h1, h1 = V^T w, so the basis is read
-// once for the dots (with w and with the newest vector) and once for w - V h; V stays
-// orthogonal to about ten units of rounding.  Bound: the FP64 pipe, two operations per basis
-// element, one in either pass (explicit second projections take four and read the basis four
-// times), and in the dots the loads.  Where w - V h loses more than 1e-2 of w's norm, the host
-// asks for one explicit pass more.
-// 128^3, FGMRES(30): 667 us per iteration with two explicit projections, 545 with a Gram matrix
-// summed in FP64, 518 with one summed in integers (dots at ten vectors: 101 -> 75 us).
-constexpr int kGsThreads = 256;
-// Of the dots: one wave at 80 registers (4 per SM with 64 registers: 93 us against 83).
-constexpr int kGsBlocks = 3 * kNumSM;
-constexpr int kGsUpdateBlocks = 4 * kNumSM;  // of the update: one wave (8 per SM left a second, 59 us against 46)
-constexpr int kGsTile = 4;             // basis vectors per sweep over a block's elements
-constexpr int kGsLd = 64;              // row length of the Gram matrix
-// Device scalars of an iteration (restart <= 63): h in [0, j], ||w - V h|| and its reciprocal.
-constexpr int kSlotNorm = 63, kSlotInv = 64;
-
-// Sums of 8 values over a warp by halving: after the exchange at distances 16, 8 and 4 a
-// lane holds one value, summed on at 2 and 1: 9 additions instead of 40.  The lane's value
-// is number lane >> 2.
-__device__ __forceinline__ double warp_sum8(double (&a)[8]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 4; k > 0; k >>= 1) {
-    const bool up = lane & (4 * k);
-#pragma unroll
-    for (int q = 0; q < k; ++q) {
-      const double keep = up ? a[q + k] : a[q], send = up ? a[q] : a[q + k];
-      a[q] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * k);
-    }
-  }
-  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
-  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
-  return a[0];
-}
-
-// G's entries are summed in integers.  The basis is normalised, |v| <= 1, so an entry in
-// units of 2^-60 is h 2^30 + l with |h| <= 2^30 and |l| <= 2^29, and a product is four 32-bit
-// multiply-adds into three 64-bit sums; those and the split (20 integer instructions) run
-// beside the FP64 pipe, which is left with the dots with w alone.  An entry's rounding, at
-// most 2^-61, is all the error: |G - V^T V| measured 7e-19 on random and smooth vectors of
-// 300k entries and 1.4e-16 at worst (a constant against one cell with a tail of 1e-18),
-// where FP64 sums leave up to 8e-17, the rounding of a diagonal entry.
-struct UnitFixed {
-  int h, l;
-};
-__device__ __forceinline__ UnitFixed unit_fixed(double v) {
-  const int hi = __double2hiint(v), sg = hi >> 31;
-  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu, s = min(1023u - e, 63u);
-  // twice the magnitude in units of 2^-60, shifted, then rounded to nearest
-  unsigned long long m = (unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32;
-  m |= (unsigned)__double2loint(v);
-  m = (((m << 9) >> s) + 1) >> 1;
-  const int h = (int)((m + (1u << 29)) >> 30), l = (int)((unsigned)m - ((unsigned)h << 30));
-  return {(h ^ sg) - sg, (l ^ sg) - sg};
-}
-// Sums of products: hh 2^-60 + x 2^-90 + ll 2^-120, carried after every kUnitRun of
-// them.  |ll| grows by 2^58 a product; |x| stays below 2 2^29 sqrt(16) 2^30 and |hh| below
-// 2^60 because sum h^2 <= 2^60 over a whole vector.
-constexpr int kUnitRun = 16;
-struct UnitSum {
-  long long hh = 0, x = 0, ll = 0;
-  __device__ __forceinline__ void add(UnitFixed a, UnitFixed b) {
-    hh += (long long)a.h * b.h;
-    x += (long long)a.h * b.l;
-    x += (long long)a.l * b.h;
-    ll += (long long)a.l * b.l;
-  }
-  __device__ __forceinline__ void carry() {
-    x += ll >> 30;
-    ll &= (1 << 30) - 1;
-    hh += x >> 30;
-    x &= (1 << 30) - 1;
-  }
-  // The sum in units of 2^-62, rounded to one of them (a thread's; one conversion).
-  __device__ __forceinline__ double value() {
-    carry();
-    return (double)(4 * hh + ((x + (1 << 27)) >> 28));
-  }
-};
-
-// Copies of 8 bytes into the thread's own words of shared memory, kGsStages elements deep:
-// the loads of the next elements run under this one's arithmetic and hold no registers
-// (with plain loads the warps waited for memory two thirds of the time: 147 us, ten vectors).
-constexpr int kGsStages = 3;
-typedef double GsStage[kGsTile + 2][kGsThreads];
-__device__ __forceinline__ void copy8(double* dst, const double* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-
-// The block's sums over its elements of M basis vectors (from v0) times w and vj, into
-// a[q] and a[4 + q].
-template <int M>
-__device__ __forceinline__ void gs_tile(long long n, const double* v0, const double* w, const double* vj,
-                                        GsStage (&st)[kGsStages], double (&a)[8]) {
-  const long long stride = (long long)gridDim.x * kGsThreads;
-  const int t = threadIdx.x;
-  auto fetch = [&](int slot, long long i) {
-    if (i < n) {
-#pragma unroll
-      for (int q = 0; q < M; ++q) copy8(&st[slot][q][t], v0 + q * n + i);
-      copy8(&st[slot][kGsTile][t], w + i);
-      copy8(&st[slot][kGsTile + 1][t], vj + i);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  long long i = blockIdx.x * (long long)kGsThreads + t;
-#pragma unroll
-  for (int k = 0; k < kGsStages; ++k) fetch(k, i + k * stride);
-  UnitSum g[M];
-  int run = 0, slot = 0;
-#pragma unroll 1
-  for (; i < n; i += stride) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(kGsStages - 1) : "memory");
-    double p[M];
-    const double w0 = st[slot][kGsTile][t], x0 = st[slot][kGsTile + 1][t];
-#pragma unroll
-    for (int q = 0; q < M; ++q) p[q] = st[slot][q][t];
-    const UnitFixed f = unit_fixed(x0);
-#pragma unroll
-    for (int q = 0; q < M; ++q) {
-      a[q] = fma(p[q], w0, a[q]);
-      g[q].add(unit_fixed(p[q]), f);
-    }
-    if (++run == kUnitRun) {
-#pragma unroll
-      for (int q = 0; q < M; ++q) g[q].carry();
-      run = 0;
-    }
-    fetch(slot, i + kGsStages * stride);  // into the words just read
-    slot = slot == kGsStages - 1 ? 0 : slot + 1;
-  }
-#pragma unroll
-  for (int q = 0; q < M; ++q) a[4 + q] = g[q].value();
-}
-
-// h1 = V^T w and the newest row of G = V^T V (nv vectors, vj = V[nv - 1]); the last block
-// to finish forms h and leaves it at s[0, nv) and in the pinned mirror.
-__global__ void __launch_bounds__(kGsThreads, 3) k_gs_dots(long long n, int nv, const double* __restrict__ V,
-                                                        const double* __restrict__ w, double* __restrict__ part,
-                                                        double* __restrict__ gram, unsigned* __restrict__ ticket,
-                                                        double* __restrict__ s, double* __restrict__ mirror) {
-  constexpr int W = kGsThreads / 32;
-  __shared__ double sh[W][2 * kGsTile];
-  __shared__ double tot[2 * kGsLd];
-  __shared__ GsStage st[kGsStages];
-  __shared__ bool last;
-  const double* vj = V + (long long)(nv - 1) * n;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int q0 = 0; q0 < nv; q0 += kGsTile) {
-    double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const double* v0 = V + (long long)q0 * n;
-    const int m = min(kGsTile, nv - q0);
-    if (m == 4) gs_tile<4>(n, v0, w, vj, st, a);
-    else if (m == 3) gs_tile<3>(n, v0, w, vj, st, a);
-    else if (m == 2) gs_tile<2>(n, v0, w, vj, st, a);
-    else gs_tile<1>(n, v0, w, vj, st, a);
-    const double r = warp_sum8(a);
-    if ((lane & 3) == 0) sh[wid][lane >> 2] = r;
-    __syncthreads();
-    if (threadIdx.x < 8 && (threadIdx.x & 3) < m) {
-      double t = 0.0;
-      for (int k = 0; k < W; ++k) t += sh[k][threadIdx.x];
-      const int q = (threadIdx.x >> 2) * kGsLd + q0 + (threadIdx.x & 3);
-      part[(long long)q * gridDim.x + blockIdx.x] = t;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x < 8) __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  for (int t = wid; t < 2 * nv; t += W) {
-    const int q = t < nv ? t : kGsLd + t - nv;
-    double a = 0.0;
-    for (int k = lane; k < (int)gridDim.x; k += 32) a += __ldcg(&part[(long long)q * gridDim.x + k]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if (lane == 0) tot[q] = t < nv ? a : a * 0x1p-62;
-  }
-  __syncthreads();
-  if (threadIdx.x < nv)
-    gram[(nv - 1) * kGsLd + threadIdx.x] = gram[threadIdx.x * kGsLd + nv - 1] = tot[kGsLd + threadIdx.x];
-  __syncthreads();
-  for (int i = wid; i < nv; i += W) {  // h_i = h1_i + sum_q (I - G)_iq h1_q
-    double d = 0.0;
-    for (int q = lane; q < nv; q += 32) d = fma((q == i ? 1.0 : 0.0) - gram[i * kGsLd + q], tot[q], d);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
-    if (lane == 0) s[i] = mirror[i] = tot[i] + d;
-  }
-  if (threadIdx.x == 0) *ticket = 0;
-}
-
-// out = w - V h (w may be out) and its norm: the last block leaves ||out|| and 1/||out||
-// (0 for a zero vector) in the scalars and the norm in the mirror.
-__global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, const double* __restrict__ V,
-                                                          const double* w, double* out, double* __restrict__ part,
-                                                          unsigned* __restrict__ ticket, double* __restrict__ s,
-                                                          double* __restrict__ mirror) {
-  __shared__ double hs[kGsLd];
-  __shared__ bool last;
-  for (int q = threadIdx.x; q < nv; q += kGsThreads) hs[q] = s[q];
-  __syncthreads();
-  const long long stride = (long long)gridDim.x * kGsThreads;
-  double acc[1] = {0.0};
-  long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x;
-  for (; i + stride < n; i += 2 * stride) {
-    double t = w[i], u = w[i + stride];
-    const double* v = V + i;
-#pragma unroll 4
-    for (int q = 0; q < nv; ++q, v += n) {
-      t = fma(-hs[q], v[0], t);
-      u = fma(-hs[q], v[stride], u);
-    }
-    out[i] = t;
-    out[i + stride] = u;
-    acc[0] = fma(t, t, acc[0]);
-    acc[0] = fma(u, u, acc[0]);
-  }
-  if (i < n) {
-    double t = w[i];
-#pragma unroll 4
-    for (int q = 0; q < nv; ++q) t = fma(-hs[q], V[(long long)q * n + i], t);
-    out[i] = t;
-    acc[0] = fma(t, t, acc[0]);
-  }
-  block_sum<1>(acc);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = acc[0];
-    __threadfence();
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  acc[0] = 0.0;
-  for (int k = threadIdx.x; k < (int)gridDim.x; k += kGsThreads) acc[0] += __ldcg(&part[k]);
-  block_sum<1>(acc);
-  if (threadIdx.x == 0) {
-    const double h = sqrt(acc[0]);
-    s[kSlotNorm] = mirror[kSlotNorm] = h;
-    s[kSlotInv] = h > 0 ? 1.0 / h : 0.0;
-    *ticket = 0;
-  }
-}
-
-// V = f src (f from the device if fdev), and the V-cycle's right-hand side with it (scaled
-// by sc, if given).
-template <class T>
-__global__ void k_stage(long long n, const double* src, const double* __restrict__ fdev, double f, double* V,
-                        const T* __restrict__ sc, T* __restrict__ b) {
-  if (fdev) f = *fdev;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const double v = f * src[i];
-    V[i] = v;
-    if (b) b[i] = sc ? sc[i] * (T)v : (T)v;
-  }
-}
 
 // y += sign * sum_q coef[q] V[q]
 __global__ void k_multiaxpy(long long n, int nv, const double* __restrict__ V, const double* __restrict__ coef,
