@@ -300,6 +300,7 @@ struct KrylovWork {
   double* w = nullptr;
   double* hcoef = nullptr;  // device coefficients (m+1)
   double* gram = nullptr;   // V^T V of FGMRES' basis (64 x 64)
+  unsigned* peak = nullptr; // high words of the basis vectors' largest entries (64)
   void* fcg = nullptr;      // FCG's scalars on the device (FcgDev)
   void* fcg_out = nullptr;  // and what the host reads of them (pinned)
   int fail_reason = 0;      // last failure: 0 none, FCG 1 maxit, 2 (p, J p) <= 0, 3 residual growth;

@@ -44,29 +44,41 @@ __device__ __forceinline__ double warp_sum8(double (&a)[8]) {
   return a[0];
 }
 
-// G's entries are summed in integers.  The basis is normalised, |v| <= 1, so an entry in
-// units of 2^-60 is h 2^30 + l with |h| <= 2^30 and |l| <= 2^29, and a product is four 32-bit
-// multiply-adds into three 64-bit sums; those and the split (20 integer instructions) run
-// beside the FP64 pipe, which is left with the dots with w alone.  An entry's rounding, at
-// most 2^-61, is all the error: |G - V^T V| measured 7e-19 on random and smooth vectors of
-// 300k entries and 1.4e-16 at worst (a constant against one cell with a tail of 1e-18),
-// where FP64 sums leave up to 8e-17, the rounding of a diagonal entry.
+// G's entries are summed in integers, in units of a power of two that follows each vector's
+// largest entry.  With 2^(top - 1023) above every |v|, an entry in units of 2^(top - 1083) is
+// h 2^30 + l with |h| <= 2^30 and |l| <= 2^29, and a product is four 32-bit multiply-adds into
+// three 64-bit sums; those and the split (20 integer instructions) run beside the FP64 pipe,
+// which is left with the dots with w alone.  An entry's rounding, half a unit, is all that
+// the integers lose, and like entries lose alike: G_ab is off by up to u_a ||b||_1 + u_b ||a||_1
+// (u half the units).  A spread vector of n cells has a largest entry near n^-1/2, which
+// makes that about 2^-58 for every n (in units of 2^-60 for all vectors it was 2^-60 n^1/2,
+// measured 3.8e-15 for a constant of 16M cells); under a single large entry a tail keeps
+// units of 2^-60.  |G - V^T V| measured on constant, smooth, random and one-sided vectors of
+// 1e3 to 1.6e7 cells 4.4e-16 at most, with a single large entry 6.7e-16, on the bases of 128^3
+// and 399 x 401 x 19 solves 2.2e-16; torch's FP64 dots of the same: 2.2e-16, 7.8e-16 and 2.2e-16.
 struct UnitFixed {
   int h, l;
 };
-__device__ __forceinline__ UnitFixed unit_fixed(double v) {
+// top for a vector whose largest |v| has the high word hi (read as unsigned): h of per-thread
+// sums of m products may not pass 2^60, so the unit leaves c = ceil(log2(m) / 2) bits over it;
+// 1023 at most, which serves every vector of norm 1 (the sum of all h^2 is 2^60 then).
+__device__ __forceinline__ unsigned unit_top(unsigned hi, long long m) {
+  const int c = m > 1 ? (65 - __clzll(m - 1)) / 2 : 0;
+  return (unsigned)min(max((int)(hi >> 20) + 1 + c, 1023 - 40), 1023);
+}
+__device__ __forceinline__ UnitFixed unit_fixed(double v, unsigned top) {
   const int hi = __double2hiint(v), sg = hi >> 31;
-  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu, s = min(1023u - e, 63u);
-  // twice the magnitude in units of 2^-60, shifted, then rounded to nearest
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu, s = min(top - e, 63u);
+  // twice the magnitude in units, shifted, then rounded to nearest
   unsigned long long m = (unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32;
   m |= (unsigned)__double2loint(v);
   m = (((m << 9) >> s) + 1) >> 1;
   const int h = (int)((m + (1u << 29)) >> 30), l = (int)((unsigned)m - ((unsigned)h << 30));
   return {(h ^ sg) - sg, (l ^ sg) - sg};
 }
-// Sums of products: hh 2^-60 + x 2^-90 + ll 2^-120, carried after every kUnitRun of
-// them.  |ll| grows by 2^58 a product; |x| stays below 2 2^29 sqrt(16) 2^30 and |hh| below
-// 2^60 because sum h^2 <= 2^60 over a whole vector.
+// Sums of products: hh 2^-60 + x 2^-90 + ll 2^-120 (in the vectors' scales), carried after
+// every kUnitRun of them.  |ll| grows by 2^58 a product; |x| stays below 2 2^29 sqrt(16) 2^30
+// and |hh| below 2^60 because sum h^2 <= 2^60 over a thread's share of a vector (unit_top).
 constexpr int kUnitRun = 16;
 struct UnitSum {
   long long hh = 0, x = 0, ll = 0;
@@ -82,10 +94,15 @@ struct UnitSum {
     hh += x >> 30;
     x &= (1 << 30) - 1;
   }
-  // The sum in units of 2^-62, rounded to one of them (a thread's; one conversion).
+  // The sum in units of 2^-60, with one conversion of its leading 61 bits (rounded to a fixed
+  // unit of 2^-62, a constant's equal sums were off by 116736 times the same remainder:
+  // 9e-15 for 300k cells).
   __device__ __forceinline__ double value() {
     carry();
-    return (double)(4 * hh + ((x + (1 << 27)) >> 28));
+    const int k = min(__clzll(hh ^ (hh >> 63)) - 2, 30);  // hh 2^k below 2^62
+    const long long r = k < 30 ? 1LL << (29 - k) : 0;
+    return (double)((long long)((unsigned long long)hh << k) + ((x + r) >> (30 - k))) *
+           __hiloint2double((1023 - k) << 20, 0);
   }
 };
 
@@ -100,10 +117,10 @@ __device__ __forceinline__ void copy8(double* dst, const double* src) {
 }
 
 // The block's sums over its elements of M basis vectors (from v0) times w and vj, into
-// a[q] and a[4 + q].
+// a[q] and a[4 + q]; tops and topj: the vectors' unit_top.
 template <int M>
 __device__ __forceinline__ void gs_tile(long long n, const double* v0, const double* w, const double* vj,
-                                        GsStage (&st)[kGsStages], double (&a)[8]) {
+                                        const unsigned* tops, unsigned topj, GsStage (&st)[kGsStages], double (&a)[8]) {
   const long long stride = (long long)gridDim.x * kGsThreads;
   const int t = threadIdx.x;
   auto fetch = [&](int slot, long long i) {
@@ -119,6 +136,9 @@ __device__ __forceinline__ void gs_tile(long long n, const double* v0, const dou
 #pragma unroll
   for (int k = 0; k < kGsStages; ++k) fetch(k, i + k * stride);
   UnitSum g[M];
+  unsigned top[M];
+#pragma unroll
+  for (int q = 0; q < M; ++q) top[q] = tops[q];
   int run = 0, slot = 0;
 #pragma unroll 1
   for (; i < n; i += stride) {
@@ -127,11 +147,11 @@ __device__ __forceinline__ void gs_tile(long long n, const double* v0, const dou
     const double w0 = st[slot][kGsTile][t], x0 = st[slot][kGsTile + 1][t];
 #pragma unroll
     for (int q = 0; q < M; ++q) p[q] = st[slot][q][t];
-    const UnitFixed f = unit_fixed(x0);
+    const UnitFixed f = unit_fixed(x0, topj);
 #pragma unroll
     for (int q = 0; q < M; ++q) {
       a[q] = fma(p[q], w0, a[q]);
-      g[q].add(unit_fixed(p[q]), f);
+      g[q].add(unit_fixed(p[q], top[q]), f);
     }
     if (++run == kUnitRun) {
 #pragma unroll
@@ -149,23 +169,31 @@ __device__ __forceinline__ void gs_tile(long long n, const double* v0, const dou
 // to finish forms h and leaves it at s[0, nv) and in the pinned mirror.
 __global__ void __launch_bounds__(kGsThreads, 3) k_gs_dots(long long n, int nv, const double* __restrict__ V,
                                                         const double* __restrict__ w, double* __restrict__ part,
-                                                        double* __restrict__ gram, unsigned* __restrict__ ticket,
-                                                        double* __restrict__ s, double* __restrict__ mirror) {
+                                                        double* __restrict__ gram, const unsigned* __restrict__ peak,
+                                                        unsigned* __restrict__ ticket, double* __restrict__ s,
+                                                        double* __restrict__ mirror) {
   constexpr int W = kGsThreads / 32;
   __shared__ double sh[W][2 * kGsTile];
   __shared__ double tot[2 * kGsLd];
   __shared__ GsStage st[kGsStages];
   __shared__ bool last;
   const double* vj = V + (long long)(nv - 1) * n;
+  __shared__ unsigned tops[kGsLd];
+  if (threadIdx.x < nv) {
+    const long long threads = (long long)gridDim.x * kGsThreads;
+    tops[threadIdx.x] = unit_top(peak[threadIdx.x], (n + threads - 1) / threads);
+  }
+  __syncthreads();
+  const unsigned topj = tops[nv - 1];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int q0 = 0; q0 < nv; q0 += kGsTile) {
     double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const double* v0 = V + (long long)q0 * n;
     const int m = min(kGsTile, nv - q0);
-    if (m == 4) gs_tile<4>(n, v0, w, vj, st, a);
-    else if (m == 3) gs_tile<3>(n, v0, w, vj, st, a);
-    else if (m == 2) gs_tile<2>(n, v0, w, vj, st, a);
-    else gs_tile<1>(n, v0, w, vj, st, a);
+    if (m == 4) gs_tile<4>(n, v0, w, vj, tops + q0, topj, st, a);
+    else if (m == 3) gs_tile<3>(n, v0, w, vj, tops + q0, topj, st, a);
+    else if (m == 2) gs_tile<2>(n, v0, w, vj, tops + q0, topj, st, a);
+    else gs_tile<1>(n, v0, w, vj, tops + q0, topj, st, a);
     const double r = warp_sum8(a);
     if ((lane & 3) == 0) sh[wid][lane >> 2] = r;
     __syncthreads();
@@ -189,7 +217,13 @@ __global__ void __launch_bounds__(kGsThreads, 3) k_gs_dots(long long n, int nv, 
     for (int k = lane; k < (int)gridDim.x; k += 32) a += __ldcg(&part[(long long)q * gridDim.x + k]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if (lane == 0) tot[q] = t < nv ? a : a * 0x1p-62;
+    if (lane == 0) {
+      if (t >= nv) {  // from the integers' units
+        const int k = 60 + 2 * 1023 - (int)tops[t - nv] - (int)tops[nv - 1];
+        a *= __hiloint2double((1023 - k) << 20, 0);
+      }
+      tot[q] = a;
+    }
   }
   __syncthreads();
   if (threadIdx.x < nv)
@@ -205,18 +239,42 @@ __global__ void __launch_bounds__(kGsThreads, 3) k_gs_dots(long long n, int nv, 
   if (threadIdx.x == 0) *ticket = 0;
 }
 
+// High word of the block's largest value, in thread 0.
+__device__ __forceinline__ unsigned gs_block_max(unsigned hi) {
+  __shared__ unsigned sh[kGsThreads / 32];
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = hi;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int k = 1; k < kGsThreads / 32; ++k) hi = max(hi, sh[k]);
+  return hi;
+}
+__device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+// *peak, zero before: the high word of the largest |f v|, for a cycle's first vector.
+__global__ void __launch_bounds__(kGsThreads) k_gs_peak(long long n, const double* __restrict__ v, double f,
+                                                        unsigned* __restrict__ peak) {
+  unsigned hi = 0;
+  for (long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kGsThreads)
+    hi = max(hi, abs_hi(f * v[i]));
+  hi = gs_block_max(hi);
+  if (threadIdx.x == 0) atomicMax(peak, hi);
+}
+
 // out = w - V h (w may be out) and its norm: the last block leaves ||out|| and 1/||out||
-// (0 for a zero vector) in the scalars and the norm in the mirror.
+// (0 for a zero vector) in the scalars, the norm in the mirror, and in *peak (the next
+// vector's) the high word of the largest |out| / ||out||, or one more.
 __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, const double* __restrict__ V,
                                                           const double* w, double* out, double* __restrict__ part,
-                                                          unsigned* __restrict__ ticket, double* __restrict__ s,
-                                                          double* __restrict__ mirror) {
+                                                          unsigned* __restrict__ peak, unsigned* __restrict__ ticket,
+                                                          double* __restrict__ s, double* __restrict__ mirror) {
   __shared__ double hs[kGsLd];
   __shared__ bool last;
   for (int q = threadIdx.x; q < nv; q += kGsThreads) hs[q] = s[q];
   __syncthreads();
   const long long stride = (long long)gridDim.x * kGsThreads;
   double acc[1] = {0.0};
+  unsigned hi = 0;
   long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x;
   for (; i + stride < n; i += 2 * stride) {
     double t = w[i], u = w[i + stride];
@@ -230,6 +288,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, c
     out[i + stride] = u;
     acc[0] = fma(t, t, acc[0]);
     acc[0] = fma(u, u, acc[0]);
+    hi = max(hi, max(abs_hi(t), abs_hi(u)));
   }
   if (i < n) {
     double t = w[i];
@@ -237,10 +296,13 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, c
     for (int q = 0; q < nv; ++q) t = fma(-hs[q], V[(long long)q * n + i], t);
     out[i] = t;
     acc[0] = fma(t, t, acc[0]);
+    hi = max(hi, abs_hi(t));
   }
   block_sum<1>(acc);
+  hi = gs_block_max(hi);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = acc[0];
+    part[gridDim.x + blockIdx.x] = __hiloint2double((int)hi, 0);
     __threadfence();
     last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
@@ -248,12 +310,18 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, c
   if (!last) return;
   __threadfence();
   acc[0] = 0.0;
-  for (int k = threadIdx.x; k < (int)gridDim.x; k += kGsThreads) acc[0] += __ldcg(&part[k]);
+  hi = 0;
+  for (int k = threadIdx.x; k < (int)gridDim.x; k += kGsThreads) {
+    acc[0] += __ldcg(&part[k]);
+    hi = max(hi, abs_hi(__ldcg(&part[gridDim.x + k])));
+  }
   block_sum<1>(acc);
+  hi = gs_block_max(hi);
   if (threadIdx.x == 0) {
-    const double h = sqrt(acc[0]);
+    const double h = sqrt(acc[0]), inv = h > 0 ? 1.0 / h : 0.0;
     s[kSlotNorm] = mirror[kSlotNorm] = h;
-    s[kSlotInv] = h > 0 ? 1.0 / h : 0.0;
+    s[kSlotInv] = inv;
+    *peak = abs_hi(__hiloint2double((int)hi, -1) * inv);
     *ticket = 0;
   }
 }

@@ -627,6 +627,7 @@ int rich_destroy(rich_ctx* c) {
   dfree(k.w);
   dfree(k.hcoef);
   dfree(k.gram);
+  dfree(k.peak);
   {
     char* d = static_cast<char*>(k.fcg);
     dfree(d);

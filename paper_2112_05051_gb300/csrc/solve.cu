@@ -1173,6 +1173,7 @@ static int ensure_krylov(rich_ctx* c, int m) {
     k.n = n;
   }
   if (m > 0 && !k.gram) RICH_CHECK(dalloc(&k.gram, kGsLd * kGsLd));
+  if (m > 0 && !k.peak) RICH_CHECK(dalloc(&k.peak, kGsLd));
   if (m > 0 && k.m < m) {
     dfree(k.V);
     dfree(k.Z);
@@ -1612,12 +1613,12 @@ static int gs_pass(rich_ctx* c, int nv, const double* w, double* out) {
   const int g = std::min(grid_for(n), kGsBlocks), gu = std::min(grid_for(n, 2 * kBlock), kGsUpdateBlocks);
   {
     ProfScope ps("multidot", c->st, (double)n * 8.0 * (nv + 1), 2.0 * n * nv);  // FP64 operations; G is integer
-    k_gs_dots<<<g, kGsThreads, 0, c->st>>>(n, nv, k.V, w, c->partials, k.gram, c->ticket, c->dsc, c->hsc);
+    k_gs_dots<<<g, kGsThreads, 0, c->st>>>(n, nv, k.V, w, c->partials, k.gram, k.peak, c->ticket, c->dsc, c->hsc);
   }
   RICH_LAUNCH_CHECK();
   {
     ProfScope ps("orth_axpy", c->st, (double)n * 8.0 * (nv + 2), 2.0 * n * (nv + 1));
-    k_gs_update<<<gu, kGsThreads, 0, c->st>>>(n, nv, k.V, w, out, c->partials, c->ticket, c->dsc, c->hsc);
+    k_gs_update<<<gu, kGsThreads, 0, c->st>>>(n, nv, k.V, w, out, c->partials, k.peak + nv, c->ticket, c->dsc, c->hsc);
   }
   RICH_LAUNCH_CHECK();
   return RICH_OK;
@@ -1654,6 +1655,9 @@ static int fgmres(rich_ctx* c, const double* b, double* x, const rich_krylov_opt
   for (;;) {
     std::fill(gv.begin(), gv.end(), 0.0);
     gv[0] = beta;
+    RICH_CUDA(cudaMemsetAsync(k.peak, 0, sizeof(unsigned), c->st));
+    k_gs_peak<<<std::min(grid_for(n), kGsUpdateBlocks), kGsThreads, 0, c->st>>>(n, r0, 1.0 / beta, k.peak);
+    RICH_LAUNCH_CHECK();
     int jdone = 0;
     bool conv = false;
     for (int j = 0; j < m; ++j) {
