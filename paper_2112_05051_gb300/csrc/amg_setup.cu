@@ -1913,25 +1913,14 @@ __global__ void k_stencil4(long long n, const double* __restrict__ A7, Stencil4<
   }
 }
 
-// s = l1^-1/2 and q = l1^1/2 of every row, kept in FP64 for k_scaled: the hardware's
-// approximation (2^-20) and one cubically convergent step y (1 + e/2 + 3/8 e^2),
-// e = 1 - l1 y^2; a norm near the ends of the exponent range takes sqrt() and a division.
+// s = l1^-1/2 and q = l1^1/2 of every row, kept in FP64 for k_scaled.
 __global__ void k_scale_rows(long long n, const double* __restrict__ A7, double* __restrict__ s, double* __restrict__ q,
                              float* __restrict__ s32, float* __restrict__ q32) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     double l1 = A7[i];
 #pragma unroll
     for (int f = 1; f < 7; ++f) l1 -= A7[f * n + i];
-    double r;
-    const unsigned e = ((unsigned)__double2hiint(l1) >> 20) & 0x7ffu;
-    if (__double2hiint(l1) >= 0 && e - 123u < 1800u) {
-      double y;
-      asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(l1));
-      const double d = fma(-l1 * y, y, 1.0);
-      r = fma(y * d, fma(0.375, d, 0.5), y);
-    } else {
-      r = 1.0 / sqrt(l1);
-    }
+    const double r = rsqrt(l1);
     s[i] = r;
     const double p = l1 * r;
     if (q) q[i] = p;
