@@ -69,9 +69,13 @@ __device__ __forceinline__ double fixpow_exp2(long long y, unsigned long long b)
   return __longlong_as_double((long long)bits);
 }
 
-// 1/q for a normal q well inside the exponent range: the hardware's approximation
-// (relative error e0 ~ 2^-20) and one cubically convergent step x (1 + e + e^2),
-// e = 1 - q x: three FP64 operations, error below 1 ulp.
+// 1/q for a normal q well inside the exponent range.  With x within 2^-19 of 1/q and
+// e = 1 - q x, 1/q = x / (1 - e) = x (1 + e + e^2 + ...): one step of the cubically convergent
+// iteration x (1 + e + e^2) (M. Altman, Pacific J. Math. 10 (1960) 1107) from the machine's
+// reciprocal of q's leading 20 bits.  What is cut off is below 2^-57, e is exact to
+// 2^-53 |e|, and the last multiply-add rounds once: relative error at most 2^-53 (1 + 2^-3),
+// below 1 ulp.  Three FP64 operations, on a pipe that a correctly rounded division would
+// hold several times as long.
 __device__ __forceinline__ double fast_rcp(double q) {
   double x;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(q));
