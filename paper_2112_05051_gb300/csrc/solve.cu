@@ -881,7 +881,8 @@ static int vcycle_level_hgs(rich_ctx* c, int l, const T* b, T** xres) {
 }
 
 // b is the level's right-hand side, the result is left in *xres (one of the level's buffers).
-// first_done: the level's x holds the first sweep, D_l1^-1 b, already (the restriction's y2).
+// first_done: the level's x holds the first sweep, D_l1^-1 b, already (the restriction's y2;
+// with nu1 > 0 on every level below the finest but a dense coarsest one).
 template <class T>
 static int vcycle_level(rich_ctx* c, int l, const T* b, T** xres, bool first_done) {
   Hierarchy& H = c->H;
@@ -930,14 +931,11 @@ static int vcycle_level(rich_ctx* c, int l, const T* b, T** xres, bool first_don
     RICH_LAUNCH_CHECK();
     return RICH_OK;
   };
-  const T* cur = x;  // where the iterate is: on the finest level the first sweep's is b itself
+  // where the iterate is: the first sweep from x = 0 gives b itself on the finest level, and
+  // below it x holds it already (first_done)
+  const T* cur = x;
   if (nu1 > 0) {
-    if (st0) {
-      cur = b;
-    } else if (!first_done) {  // first sweep from x = 0: x = D_l1^-1 b, elementwise
-      k_jacobi0<T><<<g, kBlock, 0, c->st>>>(n, v.dinv, b, x);
-      RICH_LAUNCH_CHECK();
-    }
+    if (st0) cur = b;
     for (int s = 1; s < nu1; ++s) {
       T* to = cur == x ? t : x;
       RICH_CHECK(sweep(cur, to));
