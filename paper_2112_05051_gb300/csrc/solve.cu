@@ -1537,12 +1537,15 @@ static int fcg_solve(rich_ctx* c, int S, const double* b, double* x, const rich_
       if (waited && !running()) break;
       if (!H.fcg_exec[fcg_slot(S)]) fcg_capture<T>(c, S);
       if (H.fcg_exec[fcg_slot(S)]) {
-        const int it0 = waited ? out[0].it : 0;
+        auto most = [&]() {  // iterations of the problem that went longest
+          int it = 0;
+          for (int s = 0; s < S; ++s) it = std::max(it, out[s].it);
+          return it;
+        };
+        const int it0 = waited ? most() : 0;
         RICH_CUDA(cudaGraphLaunch(H.fcg_exec[fcg_slot(S)], c->st));
         RICH_CUDA(cudaStreamSynchronize(c->st));
-        int most = 1;
-        for (int s = 0; s < S; ++s) most = std::max(most, out[s].it - it0);
-        count_launches(most * H.fcg_nodes[fcg_slot(S)]);
+        count_launches(std::max(1, most() - it0) * H.fcg_nodes[fcg_slot(S)]);
         break;
       }
     }
