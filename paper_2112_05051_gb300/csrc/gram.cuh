@@ -106,8 +106,9 @@ struct UnitSum {
     carry();
     const int k = min(__clzll(hh ^ (hh >> 63)) - 2, 30);  // hh 2^k below 2^62
     const long long r = k < 30 ? 1LL << (29 - k) : 0;
-    return (double)((long long)((unsigned long long)hh << k) + ((x + r) >> (30 - k))) *
-           __hiloint2double((1023 - k) << 20, 0);
+    const long long t = (long long)((unsigned long long)hh << k) + ((x + r) >> (30 - k));
+    const double v = (double)t;  // 0 or at least 1: its exponent takes the 2^-k
+    return __hiloint2double(__double2hiint(v) - (t ? k << 20 : 0), __double2loint(v));
   }
 };
 
@@ -122,10 +123,12 @@ __device__ __forceinline__ void copy8(double* dst, const double* src) {
 }
 
 // The block's sums over its elements of M basis vectors (from v0) times w and vj, into
-// a[q] and a[4 + q]; tops and topj: the vectors' unit_top.
+// a[q] and a[4 + q].  tops: the nv vectors' unit_top, filled here for the first sweep (the
+// loads are under way by then) from this thread's vector's peak.
 template <int M>
 __device__ __forceinline__ void gs_tile(long long n, const double* v0, const double* w, const double* vj,
-                                        const unsigned* tops, unsigned topj, GsStage (&st)[kGsStages], double (&a)[8]) {
+                                        unsigned* tops, int q0, int nv, unsigned peak, GsStage (&st)[kGsStages],
+                                        double (&a)[8]) {
   const long long stride = (long long)gridDim.x * kGsThreads;
   const int t = threadIdx.x;
   auto fetch = [&](int slot, long long i) {
@@ -140,10 +143,15 @@ __device__ __forceinline__ void gs_tile(long long n, const double* v0, const dou
   long long i = blockIdx.x * (long long)kGsThreads + t;
 #pragma unroll
   for (int k = 0; k < kGsStages; ++k) fetch(k, i + k * stride);
+  if (q0 == 0) {
+    if (t < nv) tops[t] = unit_top(peak, (n + stride - 1) / stride);
+    __syncthreads();
+  }
   UnitSum g[M];
   unsigned top[M];
+  const unsigned topj = tops[nv - 1];
 #pragma unroll
-  for (int q = 0; q < M; ++q) top[q] = tops[q];
+  for (int q = 0; q < M; ++q) top[q] = tops[q0 + q];
   int run = 0, slot = 0;
 #pragma unroll 1
   for (; i < n; i += stride) {
@@ -184,21 +192,16 @@ __global__ void __launch_bounds__(kGsThreads, 3) k_gs_dots(long long n, int nv, 
   __shared__ bool last;
   const double* vj = V + (long long)(nv - 1) * n;
   __shared__ unsigned tops[kGsLd];
-  if (threadIdx.x < nv) {
-    const long long threads = (long long)gridDim.x * kGsThreads;
-    tops[threadIdx.x] = unit_top(peak[threadIdx.x], (n + threads - 1) / threads);
-  }
-  __syncthreads();
-  const unsigned topj = tops[nv - 1];
+  const unsigned own = threadIdx.x < nv ? peak[threadIdx.x] : 0;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int q0 = 0; q0 < nv; q0 += kGsTile) {
     double a[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     const double* v0 = V + (long long)q0 * n;
     const int m = min(kGsTile, nv - q0);
-    if (m == 4) gs_tile<4>(n, v0, w, vj, tops + q0, topj, st, a);
-    else if (m == 3) gs_tile<3>(n, v0, w, vj, tops + q0, topj, st, a);
-    else if (m == 2) gs_tile<2>(n, v0, w, vj, tops + q0, topj, st, a);
-    else gs_tile<1>(n, v0, w, vj, tops + q0, topj, st, a);
+    if (m == 4) gs_tile<4>(n, v0, w, vj, tops, q0, nv, own, st, a);
+    else if (m == 3) gs_tile<3>(n, v0, w, vj, tops, q0, nv, own, st, a);
+    else if (m == 2) gs_tile<2>(n, v0, w, vj, tops, q0, nv, own, st, a);
+    else gs_tile<1>(n, v0, w, vj, tops, q0, nv, own, st, a);
     const double r = warp_sum8(a);
     if ((lane & 3) == 0) sh[wid][lane >> 2] = r;
     __syncthreads();
@@ -244,16 +247,6 @@ __global__ void __launch_bounds__(kGsThreads, 3) k_gs_dots(long long n, int nv, 
   if (threadIdx.x == 0) *ticket = 0;
 }
 
-// High word of the block's largest value, in thread 0.
-__device__ __forceinline__ unsigned gs_block_max(unsigned hi) {
-  __shared__ unsigned sh[kGsThreads / 32];
-  hi = __reduce_max_sync(0xffffffffu, hi);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = hi;
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 1; k < kGsThreads / 32; ++k) hi = max(hi, sh[k]);
-  return hi;
-}
 __device__ __forceinline__ unsigned abs_hi(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
 // *peak, zero before: the high word of the largest |f v|, for a cycle's first vector.
@@ -262,8 +255,8 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_peak(long long n, const doubl
   unsigned hi = 0;
   for (long long i = blockIdx.x * (long long)kGsThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kGsThreads)
     hi = max(hi, abs_hi(f * v[i]));
-  hi = gs_block_max(hi);
-  if (threadIdx.x == 0) atomicMax(peak, hi);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0 && hi > __ldcg(peak)) atomicMax(peak, hi);
 }
 
 // out = w - V h (w may be out) and its norm: the last block leaves ||out|| and 1/||out||
@@ -275,6 +268,8 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, c
                                                           double* __restrict__ s, double* __restrict__ mirror) {
   __shared__ double hs[kGsLd];
   __shared__ bool last;
+  __shared__ unsigned big[2];  // largest high words, of the block and of all
+  if (threadIdx.x < 2) big[threadIdx.x] = 0;
   for (int q = threadIdx.x; q < nv; q += kGsThreads) hs[q] = s[q];
   __syncthreads();
   const long long stride = (long long)gridDim.x * kGsThreads;
@@ -303,11 +298,12 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, c
     acc[0] = fma(t, t, acc[0]);
     hi = max(hi, abs_hi(t));
   }
-  block_sum<1>(acc);
-  hi = gs_block_max(hi);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0) atomicMax(&big[0], hi);
+  block_sum<1>(acc);  // (its barriers order big, too)
   if (threadIdx.x == 0) {
     part[blockIdx.x] = acc[0];
-    part[gridDim.x + blockIdx.x] = __hiloint2double((int)hi, 0);
+    part[gridDim.x + blockIdx.x] = __hiloint2double((int)big[0], 0);
     __threadfence();
     last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
@@ -320,13 +316,14 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(long long n, int nv, c
     acc[0] += __ldcg(&part[k]);
     hi = max(hi, abs_hi(__ldcg(&part[gridDim.x + k])));
   }
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if ((threadIdx.x & 31) == 0) atomicMax(&big[1], hi);
   block_sum<1>(acc);
-  hi = gs_block_max(hi);
   if (threadIdx.x == 0) {
     const double h = sqrt(acc[0]), inv = h > 0 ? 1.0 / h : 0.0;
     s[kSlotNorm] = mirror[kSlotNorm] = h;
     s[kSlotInv] = inv;
-    *peak = abs_hi(__hiloint2double((int)hi, -1) * inv);
+    *peak = abs_hi(__hiloint2double((int)big[1], -1) * inv);
     *ticket = 0;
   }
 }
