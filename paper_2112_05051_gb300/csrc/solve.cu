@@ -363,7 +363,18 @@ struct TuneVal {
   float us;      // its time per launch
   int best_csr;  // fastest CSR candidate (used where a matrix of the class has no SELL copy)
 };
-constexpr long long kTuneDelay = 60000;  // ~30 us: longer than the host takes to queue the timed launches
+constexpr long long kTuneDelay = 24000;  // ~12 us: longer than the host takes to queue a candidate's timed launches
+struct TuneEvents {
+  std::vector<cudaEvent_t> e;
+  bool ok = true;
+  explicit TuneEvents(size_t n) : e(n, nullptr) {
+    for (auto& x : e) ok = ok && cudaEventCreate(&x) == cudaSuccess;
+  }
+  ~TuneEvents() {
+    for (auto x : e)
+      if (x) cudaEventDestroy(x);
+  }
+};
 static std::mutex g_tune_mu;
 static std::map<TuneKey, TuneVal> g_tune;
 
@@ -426,39 +437,42 @@ static int csr_op(rich_ctx* c, int n, long long nnz, const int* rp, const int* c
       // (a 256 MB write before it) was measured and chose worse variants: the same
       // headline, 3 % less in the mixed mode, whose FP32 levels stay in L2 between
       // the sweeps of a V-cycle.
-      cudaEvent_t e0, e1;
-      RICH_CUDA(cudaEventCreate(&e0));
-      RICH_CUDA(cudaEventCreate(&e1));
       float best = 1e30f, best_csr_us = 1e30f;
       int best_csr = v;
       const Sell* sl = sell_ok ? src->s : nullptr;
       const T* sval = sell_ok ? (sizeof(T) == 8 ? (const T*)sl->val : (const T*)sl->val32) : nullptr;
+      // The timed launches queue up behind a delay, so that the events see the GPU alone, and
+      // all candidates are waited for once.  (With a wait for each, and 30 us of delay, a first
+      // FCG solve at 48^3 MIXED on a new context took 5.7 ms, 4.6 so.)
+      std::vector<int> cand;
       for (int g : {1, 2, 4, 8, 16, 32, 1 | kUnroll, 2 | kUnroll, 4 | kUnroll, 8 | kUnroll, 16 | kUnroll,
-                    32 | kUnroll, kSellVariant,
-                    kSellVariant8, kSellVariant2, kSellVariantP}) {
-        if (is_sell(g) && !sell_ok) continue;
-        csr_launch<T, MODE>(c->st, g, n, rp, col, val, dinv, b, x, scratch, sl, sval, y2);
-        gpu_delay(c->st, kTuneDelay);  // the launches queue up behind it: the events see the GPU alone
-        RICH_CUDA(cudaEventRecord(e0, c->st));
+                    32 | kUnroll, kSellVariant, kSellVariant8, kSellVariant2, kSellVariantP})
+        if (!is_sell(g) || sell_ok) cand.push_back(g);
+      TuneEvents ev(2 * cand.size());
+      if (!ev.ok) return RICH_ECUDA;
+      for (size_t k = 0; k < cand.size(); ++k) {
+        csr_launch<T, MODE>(c->st, cand[k], n, rp, col, val, dinv, b, x, scratch, sl, sval, y2);
+        gpu_delay(c->st, kTuneDelay);
+        RICH_CUDA(cudaEventRecord(ev.e[2 * k], c->st));
         for (int rep = 0; rep < 3; ++rep)
-          csr_launch<T, MODE>(c->st, g, n, rp, col, val, dinv, b, x, scratch, sl, sval, y2);
-        RICH_CUDA(cudaEventRecord(e1, c->st));
-        RICH_CUDA(cudaEventSynchronize(e1));
-        float ms = 0.f;
-        RICH_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+          csr_launch<T, MODE>(c->st, cand[k], n, rp, col, val, dinv, b, x, scratch, sl, sval, y2);
+        RICH_CUDA(cudaEventRecord(ev.e[2 * k + 1], c->st));
         count_launches(4);
+      }
+      RICH_CUDA(cudaEventSynchronize(ev.e.back()));
+      for (size_t k = 0; k < cand.size(); ++k) {
+        float ms = 0.f;
+        RICH_CUDA(cudaEventElapsedTime(&ms, ev.e[2 * k], ev.e[2 * k + 1]));
         if (ms < best) {
           best = ms;
-          v = g;
+          v = cand[k];
         }
-        if (!is_sell(g) && ms < best_csr_us) {
+        if (!is_sell(cand[k]) && ms < best_csr_us) {
           best_csr_us = ms;
-          best_csr = g;
+          best_csr = cand[k];
         }
       }
       RICH_CUDA(cudaGetLastError());
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
       dfree(scratch);
       g_tune[key] = {v, best * 1000.f / 3.f, best_csr};
       if (sell_ok && !is_sell(v) && !had_copy) {  // the copy lost: not kept, not refreshed
