@@ -2001,11 +2001,15 @@ static int fine_stencil(rich_ctx* c) {
   return RICH_OK;
 }
 
-static int level_diag_data(rich_ctx* c, Level& L) {
+// l1: the level's sweeps read 1/l1 (a scaled finest level's read ScaledSt instead); cast: the
+// FP32 values, which MIXED's products and sweeps read.
+static int level_diag_data(rich_ctx* c, Level& L, bool l1 = true, bool cast = true) {
   bool mp = c->prec == RICH_PREC_MIXED;
-  k_l1dinv<<<grid_for(L.n), kBlock, 0, c->st>>>(L.n, L.A.rowptr, L.A.val, L.dinv, mp ? L.dinv32 : nullptr);
-  RICH_LAUNCH_CHECK();
-  if (mp) {
+  if (l1) {
+    k_l1dinv<<<grid_for(L.n), kBlock, 0, c->st>>>(L.n, L.A.rowptr, L.A.val, L.dinv, mp ? L.dinv32 : nullptr);
+    RICH_LAUNCH_CHECK();
+  }
+  if (mp && cast) {
     k_cast<<<grid_for(L.A.nnz), kBlock, 0, c->st>>>(L.A.nnz, L.A.val, L.A32);
     RICH_LAUNCH_CHECK();
   }
@@ -2416,7 +2420,7 @@ int amg_build(rich_ctx* c, const rich_amg_opts* o) {
   H.scaled = H.nlev > 1 && H.opts.smoother == RICH_SMOOTH_L1JACOBI;
   for (int l = 0; l < H.nlev; ++l) {
     RICH_CHECK(level_alloc_vectors(c, H.lv[l]));
-    RICH_CHECK(level_diag_data(c, H.lv[l]));
+    RICH_CHECK(level_diag_data(c, H.lv[l], l > 0 || !H.scaled));
   }
   RICH_CHECK(fine_stencil(c));
   if (H.dense) {
@@ -2452,7 +2456,7 @@ int amg_refresh(rich_ctx* c) {
     // The V-cycle runs in FP32, so the Galerkin products do too: A32_{l+1} =
     // R32 (A32_l P32), on the patterns kept from the setup.  The FP64 values of
     // the coarse levels keep their setup-time content and are not read again.
-    RICH_CHECK(level_diag_data(c, H.lv[0]));
+    RICH_CHECK(level_diag_data(c, H.lv[0], !H.scaled));
     for (int l = 0; l + 1 < H.nlev; ++l) {
       Level& L = H.lv[l];
       Level& N = H.lv[l + 1];
@@ -2467,7 +2471,7 @@ int amg_refresh(rich_ctx* c) {
       RICH_CHECK(spgemm_numeric(c, L.A, L.P, L.AP, L.u_ap, 0, l, &L.pl_ap));
       RICH_CHECK(spgemm_numeric(c, L.R, L.AP, H.lv[l + 1].A, L.u_rap, 1, l, &L.pl_rap));
     }
-    for (int l = 0; l < H.nlev; ++l) RICH_CHECK(level_diag_data(c, H.lv[l]));
+    for (int l = H.scaled ? 1 : 0; l < H.nlev; ++l) RICH_CHECK(level_diag_data(c, H.lv[l]));
   }
   for (int l = 1; l < H.nlev; ++l) RICH_CHECK(sell_fill_a(c, H.lv[l]));
   RICH_CHECK(fine_stencil(c));
@@ -2484,7 +2488,7 @@ int amg_update_fine(rich_ctx* c) {
   }
   RICH_CHECK(refresh_a0_values(c));
   H.lv[0].A = c->A0;
-  RICH_CHECK(level_diag_data(c, H.lv[0]));
+  RICH_CHECK(level_diag_data(c, H.lv[0], !H.scaled, !H.scaled));
   RICH_CHECK(fine_stencil(c));
   if (H.nlev == 1) return coarse_inverse(c);
   return RICH_OK;
