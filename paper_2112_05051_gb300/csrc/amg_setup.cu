@@ -1170,9 +1170,9 @@ __device__ __forceinline__ T pl_sum(const int2* __restrict__ p, int left, const 
 // warp and load, and as many steps as the longest of 32 neighbours), 880 us so.
 // SPLIT: a block per slice, for products whose slices are few and long, where a warp's chain
 // of loads would be the time: its warps take the columns eight at a time in turn (an entry's
-// split is its own, whatever slice it shares) and their sums are added in order.  48^3 FP64,
-// all products: 328 us without, 112 us so; matching aggregates of 1024 cells on 64^3: 657
-// and 227 us.
+// split is its own, whatever slice it shares) and their sums are added in order.  All products
+// of a refresh, FP64, without and so: 48^3 437 and 135 us, 96^3 918 and 533, 128^3 1289 and
+// 1201; matching aggregates of 1024 cells on 64^3 657 and 227.
 template <class T, bool SPLIT>
 __global__ void __launch_bounds__(32 * kPlWarps) k_galerkin_lists(int nslice, const int* __restrict__ perm,
                                                                   const long long* __restrict__ sptr,
@@ -1720,9 +1720,13 @@ static int spgemm_numeric_t(rich_ctx* c, const Csr<double>& A, const T* aval, co
     auto run = [&](auto kernel, int blocks) {
       kernel<<<blocks, 32 * kPlWarps, 0, c->st>>>(pl->nslice, pl->perm, pl->sptr, pl->pairs, aval, bval, cval);
     };
-    // a warp per slice below 48 of them per SM does not hide its loads' latency (64^3, entries
-    // of 40 products in 3146 slices: 3 times longer); a pair or two per warp is not worth it
-    if (pl->nslice < 48 * kNumSM && (double)pl->np > 8.0 * (double)C.nnz)
+    // A warp per slice does not hide its loads' latency while there are few of them, the longer
+    // the entries the more are few.  FP64, a warp and a block per slice: entries of 9 products in
+    // 68 slices per SM 43 and 29 us, in 91 per SM 35 and 40; of 30 products in 77 per SM 174 and
+    // 62, in 320 per SM 283 and 230, in 620 per SM 444 and 442 (FP32 328 and 342).  A pair or two
+    // per warp (entries of 3 products) is not worth it.
+    const double len = (double)pl->np / (double)C.nnz;
+    if (pl->nslice < (len > 20.0 ? 320 : len > 8.0 ? 72 : 0) * kNumSM)
       run(k_galerkin_lists<T, true>, pl->nslice);
     else
       run(k_galerkin_lists<T, false>, (pl->nslice + kPlWarps - 1) / kPlWarps);
