@@ -1171,34 +1171,40 @@ __device__ __forceinline__ T pl_sum(const int2* __restrict__ p, int left, const 
 // SPLIT: a block per slice, for products whose slices are few and long, where a warp's chain
 // of loads would be the time: its warps take the columns eight at a time in turn (an entry's
 // split is its own, whatever slice it shares) and their sums are added in order.  All products
-// of a refresh, FP64, without and so: 48^3 437 and 135 us, 96^3 918 and 533, 128^3 1289 and
-// 1201; matching aggregates of 1024 cells on 64^3 657 and 227.
+// of a refresh, FP64, without and so: 48^3 437 and 135 us, 96^3 918 and 512, 128^3 1289 and
+// 1150; matching aggregates of 1024 cells on 64^3 657 and 227.
 template <class T, bool SPLIT>
 __global__ void __launch_bounds__(32 * kPlWarps) k_galerkin_lists(int nslice, const int* __restrict__ perm,
                                                                   const long long* __restrict__ sptr,
                                                                   const int2* __restrict__ pairs,
                                                                   const T* __restrict__ aval,
                                                                   const T* __restrict__ bval, T* __restrict__ cval) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, s = SPLIT ? blockIdx.x : blockIdx.x * kPlWarps + w;
-  if (s >= nslice) return;  // (SPLIT: no block of the grid)
-  const int2* p = pairs + sptr[s] + lane;
-  const int width = (int)((sptr[s + 1] - sptr[s]) / kSellC);
-  T acc = T(0);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (SPLIT) {
     __shared__ T part[kPlWarps][kSellC];
+    const int s = blockIdx.x, q = perm[s * kSellC + lane];
+    const int2* p = pairs + sptr[s] + lane;
+    const int width = (int)((sptr[s + 1] - sptr[s]) / kSellC);
+    T acc = T(0);
     for (int c = 8 * w; c < width; c += 8 * kPlWarps)
       acc = pl_sum<T, 8, true>(p + (long long)c * kSellC, width - c, aval, bval, acc);
     part[w][lane] = acc;
     __syncthreads();
     if (w > 0) return;
     for (int v = 1; v < kPlWarps; ++v) acc += part[v][lane];
-  } else {
-    int c = 0;
-    for (; c + 4 <= width; c += 4) acc = pl_sum<T, 4, false>(p + (long long)c * kSellC, 4, aval, bval, acc);
-    for (; c < width; ++c) acc = pl_sum<T, 1, false>(p + (long long)c * kSellC, 1, aval, bval, acc);
+    if (q >= 0) cval[q] = acc;
+    return;
   }
-  const int q = perm[s * kSellC + lane];
-  if (q >= 0) cval[q] = acc;
+  for (int s = blockIdx.x * kPlWarps + w; s < nslice; s += gridDim.x * kPlWarps) {
+    // loaded ahead of the pairs: after them, entries of 3 products took 233 us for 190 (128^3)
+    const int q = perm[s * kSellC + lane];
+    const int2* p = pairs + sptr[s] + lane;
+    const int2* end = pairs + sptr[s + 1];
+    T acc = T(0);
+    for (; p + 3 * kSellC < end; p += 4 * kSellC) acc = pl_sum<T, 4, false>(p, 4, aval, bval, acc);
+    for (; p < end; p += kSellC) acc = pl_sum<T, 1, false>(p, 1, aval, bval, acc);
+    if (q >= 0) cval[q] = acc;
+  }
 }
 
 // ---------------------------------------------------------------- coarsest level: dense inverse
@@ -1729,7 +1735,7 @@ static int spgemm_numeric_t(rich_ctx* c, const Csr<double>& A, const T* aval, co
     if (pl->nslice < (len > 20.0 ? 320 : len > 8.0 ? 72 : 0) * kNumSM)
       run(k_galerkin_lists<T, true>, pl->nslice);
     else
-      run(k_galerkin_lists<T, false>, (pl->nslice + kPlWarps - 1) / kPlWarps);
+      run(k_galerkin_lists<T, false>, grid_for(32LL * pl->nslice));
     RICH_LAUNCH_CHECK();
     return RICH_OK;
   }
