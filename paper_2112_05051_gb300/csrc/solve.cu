@@ -340,7 +340,7 @@ static int default_lanes(double avg) {
 // Autotuner of the CSR row operations: the first time an operation meets a shape
 // class (mode, value type, rows in quarter-octave bins, mean row length rounded to
 // an integer), every candidate is timed on the actual operands (output to a scratch
-// vector, one warm-up and three timed launches each, CUDA events) and the fastest
+// vector, two rounds behind a warm-up launch each, CUDA events) and the fastest
 // is kept for the rest of the process.  Classes, not exact shapes, so that
 // a stream of requests of similar size (whose coarse levels differ by a few rows)
 // tunes once.  The table is shared by all contexts (under a mutex, held while
@@ -363,7 +363,9 @@ struct TuneVal {
   float us;      // its time per launch
   int best_csr;  // fastest CSR candidate (used where a matrix of the class has no SELL copy)
 };
-constexpr long long kTuneDelay = 24000;  // ~12 us: longer than the host takes to queue a candidate's timed launches
+constexpr long long kTuneDelay = 40000;  // ~20 us: the host gets ahead of the timed launches
+constexpr size_t kTuneLast = 6;          // candidates of the second round at most
+constexpr float kTuneTick = 2.1f;        // us: what the length of a timed run is rounded to
 struct TuneEvents {
   std::vector<cudaEvent_t> e;
   bool ok = true;
@@ -441,40 +443,65 @@ static int csr_op(rich_ctx* c, int n, long long nnz, const int* rp, const int* c
       int best_csr = v;
       const Sell* sl = sell_ok ? src->s : nullptr;
       const T* sval = sell_ok ? (sizeof(T) == 8 ? (const T*)sl->val : (const T*)sl->val32) : nullptr;
-      // The timed launches queue up behind a delay, so that the events see the GPU alone, and
-      // all candidates are waited for once.  (With a wait for each, and 30 us of delay, a first
-      // FCG solve at 48^3 MIXED on a new context took 5.7 ms, 4.6 so.)
+      // us per launch of each candidate: the launches queue up behind a delay, so that the
+      // events see the GPU alone, and all are waited for once.
+      auto measure = [&](const std::vector<int>& cand, const std::vector<int>& reps, std::vector<float>& us) -> int {
+        TuneEvents ev(2 * cand.size());
+        if (!ev.ok) return RICH_ECUDA;
+        gpu_delay(c->st, kTuneDelay);
+        for (size_t k = 0; k < cand.size(); ++k) {
+          csr_launch<T, MODE>(c->st, cand[k], n, rp, col, val, dinv, b, x, scratch, sl, sval, y2);
+          RICH_CUDA(cudaEventRecord(ev.e[2 * k], c->st));
+          for (int rep = 0; rep < reps[k]; ++rep)
+            csr_launch<T, MODE>(c->st, cand[k], n, rp, col, val, dinv, b, x, scratch, sl, sval, y2);
+          RICH_CUDA(cudaEventRecord(ev.e[2 * k + 1], c->st));
+          count_launches(1 + reps[k]);
+        }
+        RICH_CUDA(cudaEventSynchronize(ev.e.back()));
+        us.resize(cand.size());
+        for (size_t k = 0; k < cand.size(); ++k) {
+          RICH_CUDA(cudaEventElapsedTime(&us[k], ev.e[2 * k], ev.e[2 * k + 1]));
+          us[k] *= 1000.f / reps[k];
+        }
+        return RICH_OK;
+      };
+      // First two launches of each, then runs of about 60 us of those that two launches cannot
+      // tell from the fastest.  (A first V-cycle, V(1,1) at 128^3 FP64, and the later ones: 50 ms
+      // and 281 us with a wait, 30 us of delay and three launches per candidate; 45 ms and 290
+      // with one wait for all, small kernels' ties being settled by their order; 36 ms and 281 so.)
       std::vector<int> cand;
       for (int g : {1, 2, 4, 8, 16, 32, 1 | kUnroll, 2 | kUnroll, 4 | kUnroll, 8 | kUnroll, 16 | kUnroll,
                     32 | kUnroll, kSellVariant, kSellVariant8, kSellVariant2, kSellVariantP})
         if (!is_sell(g) || sell_ok) cand.push_back(g);
-      TuneEvents ev(2 * cand.size());
-      if (!ev.ok) return RICH_ECUDA;
-      for (size_t k = 0; k < cand.size(); ++k) {
-        csr_launch<T, MODE>(c->st, cand[k], n, rp, col, val, dinv, b, x, scratch, sl, sval, y2);
-        gpu_delay(c->st, kTuneDelay);
-        RICH_CUDA(cudaEventRecord(ev.e[2 * k], c->st));
-        for (int rep = 0; rep < 3; ++rep)
-          csr_launch<T, MODE>(c->st, cand[k], n, rp, col, val, dinv, b, x, scratch, sl, sval, y2);
-        RICH_CUDA(cudaEventRecord(ev.e[2 * k + 1], c->st));
-        count_launches(4);
+      std::vector<float> us, us2;
+      RICH_CHECK(measure(cand, std::vector<int>(cand.size(), 2), us));
+      std::vector<size_t> by(cand.size());
+      for (size_t k = 0; k < by.size(); ++k) by[k] = k;
+      std::stable_sort(by.begin(), by.end(), [&](size_t p, size_t q) { return us[p] < us[q]; });
+      std::vector<int> last, reps;
+      for (size_t k : by) {
+        if (last.size() == kTuneLast || us[k] > 1.02f * us[by[0]] + 0.5f * kTuneTick) break;
+        last.push_back(cand[k]);
+        reps.push_back(std::min(12, std::max(2, (int)(60.f / us[k]))));
       }
-      RICH_CUDA(cudaEventSynchronize(ev.e.back()));
-      for (size_t k = 0; k < cand.size(); ++k) {
-        float ms = 0.f;
-        RICH_CUDA(cudaEventElapsedTime(&ms, ev.e[2 * k], ev.e[2 * k + 1]));
-        if (ms < best) {
-          best = ms;
-          v = cand[k];
+      if (last.size() > 1) {
+        RICH_CHECK(measure(last, reps, us2));
+        for (size_t k = 0; k < last.size(); ++k) us[by[k]] = us2[k];
+      }
+      for (size_t k = 0; k < by.size(); ++k) {
+        const int g = cand[by[k]];
+        if (k < last.size() && us[by[k]] < best) {
+          best = us[by[k]];
+          v = g;
         }
-        if (!is_sell(cand[k]) && ms < best_csr_us) {
-          best_csr_us = ms;
-          best_csr = cand[k];
+        if (!is_sell(g) && us[by[k]] < best_csr_us) {
+          best_csr_us = us[by[k]];
+          best_csr = g;
         }
       }
       RICH_CUDA(cudaGetLastError());
       dfree(scratch);
-      g_tune[key] = {v, best * 1000.f / 3.f, best_csr};
+      g_tune[key] = {v, best, best_csr};
       if (sell_ok && !is_sell(v) && !had_copy) {  // the copy lost: not kept, not refreshed
         sell_free(*src->s);
         sell_ok = false;
