@@ -390,7 +390,7 @@ __device__ __forceinline__ long long law_log(double p) {
 // K(p) (and, below, the rest of the law) from the fixed-point powers: the sums, one
 // reciprocal each and the products are all that runs in FP64 (K alone 6 operations, the
 // whole law 23 against about 95 through log()/exp() and divisions).  FP64 pipe bound
-// both ways: the law of 2.1M cells took 380 us before and takes 110.
+// both ways: the law of 2.1M cells took 370 us before and takes 94.
 __device__ __forceinline__ double conductivity_only(double p, double ks, double ksa, const SoilP& so) {
   if (law_fast(p, so)) return ksa * fast_rcp(so.a + fixpow_exp2(law_log(p), so.qg));
   return p < 0.0 ? law_general(p, ks, so).K : ks;

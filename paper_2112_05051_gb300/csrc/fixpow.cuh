@@ -3,7 +3,7 @@
 // GB300 issues two FP64 operations per SM and clock but 64 integer multiply-adds, so
 // the log and the two exponentials of the law, about 60 FP64 instructions through
 // log()/exp(), are evaluated in fixed point on the otherwise idle integer pipe and cost
-// no FP64 operation at all: the constitutive pass of 2.1M cells went from 380 to 110 us.
+// no FP64 operation at all: the constitutive pass of 2.1M cells went from 370 to 94 us.
 // Method: table-driven logarithm and exponential (P. T. P. Tang, ACM TOMS 15 (1989) and
 // 16 (1990)) with 256-entry tables and short series, carried out in fixed point:
 //   x = 2^e m;  r = m c_i - 1 with c_i ~ 1/m (table), |r| <= 2^-9, exact to 2^-71;

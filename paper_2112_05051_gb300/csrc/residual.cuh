@@ -8,8 +8,8 @@
 // shared through shared memory instead of a pass over memory, the two cells of a
 // horizontal face compute its mean flux with four operations each, and a vertical face is
 // computed once, by the thread that marches its column.  128^3, upstream mean, norms read
-// back: 434 us as a law pass, a face pass and three single-block sums, 184 us here (38 FP64
-// operations per cell against 64 to 95); 16^3: 46 to 23 us.
+// back: 710 us as a law pass, a face pass and three single-block sums, 184 us here (38 FP64
+// operations per cell against 64 to 95); 16^3: 55 to 23 us.
 //
 // A face's flux is the same number seen from either cell (t = k (p_L - p_U), exactly
 // negated by the difference's antisymmetry), and every variant orders a cell's sum the

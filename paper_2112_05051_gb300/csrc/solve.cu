@@ -8,8 +8,8 @@
 // nu2 sweeps.  In MIXED precision every level works in FP32 with FP32
 // accumulation; the Krylov vectors and dot products stay FP64.
 //
-// Krylov scalars live in device memory; each iteration reads one small block
-// of them back for the convergence test.
+// Krylov scalars live in device memory.  FGMRES reads one small block of them back per
+// iteration for the convergence test; FCG tests on the device and is read when it stops.
 #include <algorithm>
 #include <cstdio>
 #include <map>
@@ -27,7 +27,7 @@ __global__ void k_jacobi0(int n, const T* __restrict__ dinv, const T* __restrict
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] = dinv[i] * b[i];
 }
 
-// CSR row operation with G lanes per row (G = 4..32), for levels whose rows are
+// CSR row operation with G lanes per row (G = 1..32), for levels whose rows are
 // long (coarse Galerkin operators carry tens to hundreds of entries per row).
 // MODE 0: y = A x, and y2 = dinv y if y2 (a level's right-hand side and its first sweep);
 // 1: y += A x; 2: y = x + dinv (b - A x); 3: y = b - A x; 4: y = b + dinv (A x).
@@ -482,7 +482,7 @@ static int csr_op(rich_ctx* c, int n, long long nnz, const int* rp, const int* c
       for (size_t k : by) {
         if (last.size() == kTuneLast || us[k] > 1.02f * us[by[0]] + 0.5f * kTuneTick) break;
         last.push_back(cand[k]);
-        reps.push_back(std::min(12, std::max(2, (int)(60.f / us[k]))));
+        reps.push_back(std::max(2, (int)std::min(12.f, 60.f / us[k])));
       }
       if (last.size() > 1) {
         RICH_CHECK(measure(last, reps, us2));
